@@ -425,7 +425,8 @@ static uint32_t choose_page(uint32_t N, int nsm)
 {
     const double warps = (double)nsm * 4 * 8;
     double per = (double)N * 32.0 / warps;
-    uint32_t pg = 2048;
+    // a list that outgrows a fresh page is walked twice: 4096 entries hold nearly every one
+    uint32_t pg = 4096;
     while (pg < per && pg < 65536) pg <<= 1;
     return pg;
 }
