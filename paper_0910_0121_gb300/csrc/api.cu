@@ -296,6 +296,7 @@ static int derive_box(const greem_params &p, uint32_t pb, uint32_t pe, BoxPar &b
     bp.k52_f = (float)(std::ldexp(p.L, -52) / p.r_cut);
     bp.inv_rc2 = (float)(bp.inv_rc * bp.inv_rc);
     bp.eps2 = (float)((p.eps / p.r_cut) * (p.eps / p.r_cut));
+    bp.force_scale = (float)(kForceUnit * bp.inv_rc * bp.inv_rc);
     bp.soft = p.eps > 0 ? 1 : 0;
     // r_cut pruning: prune iff (double)S_gap * (u*u) > r_cut*r_cut
     bp.T_prune = max_s_le(bp.u * bp.u, p.r_cut * p.r_cut);
@@ -1664,6 +1665,7 @@ int greem_pair_force_f32(greem_ctx *c, const double *x_g, const double *x_i, con
     bp.inv_rc2 = (float)(bp.inv_rc * bp.inv_rc);
     bp.eps = eps;
     bp.eps2 = (float)((eps / r_cut) * (eps / r_cut));
+    bp.force_scale = (float)(kForceUnit * bp.inv_rc * bp.inv_rc);
     cudaStream_t s = c->stream;
     greem::g_launches = 0;
     if (!cuda_ok(cudaMemsetAsync(c->st.p, 0, sizeof(DevStatus), s)) ||

@@ -50,6 +50,7 @@ struct BoxPar {
     float k52_f;           // (L/2^52)/r_cut rounded to float: fixed52 offsets -> r_cut units
     float inv_rc2;         // 1/r_cut^2: r_cut-unit accelerations -> physical
     float eps2;            // (eps/r_cut)^2
+    float force_scale;     // kForceUnit/r_cut^2: the pair loops' accelerations -> physical
     long long T_prune;     // prune a node iff S_gap > T_prune (exact form of the r_cut test)
     long long A[22];       // accept a node of level k iff S_d > A[k] (exact form of the theta test)
     uint32_t p_begin, p_end;
@@ -60,6 +61,7 @@ struct BoxPar {
     int kstart, rprune;
     unsigned long long tbl_off;
 };
+constexpr double kForceUnit = 32.0 / 35.0;  // the unit of the FP32 pair loops' g(R)/xi^3 (force.cu)
 constexpr int kNotPow2 = -100000;
 
 // Polls of a bounded device wait before it gives up and records ST_TIMEOUT.

@@ -46,12 +46,13 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 // Writes the one box of constants the force kernel reads (no host staging buffer) and
 // clears the status word (flags and work-queue counters), which must start at zero on
 // every call.
-__global__ void k_noalloc_box(BoxPar *bp, DevStatus *st, float inv_rc2, float eps2)
+__global__ void k_noalloc_box(BoxPar *bp, DevStatus *st, float inv_rc2, float force_scale, float eps2)
 {
     if (threadIdx.x == 0) {
         BoxPar b = {};
         b.inv_rc2 = inv_rc2;
         b.eps2 = eps2;
+        b.force_scale = force_scale;
         *bp = b;
     }
     uint32_t *w = reinterpret_cast<uint32_t *>(st);
@@ -108,7 +109,7 @@ extern "C" int greem_pair_force_f32_noalloc(const double *x_g, const double *x_i
     const double inv_rc = 1.0 / r_cut;
     // an error left by earlier work on this thread is not this call's
     cudaGetLastError();
-    k_noalloc_box<<<1, 32, 0, s>>>(bp, st, (float)(inv_rc * inv_rc), (float)((eps / r_cut) * (eps / r_cut)));
+    k_noalloc_box<<<1, 32, 0, s>>>(bp, st, (float)(inv_rc * inv_rc), (float)(kForceUnit * inv_rc * inv_rc), (float)((eps / r_cut) * (eps / r_cut)));
     if (launch_failed()) return GREEM_ERR_CUDA;
     launch_pair_setup(x_g, x_i, x_j, m_j, (uint32_t)npairs, inv_rc, groups, irel, flist, loff, llen, lraw, perm, ng,
                       s);
