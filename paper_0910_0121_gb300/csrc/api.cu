@@ -316,6 +316,7 @@ static int derive_box(const greem_params &p, uint32_t pb, uint32_t pe, BoxPar &b
     bp.lmin = lmin;
     bp.n_crit = p.n_crit;
     bp.n_leaf = p.n_leaf;
+    bp.pass_cap = force_pass_cap(pe - pb, p.n_crit);
     return GREEM_OK;
 }
 
@@ -678,7 +679,7 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
         la.st = c->st.p;
         launch_lists(la, s, nsm);
         ev_record(c, r, ev, 5);
-        launch_force_order(c->groups.p, n_groups, c->bins.p, c->order.p, s, nsm);
+        launch_force_order(c->groups.p, n_groups, c->bps.p, c->bins.p, c->order.p, s, nsm);
         ForceArgs fa = {};
         fa.wait_polls1 = c->wait_polls1;
         fa.groups = c->groups.p;
@@ -701,6 +702,7 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
         fa.st = c->st.p;
         fa.chunk = r.chunk;
         fa.warps = r.warps;
+        force_caps(c->bps_host, nbox, fa);
         if (r.precision == GREEM_F64) launch_force_f64(fa, s, nsm);
         else launch_force_f32(fa, s, nsm, r.soft);
         if (r.quad) {
@@ -1666,6 +1668,7 @@ int greem_pair_force_f32(greem_ctx *c, const double *x_g, const double *x_i, con
     bp.eps = eps;
     bp.eps2 = (float)((eps / r_cut) * (eps / r_cut));
     bp.force_scale = (float)(kForceUnit * bp.inv_rc * bp.inv_rc);
+    bp.pass_cap = 0xffffffffu;
     cudaStream_t s = c->stream;
     greem::g_launches = 0;
     if (!cuda_ok(cudaMemsetAsync(c->st.p, 0, sizeof(DevStatus), s)) ||

@@ -30,6 +30,7 @@
 // The group's list streams through a per-warp double buffer in shared memory filled by
 // 1-D bulk asynchronous copies (cp.async.bulk, the TMA engine) that complete on an
 // mbarrier; every entry is read by the part's lanes as one broadcast 16-byte load.
+#include <algorithm>
 #include <atomic>
 
 #include "common.cuh"
@@ -394,6 +395,7 @@ __device__ __forceinline__ void interact_quad(const float4 j, const float4 q0, c
 #endif
 struct LayoutTable {
     uint8_t v[32 * kImax + 1];  // log2(S) in bits 4-6, I in bits 0-3
+    uint8_t rank[6 * kImax];    // [log2(S) kImax + I - 1]: place of the layout in the work order, 1 .. 6 kImax
 };
 
 constexpr LayoutTable make_layout_table()
@@ -418,6 +420,18 @@ constexpr LayoutTable make_layout_table()
             }
         }
         cost[n] = best;
+    }
+    // the work order: cycles per list entry, most first
+    auto per_entry = [](int k) {
+        const int I = k % kImax + 1, ls = k / kImax;
+        const long w = (I % 2 == 0) ? GREEM_LAYOUT_W_EVEN : GREEM_LAYOUT_W_ODD;
+        return ((I * w + GREEM_LAYOUT_O) * 32) >> ls;
+    };
+    for (int k = 0; k < 6 * kImax; k++) {
+        int r = 1;
+        for (int q = 0; q < 6 * kImax; q++)
+            if (per_entry(q) > per_entry(k) || (per_entry(q) == per_entry(k) && q < k)) r++;
+        t.rank[k] = (uint8_t)r;
     }
     return t;
 }
@@ -635,7 +649,9 @@ __device__ __noinline__ bool group_pass(const ForceArgs &a, const Group &gr, uin
 
 // QUAD: the second-order passes over the groups' accepted nodes (after the monopole
 // launch; groups without accepted nodes are skipped).
-template <bool SOFT, bool QUAD>
+// CAP: some box's passes are capped (force_pass_cap), and a group's passes may be dealt out
+// to 2^a.share work items.
+template <bool SOFT, bool QUAD, bool CAP>
 __global__ void __launch_bounds__(GREEM_FORCE_THREADS, GREEM_FORCE_MINB) k_force_f32(ForceArgs a)
 {
     extern __shared__ __align__(128) float4 sm[];
@@ -658,10 +674,16 @@ __global__ void __launch_bounds__(GREEM_FORCE_THREADS, GREEM_FORCE_MINB) k_force
     // retried with larger lists
     if (QUAD && (a.st->flags & (ST_LIST_CAP | ST_QLIST_CAP))) return;
     const uint32_t G = *a.n_groups;
+    const uint32_t share = CAP ? (uint32_t)a.share : 0u, others = (1u << share) - 1u;
     for (;;) {
         unsigned long long gi = 0;
         if (lane == 0) gi = atomicAdd(&a.st->work[QUAD ? 3 : 1], 1ull);
         gi = __shfl_sync(FULL, gi, 0);
+        uint32_t turn = 0;
+        if (CAP) {  // work item gi: the passes turn, turn + 2^share, ... of one group
+            turn = (uint32_t)gi & others;
+            gi >>= share;
+        }
         if (gi >= G) break;
         const uint32_t g = a.order ? a.order[gi] : (uint32_t)gi;
         const Group gr = a.groups[g];
@@ -674,17 +696,28 @@ __global__ void __launch_bounds__(GREEM_FORCE_THREADS, GREEM_FORCE_MINB) k_force
         uint32_t done = 0;
         unsigned long long evals = 0;
         bool ok = true;
+        const uint32_t cap = CAP ? bp.pass_cap : 0xffffffffu;
         while (done < gr.count && ok) {
             int S, I;
+            const uint32_t n = CAP ? min(gr.count - done, cap) : gr.count - done;
+            if (QUAD) choose_layout_quad(n, S, I);
+            else choose_layout(n, S, I);
+            const uint32_t slots = (uint32_t)(32 / S) * (uint32_t)I;
+            if (CAP) {
+                const bool skip = turn != 0;  // another item's pass
+                turn = skip ? turn - 1u : others;
+                if (skip) {
+                    done += slots;
+                    continue;
+                }
+            }
             if (QUAD) {
-                choose_layout_quad(gr.count - done, S, I);
                 if (I == 1) ok = group_pass<1, SOFT, true>(a, gr, done, S, lo, len, wp, scale, eps2, lane);
                 else if (I == 2) ok = group_pass<2, SOFT, true>(a, gr, done, S, lo, len, wp, scale, eps2, lane);
                 else ok = group_pass<4, SOFT, true>(a, gr, done, S, lo, len, wp, scale, eps2, lane);
-                done += (uint32_t)(32 / S) * (uint32_t)I;
+                done += slots;
                 continue;
             }
-            choose_layout(gr.count - done, S, I);
             switch (I) {
             case 1: ok = group_pass<1, SOFT, false>(a, gr, done, S, lo, len, wp, scale, eps2, lane); break;
             case 2: ok = group_pass<2, SOFT, false>(a, gr, done, S, lo, len, wp, scale, eps2, lane); break;
@@ -704,7 +737,6 @@ __global__ void __launch_bounds__(GREEM_FORCE_THREADS, GREEM_FORCE_MINB) k_force
 #endif
             default: ok = false; break;  // not reachable: choose_layout never exceeds kImax
             }
-            const uint32_t slots = (uint32_t)(32 / S) * (uint32_t)I;
             evals += (unsigned long long)slots * len;
             done += slots;
         }
@@ -768,18 +800,21 @@ void launch_qlist_fill(const ForceArgs &a, const float4 *quad, unsigned long lon
 }
 
 // ------------------------------------------------------------------ work order
-// Groups are ordered by lane layout (I i-particles per lane, S parts), largest first, so
-// that the warps of an SM mostly run the same instantiation of group_pass at a time
-// (one instruction-cache footprint) and the cheapest groups come last.
-__device__ __forceinline__ int layout_bin(uint32_t n)
+// Groups are ordered by lane layout (I i-particles per lane, S parts), so that the warps of
+// an SM mostly run the same instantiation of group_pass at a time (one instruction-cache
+// footprint), the layout with the most cycles per list entry first and the cheapest last
+// (100 k halo particles: 0.135 -> 0.129 ms against an order by I).
+__device__ __forceinline__ int layout_bin(const Group &g, const BoxPar *__restrict__ bps)
 {
+    const uint32_t n = min(g.count, bps[g.box].pass_cap);
     if (n > 32u * kImax) return 0;
     int S, I;
     choose_layout(n, S, I);
-    return (8 - I) * 6 + (31 - __clz(S));
+    return c_layout.rank[(31 - __clz(S)) * kImax + I - 1];
 }
 
 __global__ void __launch_bounds__(256) k_bin_count(const Group *__restrict__ groups, const uint32_t *n_groups,
+                                                   const BoxPar *__restrict__ bps,
                                                    uint32_t *__restrict__ bins)
 {
     __shared__ uint32_t sb[64];
@@ -787,7 +822,7 @@ __global__ void __launch_bounds__(256) k_bin_count(const Group *__restrict__ gro
     __syncthreads();
     const uint32_t G = *n_groups;
     for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x)
-        atomicAdd(&sb[layout_bin(groups[g].count)], 1u);
+        atomicAdd(&sb[layout_bin(groups[g], bps)], 1u);
     __syncthreads();
     if (threadIdx.x < 64 && sb[threadIdx.x]) atomicAdd(&bins[threadIdx.x], sb[threadIdx.x]);
 }
@@ -811,6 +846,7 @@ __global__ void k_bin_scan(uint32_t *bins)
 }
 
 __global__ void __launch_bounds__(256) k_bin_scatter(const Group *__restrict__ groups, const uint32_t *n_groups,
+                                                     const BoxPar *__restrict__ bps,
                                                      uint32_t *__restrict__ bins, uint32_t *__restrict__ order)
 {
     const uint32_t G = *n_groups;
@@ -819,7 +855,7 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const Group *__restrict__ g
     // whole warps iterate together so that the bin atomics can be aggregated per warp
     for (uint32_t g0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); g0 < G; g0 += stride) {
         const uint32_t g = g0 + lane;
-        const uint32_t key = g < G ? (uint32_t)layout_bin(groups[g].count) : 1024u;
+        const uint32_t key = g < G ? (uint32_t)layout_bin(groups[g], bps) : 1024u;
         const unsigned peers = __match_any_sync(0xffffffffu, key);
         const int leader = __ffs(peers) - 1;
         uint32_t base = 0;
@@ -829,21 +865,21 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const Group *__restrict__ g
     }
 }
 
-void launch_force_order(const Group *groups, const uint32_t *n_groups, uint32_t *bins, uint32_t *order,
-                        cudaStream_t s, int nsm)
+void launch_force_order(const Group *groups, const uint32_t *n_groups, const BoxPar *bps, uint32_t *bins,
+                        uint32_t *order, cudaStream_t s, int nsm)
 {
     cudaMemsetAsync(bins, 0, 128 * sizeof(uint32_t), s);
-    k_bin_count<<<nsm * 4, 256, 0, s>>>(groups, n_groups, bins);
+    k_bin_count<<<nsm * 4, 256, 0, s>>>(groups, n_groups, bps, bins);
     k_bin_scan<<<1, 32, 0, s>>>(bins);
-    k_bin_scatter<<<nsm * 4, 256, 0, s>>>(groups, n_groups, bins, order);
+    k_bin_scatter<<<nsm * 4, 256, 0, s>>>(groups, n_groups, bps, bins, order);
     g_launches += 3;
 }
 
 // Per device: the shared-memory opt-in of each force-kernel instantiation, and its
 // occupancy per block shape as (smem << 8) | blocks per SM (0 = not queried yet).
 struct ForceLaunchCache {
-    std::atomic<int> smem_set[3];
-    std::atomic<long long> occ[3][17];
+    std::atomic<int> smem_set[6];
+    std::atomic<long long> occ[6][17];
 };
 static ForceLaunchCache g_force_cache[kMaxDevices];
 
@@ -853,12 +889,57 @@ size_t force_smem_bytes(int chunk, int warps)
     return (size_t)warps * 2 * (size_t)chunk * sizeof(float4);
 }
 
+// The most i-particles of a pass for a box of n particles.  4 n / n_crit estimates its
+// groups within 15% (uniform, halo and Zel'dovich sets); the lines are in groups per
+// resident warp of one GB300 (fixed, and by the box alone, so that a box gives the same
+// bits on every GPU and in every batched call).  With several groups to a warp the widest
+// passes are best (each pass streams the list again); with few, the groups at the end of
+// the queue decide the time, and narrow passes, dealt out to several work items, even it
+// out.  Force stage uncapped / at cap 8 / 16 / 32: 16^3 uniform, n_crit 64 (0.1 groups a
+// warp) 0.053 / 0.026 / 0.037 / 0.053 ms; 32^3 uniform (0.8) 0.088 / 0.055 / 0.051 / 0.067;
+// 100 k halo particles, n_crit 128 (1.3) 0.342 / 0.137 / 0.129 / 0.184; 300 k, n_crit 96
+// (5.1) 0.336 / - / 0.276 / 0.268; 1 M, n_crit 128, with the second-order pass (12.8) 1.57 /
+// - / 1.74 / 1.46; at cap 64 1.49.  At n_crit 64 a cap of 32 splits only the largest groups
+// in two and gains nothing.
+static double box_groups(uint32_t n, int n_crit) { return 4.0 * (double)n / (double)n_crit; }
+constexpr double kRefWarps = 152.0 * 16.0;
+constexpr double kCapWarps = 14.0;  // groups per warp above which no pass is capped
+
+uint32_t force_pass_cap(uint32_t n, int n_crit)
+{
+    const double per_warp = box_groups(n, n_crit) / kRefWarps;
+    if (per_warp < 0.5) return 8;
+    if (per_warp < 3.0) return 16;
+    if (per_warp < kCapWarps && n_crit > 64) return 32;
+    return 0xffffffffu;
+}
+
+// Whether any box's passes are capped, and log2 of the work items a group's passes are
+// dealt out to: about one pass each, unless the groups of a batched call are many.
+void force_caps(const BoxPar *bps, int nbox, ForceArgs &a)
+{
+    double groups = 0.0;
+    uint32_t passes = 1;
+    for (int b = 0; b < nbox; b++) {
+        const uint32_t n = bps[b].p_end - bps[b].p_begin;
+        groups += box_groups(n, bps[b].n_crit);
+        a.capped = a.capped || bps[b].pass_cap != 0xffffffffu;
+        passes = std::max(passes, std::min(n, (uint32_t)bps[b].n_crit) / bps[b].pass_cap);
+    }
+    a.share = 0;
+    while (a.share < 5 && (2u << a.share) <= passes && groups * (2 << a.share) < 2.0 * kCapWarps * kRefWarps) a.share++;
+}
+
 void launch_force_f32(const ForceArgs &a, cudaStream_t s, int nsm, bool soft, bool quad)
 {
     const int threads = 32 * a.warps;
     const size_t smem = force_smem_bytes(a.chunk, a.warps);
-    auto kern = quad ? k_force_f32<false, true> : (soft ? k_force_f32<true, false> : k_force_f32<false, false>);
-    const int which = quad ? 2 : (soft ? 1 : 0);
+    using Kern = void (*)(ForceArgs);
+    static const Kern kerns[6] = {k_force_f32<false, false, false>, k_force_f32<true, false, false>,
+                                  k_force_f32<false, true, false>,  k_force_f32<false, false, true>,
+                                  k_force_f32<true, false, true>,   k_force_f32<false, true, true>};
+    const int which = (quad ? 2 : (soft ? 1 : 0)) + (a.capped ? 3 : 0);
+    const Kern kern = kerns[which];
     // the opt-in applies to the current device only; the occupancy is queried once per
     // device and shape (not while a stream is being captured)
     const int dev = current_device_index();

@@ -52,6 +52,7 @@ __global__ void k_noalloc_box(BoxPar *bp, DevStatus *st, float inv_rc2, float fo
         BoxPar b = {};
         b.inv_rc2 = inv_rc2;
         b.eps2 = eps2;
+        b.pass_cap = 0xffffffffu;
         b.force_scale = force_scale;
         *bp = b;
     }
