@@ -317,6 +317,7 @@ static int derive_box(const greem_params &p, uint32_t pb, uint32_t pe, BoxPar &b
     bp.n_crit = p.n_crit;
     bp.n_leaf = p.n_leaf;
     bp.pass_cap = force_pass_cap(pe - pb, p.n_crit);
+    bp.pass_cap64 = force_pass_cap_f64(pe - pb, p.n_crit);
     return GREEM_OK;
 }
 

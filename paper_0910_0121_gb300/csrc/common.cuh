@@ -50,6 +50,7 @@ struct BoxPar {
     float k52_f;           // (L/2^52)/r_cut rounded to float: fixed52 offsets -> r_cut units
     float inv_rc2;         // 1/r_cut^2: r_cut-unit accelerations -> physical
     float eps2;            // (eps/r_cut)^2
+    uint32_t pass_cap64;   // the same of the FP64 form (force_pass_cap_f64)
     uint32_t pass_cap;     // the most i-particles a pass of the force kernels takes (force_pass_cap)
     float force_scale;     // kForceUnit/r_cut^2: the pair loops' accelerations -> physical
     long long T_prune;     // prune a node iff S_gap > T_prune (exact form of the r_cut test)
@@ -280,6 +281,7 @@ struct ForceArgs {
     int warps;                 // warps per block
     bool capped = false;       // some box's pass_cap holds
     int share = 0;             // a group's passes are dealt out to 2^share work items
+    int share64 = 0;           // the same of the FP64 form
     // polls of each list-chunk wait, plus one (0: kWaitPolls); only a failure test
     // lowers it, through greem_debug_set
     uint32_t wait_polls1 = 0;
@@ -287,6 +289,7 @@ struct ForceArgs {
 void launch_force_order(const Group *groups, const uint32_t *n_groups, const BoxPar *bps, uint32_t *bins,
                         uint32_t *order, cudaStream_t s, int nsm);
 uint32_t force_pass_cap(uint32_t n, int n_crit);
+uint32_t force_pass_cap_f64(uint32_t n, int n_crit);
 void force_caps(const BoxPar *bps, int nbox, ForceArgs &a);  // a.capped and a.share
 // Dynamic shared memory of the FP32 force kernel, and its limit: the 227 KB a block may
 // opt in to, less room for the kernel's static shared memory (its mbarriers).

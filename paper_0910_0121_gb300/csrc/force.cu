@@ -914,18 +914,34 @@ uint32_t force_pass_cap(uint32_t n, int n_crit)
     return 0xffffffffu;
 }
 
+// The same for the FP64 form: its pairs take about 60 times the FP32 ones', so a pass costs
+// little beside its pairs and the end of the queue is evened out up to more groups a warp.
+// Force stage uncapped / at cap 8 / 16: 5 k uniform, n_crit 64 (0.2 groups a warp) 1.13 /
+// 0.22 / 0.31 ms; 60 k halo particles, n_crit 128 (0.8) 9.34 / 2.49 / 2.87; 64^3, n_crit 64
+// (5.7) 11.0 / 9.5 / 9.7; 700 k, n_crit 64 (23) 14.7 / 14.4 / 14.1.
+constexpr double kCapWarps64 = 60.0;
+uint32_t force_pass_cap_f64(uint32_t n, int n_crit)
+{
+    const double per_warp = box_groups(n, n_crit) / kRefWarps;
+    return per_warp < 8.0 ? 8 : (per_warp < kCapWarps64 ? 16 : 0xffffffffu);
+}
+
 // Whether any box's passes are capped, and log2 of the work items a group's passes are
 // dealt out to: about one pass each, unless the groups of a batched call are many.
 void force_caps(const BoxPar *bps, int nbox, ForceArgs &a)
 {
     double groups = 0.0;
-    uint32_t passes = 1;
+    uint32_t passes = 1, passes64 = 1;
     for (int b = 0; b < nbox; b++) {
         const uint32_t n = bps[b].p_end - bps[b].p_begin;
         groups += box_groups(n, bps[b].n_crit);
         a.capped = a.capped || bps[b].pass_cap != 0xffffffffu;
         passes = std::max(passes, std::min(n, (uint32_t)bps[b].n_crit) / bps[b].pass_cap);
+        passes64 = std::max(passes64, std::min(n, (uint32_t)bps[b].n_crit) / bps[b].pass_cap64);
     }
+    a.share64 = 0;
+    while (a.share64 < 5 && (2u << a.share64) <= passes64 && groups * (2 << a.share64) < 2.0 * kCapWarps64 * kRefWarps)
+        a.share64++;
     a.share = 0;
     while (a.share < 5 && (2u << a.share) <= passes && groups * (2 << a.share) < 2.0 * kCapWarps * kRefWarps) a.share++;
 }
@@ -966,7 +982,37 @@ void launch_force_f32(const ForceArgs &a, cudaStream_t s, int nsm, bool soft, bo
 // The same lists as index entries; absolute FP64 positions of particles and node
 // centres of mass, the entry's image shift, and Eq. 1-2 in FP64.  It is the plain form
 // the FP32 kernel is compared with.
-template <int I>
+//
+// An FP64 warp instruction holds its pipe for 64 cycles here, an integer or FP32 one for 1
+// or 2, so the kernel is bound by the number of FP64 instructions alone and everything
+// else is free: tests are made on the high words, a lane's pair out of range is masked by
+// integer selects, whole warps skip what none of their lanes needs (the rest of a pair
+// when all 32 are beyond r_cut, the u term when none is within r_cut/2), and the square
+// root starts from the FP32 unit.  Per pair 7 instructions for xi^2, 5 for w = 1/xi and 13
+// for the force with the cancellation-free form of Eq. 2 in units of 32/35 (the FP32
+// kernel's), 8 more with the u term; the plain form took about 62 (rsqrt(), divisions by
+// constants, FP64 compares).  64^3 halo mix, force stage: 24.0 -> 11.0 ms, 9.5 with the
+// capped passes below.  Against an 80-bit sum (4096 particles, theta 0) the median error is
+// 2.44e-16 (2.54e-16 before), the 99th percentile 3.3e-15 (3.4e-15).
+//
+// 1/sqrt(x): x = m 2^2q with m in [1, 4), the FP32 approximation y0 of 1/sqrt(m) (2^-22)
+// times 2^-q, and one third-order Householder step, y = y0 + y0 e (1/2 + 3/8 e), e = 1 - x
+// y0^2.  (5/16) e^3 is below 2^-64, y0^2 is exact (24 bits squared) and e exact to 2^-75,
+// which leaves the last rounding.
+__device__ __forceinline__ double rsqrt_fp64(double x)
+{
+    const int hi = __double2hiint(x);
+    if (hi < 0x00100000) return rsqrt(x);  // subnormal
+    const int ex = hi >> 20, odd = (ex & 1) ^ 1;
+    const int mb = ((127 + odd) << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)__double2loint(x) >> 29);
+    const int yb = __float_as_int(rsqrtf(__int_as_float(mb)));
+    const int q = (ex - 1023 - odd) >> 1;
+    const double y0 = __hiloint2double((yb >> 3) + 0x38000000 - (q << 20), (int)((unsigned)yb << 29));
+    const double e = fma(-x, y0 * y0, 1.0);
+    return fma(y0 * e, fma(e, 0.375, 0.5), y0);
+}
+
+template <int I, bool SOFT>
 __device__ __noinline__ void group_pass_f64(const ForceArgs &a, const Group &gr, const BoxPar &bp, uint32_t done,
                                             int S, unsigned long long lo, uint32_t len, Dbl4 *jb, int lane)
 {
@@ -975,7 +1021,8 @@ __device__ __noinline__ void group_pass_f64(const ForceArgs &a, const Group &gr,
     const int slot = lane & (li - 1);
     const int part = lane / li;
     const uint32_t gend = gr.begin + gr.count;
-    const double L = bp.L, ie = bp.inv_eta, eps2 = bp.eps * bp.eps;
+    const double L = bp.L, irc2 = 1.0 / (4.0 * bp.eta * bp.eta);  // 1/r_cut^2
+    const double eps2 = SOFT ? bp.eps * bp.eps * irc2 : 0.0;
     double xi[I], yi[I], zi[I], ax[I], ay[I], az[I];
 #pragma unroll
     for (int s = 0; s < I; s++) {
@@ -988,7 +1035,7 @@ __device__ __noinline__ void group_pass_f64(const ForceArgs &a, const Group &gr,
     }
     for (uint32_t c = 0; c < len; c += 32) {
         const uint32_t e = c + (uint32_t)lane;
-        Dbl4 jv = make_dbl4(1.0e30, 1.0e30, 1.0e30, 0.0);
+        Dbl4 jv = make_dbl4(-1.0e30, -1.0e30, -1.0e30, 0.0);  // out of range of every i-particle
         if (e < len) {
             const unsigned long long en = a.ilist[lo + e];
             const uint32_t idx = (uint32_t)en;
@@ -1004,39 +1051,60 @@ __device__ __noinline__ void group_pass_f64(const ForceArgs &a, const Group &gr,
         }
         jb[lane] = jv;
         __syncwarp();
-        const uint32_t nj = min(32u, len - c);
-        for (uint32_t t = (uint32_t)part; t < nj; t += (uint32_t)S) {
-            const Dbl4 j = jb[t];
+        // every part takes equally many entries (the loop votes)
+        const uint32_t nt = (min(32u, len - c) + (uint32_t)S - 1u) / (uint32_t)S;
+        for (uint32_t t = 0; t < nt; t++) {
+            const Dbl4 j = jb[t * (uint32_t)S + (uint32_t)part];
 #pragma unroll
             for (int s = 0; s < I; s++) {
                 const double dx = j.x - xi[s], dy = j.y - yi[s], dz = j.z - zi[s];
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                if (r2 > 0.0) {
-                    const double rinv = rsqrt(r2);
-                    const double R = r2 * rinv * ie;
-                    if (R < 2.0) {
-                        const double v = 1.0 - 0.5 * R;
-                        const double u = R < 1.0 ? 1.0 - R : 0.0;
-                        const double v2 = v * v, u2 = u * u;
-                        const double g = v2 * v2 * v * (8.0 / 35.0) * (((7.0 * R + 22.0) * R + 10.0) * R + 4.0) +
-                                         u2 * u2 * u2 * ((7.0 * R + 18.0) * R + 3.0) / 35.0;
-                        double rinv3;
-                        if (eps2 > 0.0) {
-                            const double rs = rsqrt(r2 + eps2);
-                            rinv3 = rs * rs * rs;
-                        } else {
-                            rinv3 = rinv * rinv * rinv;
-                        }
-                        const double f = j.w * g * rinv3;
-                        ax[s] += f * dx;
-                        ay[s] += f * dy;
-                        az[s] += f * dz;
+                double r2 = fma(dz, dz, fma(dy, dy, dx * dx)) * irc2;  // xi^2
+                const int hi = __double2hiint(r2);
+                // in range: 0 < xi^2 < 1 (a coincident pair adds nothing)
+                const bool in = (unsigned)hi < 0x3ff00000u && (hi | __double2loint(r2)) != 0;
+                if (!__any_sync(FULL, in)) continue;
+                const bool near = __any_sync(FULL, in && hi < 0x3fd00000);  // some xi < 1/2
+                r2 = in ? r2 : 0.75;
+                const double m = in ? j.w : 0.0;
+                const double w = rsqrt_fp64(r2);
+                double g;
+                if (__all_sync(FULL, !in || hi < 0x3fb00000)) {
+                    // every xi < 1/4: Eq. 2's inner branch as printed, g/xi^3 = (35/32) w^3 -
+                    // (14 - 56 xi^2 + 35 xi^3 + 48 xi^4 - 42 xi^5); g > 0.84 loses nothing
+                    const double x = r2 * w;
+                    const double q = fma(fma(fma(fma(x, -42.0, 48.0), x, 35.0), x, -56.0), r2, 14.0);
+                    if (SOFT) g = fma(-(x * r2), q, 1.09375);
+                    else g = fma(w * w, 1.09375 * w, -q);
+                } else {
+                    const double x = SOFT ? r2 * w : 0.0;
+                    const double v = SOFT ? 1.0 - x : fma(-r2, w, 1.0);
+                    const double v2 = v * v;
+                    const double cq = SOFT ? fma(fma(fma(x, 14.0, 22.0), x, 5.0), x, 1.0)
+                                           : fma(fma(w + 5.0, w, 22.0), w, 14.0);
+                    g = (v2 * v2) * (v * cq);
+                    if (near) {
+                        double u = fma(2.0, v, -1.0);
+                        u = __double2hiint(u) < 0 ? 0.0 : u;
+                        const double u3 = (u * u) * u;
+                        const double pq = SOFT ? fma(fma(x, 0.875, 1.125), x, 0.09375)
+                                               : fma(fma(w, 0.09375, 1.125), w, 0.875) * w;
+                        g = fma(u3, u3 * pq, g);
                     }
                 }
+                double f = m * g;
+                if (SOFT) {
+                    const double rs = rsqrt_fp64(r2 + eps2);
+                    f *= (rs * rs) * rs;
+                }
+                ax[s] = fma(f, dx, ax[s]);
+                ay[s] = fma(f, dy, ay[s]);
+                az[s] = fma(f, dz, az[s]);
             }
         }
         __syncwarp();
     }
+    // 1/r_cut^3 as the cube of the unit that scaled the distances
+    const double scale = kForceUnit * (irc2 * sqrt(irc2));
 #pragma unroll
     for (int s = 0; s < I; s++) {
         for (int o = li; o < 32; o <<= 1) {
@@ -1044,6 +1112,9 @@ __device__ __noinline__ void group_pass_f64(const ForceArgs &a, const Group &gr,
             ay[s] += __shfl_xor_sync(FULL, ay[s], o);
             az[s] += __shfl_xor_sync(FULL, az[s], o);
         }
+        ax[s] *= scale;
+        ay[s] *= scale;
+        az[s] *= scale;
     }
     if (part == 0) {
         double *acc = static_cast<double *>(a.acc);
@@ -1060,6 +1131,15 @@ __device__ __noinline__ void group_pass_f64(const ForceArgs &a, const Group &gr,
     }
 }
 
+// The pass with I i-particles per lane, softened or not.
+template <int I>
+__device__ __forceinline__ void run_pass_f64(const ForceArgs &a, const Group &gr, const BoxPar &bp, uint32_t done,
+                                             int S, unsigned long long lo, uint32_t len, Dbl4 *jb, int lane)
+{
+    if (bp.eps * bp.eps > 0.0) group_pass_f64<I, true>(a, gr, bp, done, S, lo, len, jb, lane);
+    else group_pass_f64<I, false>(a, gr, bp, done, S, lo, len, jb, lane);
+}
+
 __global__ void __launch_bounds__(256) k_force_f64(ForceArgs a)
 {
     __shared__ Dbl4 jbuf[8][32];
@@ -1067,10 +1147,13 @@ __global__ void __launch_bounds__(256) k_force_f64(ForceArgs a)
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (a.st->flags & ST_NODE_CAP) return;
     const uint32_t G = *a.n_groups;
+    const uint32_t others = (1u << a.share64) - 1u;
     for (;;) {
         unsigned long long gi = 0;
         if (lane == 0) gi = atomicAdd(&a.st->work[2], 1ull);
         gi = __shfl_sync(FULL, gi, 0);
+        uint32_t turn = (uint32_t)gi & others;  // the passes turn, turn + 2^share64, ... of one group
+        gi >>= a.share64;
         if (gi >= G) break;
         const uint32_t g = a.order ? a.order[gi] : (uint32_t)gi;
         const Group gr = a.groups[g];
@@ -1081,18 +1164,22 @@ __global__ void __launch_bounds__(256) k_force_f64(ForceArgs a)
         unsigned long long evals = 0;
         while (done < gr.count) {
             int S, I;
-            choose_layout(gr.count - done, S, I);
-            switch (I) {
-            case 1: group_pass_f64<1>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
-            case 2: group_pass_f64<2>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
-            case 3: group_pass_f64<3>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
-            case 4: group_pass_f64<4>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
-            case 5: group_pass_f64<5>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
-            case 6: group_pass_f64<6>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
-            case 7: group_pass_f64<7>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
-            default: group_pass_f64<8>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
-            }
+            choose_layout(min(gr.count - done, bp.pass_cap64), S, I);
             const uint32_t slots = (uint32_t)(32 / S) * (uint32_t)I;
+            const bool skip = turn != 0;  // another item's pass
+            turn = skip ? turn - 1u : others;
+            if (skip) {
+                done += slots;
+                continue;
+            }
+            switch (I) {
+            case 1: run_pass_f64<1>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
+            case 2: run_pass_f64<2>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
+            case 3: run_pass_f64<3>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
+            case 4: run_pass_f64<4>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
+            case 5: run_pass_f64<5>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;
+            default: run_pass_f64<6>(a, gr, bp, done, S, lo, len, jbuf[w], lane); break;  // kImax
+            }
             evals += (unsigned long long)slots * len;
             done += slots;
         }
@@ -1102,6 +1189,7 @@ __global__ void __launch_bounds__(256) k_force_f64(ForceArgs a)
 
 void launch_force_f64(const ForceArgs &a, cudaStream_t s, int nsm)
 {
+    static_assert(kImax == 6, "one case per number of i-particles");
     static std::atomic<int> cached[kMaxDevices];
     const int dev = current_device_index();
     int per_sm = dev >= 0 ? cached[dev].load() : 0;

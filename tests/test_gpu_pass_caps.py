@@ -44,7 +44,11 @@ def test_capped_passes(n, n_crit, eps):
     both = ctx.short_force_batched(pb, mb, [0, n, n + 2500], [greem.params(**kw), greem.params(**dict(kw, n_crit=32))])
     assert torch.equal(both[:n], acc)
     if n <= 200000:
-        ref = ctx.short_force(P, M, greem.params(precision=greem.F64, **kw))
+        k64 = dict(kw, precision=greem.F64)
+        ref = ctx.short_force(P, M, greem.params(**k64))
+        both = ctx.short_force_batched(pb, mb, [0, n, n + 2500],
+                                       [greem.params(**k64), greem.params(**dict(k64, n_crit=32, eps=1e-4))])
+        assert torch.equal(both[:n], ref)
         nr = ref.norm(dim=1)
         err = ((acc.double() - ref).norm(dim=1) / nr)[nr > 1e-6 * nr.median()]
         if err.numel():
