@@ -57,7 +57,7 @@ struct greem_ctx {
     DBuf<double> xs, ys, zs;
     DBuf<float> ms;
     // S3-S4
-    DBuf<uint8_t> d8, K8, nchild;
+    DBuf<uint8_t> d8, K8;
     DBuf<uint32_t> own, base, ctr, gflag, gidx;
     DBuf<Node> nodes;
     DBuf<Dbl4> raw, mom64;
@@ -464,7 +464,6 @@ static int size_buffers(greem_ctx *c, const RunCfg &r)
     ENS(irel, N);
     const size_t nc = c->node_cap;
     ENS(nodes, nc);
-    ENS(nchild, nc);
     ENS(ctr, nc);
     ENS(raw, nc);
     ENS(mom64, nc);
@@ -481,7 +480,7 @@ static int size_buffers(greem_ctx *c, const RunCfg &r)
         ENS(qlist, c->qcap * 3);
     }
     ENS(kids, nc * 8);
-    ENS(lvl, 192);
+    ENS(lvl, kLvlWords);
     ENS(bps, (size_t)r.nbox);
     ENS(box_off, (size_t)r.nbox + 1);
     ENS(st, 1);
@@ -617,11 +616,11 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     launch_gather(r.pos, r.mass, perm, N, c->box_off.p, nbox, c->bps.p, c->xs.p, c->ys.p, c->zs.p, c->ms.p, c->st.p,
                   s);
     ev_record(c, r, ev, 2);
-    launch_tree_prep(ks, N, c->box_off.p, nbox, c->bps.p, c->d8.p, c->K8.p, c->own.p, s);
+    launch_tree_prep(ks, N, c->box_off.p, nbox, c->bps.p, c->d8.p, c->K8.p, c->own.p, c->lvl.p, s);
     scan_u32(c->own.p, c->base.p, N, c->scratch.p, s);
     const uint32_t *n_nodes = c->base.p + N;
     launch_tree_fill(ks, N, c->box_off.p, nbox, c->d8.p, c->K8.p, c->base.p, c->nodes.p, ncap, c->st.p, s, nsm);
-    launch_tree_links(c->nodes.p, n_nodes, ncap, c->nchild.p, c->kids.p, s, nsm);
+    launch_tree_links(c->nodes.p, n_nodes, ncap, c->kids.p, c->lvl.p, s, nsm);
     // fork: the moments (FP64-bound) on s; the particle offsets and the groups (integer
     // work, reading only the tree) on the second stream
     cudaStream_t s2 = c->aux;
@@ -649,7 +648,7 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     cudaStreamWaitEvent(s, c->ev_join, 0);
     if (r.quad)
         launch_quadrupoles(c->nodes.p, n_nodes, ncap, c->kids.p, c->poff.p, c->noff.p, c->lvl.p, c->ctr.p,
-                           c->box_off.p, nbox, c->bps.p, c->quad.p, s, nsm);
+                           N, c->box_off.p, nbox, c->bps.p, c->quad.p, s, nsm);
     ev_record(c, r, ev, 4);
     if (r.lists_force) {
         ListArgs la;
@@ -956,7 +955,7 @@ void greem_destroy(greem_ctx *c)
     release(c->k0); release(c->k1); release(c->v0); release(c->v1); release(c->hist); release(c->scratch);
     release(c->rs_status); release(c->rs_runs);
     release(c->xs); release(c->ys); release(c->zs); release(c->ms);
-    release(c->d8); release(c->K8); release(c->nchild); release(c->own); release(c->base); release(c->ctr);
+    release(c->d8); release(c->K8); release(c->own); release(c->base); release(c->ctr);
     release(c->gflag); release(c->gidx); release(c->nodes); release(c->raw); release(c->mom64); release(c->noff);
     release(c->poff); release(c->pcell); release(c->lbox); release(c->irel); release(c->groups); release(c->gbox); release(c->quad);
     release(c->flist); release(c->ilist); release(c->loff);

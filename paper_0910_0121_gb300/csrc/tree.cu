@@ -14,7 +14,10 @@
 // prefix, so K_i comes from a sliding maximum over such windows.  Particle i then owns
 // the nodes (i, d_i) ... (i, K_i); an exclusive scan of the ownership counts numbers
 // the nodes in DFS preorder, because preorder is the order of (begin, level).
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <atomic>
 
 #include "common.cuh"
 
@@ -46,8 +49,10 @@ constexpr int kPrepHalo = 64;
 __global__ void __launch_bounds__(256) k_tree_prep(const uint64_t *__restrict__ keys, uint32_t N,
                                                    const uint32_t *__restrict__ box_off, int nbox,
                                                    const BoxPar *__restrict__ bps, uint8_t *__restrict__ d8,
-                                                   uint8_t *__restrict__ K8, uint32_t *__restrict__ own)
+                                                   uint8_t *__restrict__ K8, uint32_t *__restrict__ own,
+                                                   uint32_t *__restrict__ lvl)
 {
+    if (blockIdx.x == 0 && threadIdx.x < kLvlWords) lvl[threadIdx.x] = 0;  // counted by k_tree_links
     __shared__ int8_t ws[256 + kPrepHalo];
     const long long i0 = (long long)blockIdx.x * 256;
     for (int k = threadIdx.x; k < 256 + kPrepHalo; k += 256) {
@@ -91,9 +96,9 @@ __global__ void __launch_bounds__(256) k_tree_prep(const uint64_t *__restrict__ 
 }
 
 void launch_tree_prep(const uint64_t *keys, uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps,
-                      uint8_t *d8, uint8_t *K8, uint32_t *own, cudaStream_t s)
+                      uint8_t *d8, uint8_t *K8, uint32_t *own, uint32_t *lvl, cudaStream_t s)
 {
-    k_tree_prep<<<(N + 255) / 256, 256, 0, s>>>(keys, N, box_off, nbox, bps, d8, K8, own);
+    k_tree_prep<<<(N + 255) / 256, 256, 0, s>>>(keys, N, box_off, nbox, bps, d8, K8, own, lvl);
     g_launches++;
 }
 
@@ -214,13 +219,17 @@ __device__ __forceinline__ uint32_t node_count(const uint32_t *n_nodes, uint32_t
 
 // Parent links, child counts, the child table (up to 8 children per internal node,
 // unused slots kNone) and each node's child-octant mask (bits 16-23 of lvl; octant =
-// x<<2 | y<<1 | z of the child's cell within the parent's): the children of an internal
+// x<<2 | y<<1 | z of the child's cell within the parent's); the internal nodes of each
+// level are counted on the way (lvl[level]).  The children of an internal
 // node p are p+1 and then the skip chain while it stays inside p's particle range, in
 // Morton order, so slot q holds the child in the octant of the mask's (q+1)-th set bit.
 __global__ void __launch_bounds__(256) k_tree_links(Node *__restrict__ nodes, const uint32_t *__restrict__ n_nodes,
-                                                    uint32_t node_cap, uint8_t *__restrict__ nchild,
-                                                    uint32_t *__restrict__ kids)
+                                                    uint32_t node_cap, uint32_t *__restrict__ kids,
+                                                    uint32_t *__restrict__ lvl)
 {
+    __shared__ uint32_t cnt_[32];
+    if (threadIdx.x < 32) cnt_[threadIdx.x] = 0;
+    __syncthreads();
     const uint32_t nn = node_count(n_nodes, node_cap);
     for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < nn; p += gridDim.x * blockDim.x) {
         const Node np = nodes[p];
@@ -242,18 +251,20 @@ __global__ void __launch_bounds__(256) k_tree_links(Node *__restrict__ nodes, co
                 c = nc.skip;
             }
             nodes[p].lvl = np.lvl | (mask << 16);
+            atomicAdd(&cnt_[np.lvl & 255u], 1u);
         }
-        nchild[p] = (uint8_t)cnt;
         uint4 *kp = reinterpret_cast<uint4 *>(kids + (size_t)p * 8);
         kp[0] = make_uint4(slot[0], slot[1], slot[2], slot[3]);
         kp[1] = make_uint4(slot[4], slot[5], slot[6], slot[7]);
     }
+    __syncthreads();
+    if (threadIdx.x < 32 && cnt_[threadIdx.x]) atomicAdd(&lvl[threadIdx.x], cnt_[threadIdx.x]);
 }
 
-void launch_tree_links(Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, uint8_t *nchild, uint32_t *kids,
+void launch_tree_links(Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, uint32_t *kids, uint32_t *lvl,
                        cudaStream_t s, int nsm)
 {
-    k_tree_links<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, node_cap, nchild, kids);
+    k_tree_links<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, node_cap, kids, lvl);
     g_launches++;
 }
 
@@ -266,73 +277,51 @@ void launch_tree_links(Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, 
 // children's raw moments in child order.  Every sum has a fixed order, so the result
 // does not depend on scheduling.
 //
-// lvl[0..64): nodes per bucket, lvl[64..128): bucket start, lvl[128..192): cursor.
-constexpr int kLeafBucket = 32;
+// lvl[0..32): internal nodes per level (k_tree_links), lvl[32..64): each level's first place
+// in inodes, lvl[64..96): places taken so far.
 
-__device__ __forceinline__ uint32_t node_bucket(const Node &nd)
+// The exclusive prefix sums of the level counts, by the first warp of a block (smem start).
+__device__ __forceinline__ void level_starts(const uint32_t *__restrict__ lvl, uint32_t *start)
 {
-    return (nd.lvl & 256u) ? kLeafBucket + min(nd.end - nd.begin, 31u) : (nd.lvl & 255u);
-}
-
-__global__ void __launch_bounds__(256) k_node_buckets(const Node *__restrict__ nodes,
-                                                      const uint32_t *__restrict__ n_nodes, uint32_t node_cap,
-                                                      uint32_t *__restrict__ lvl)
-{
-    __shared__ uint32_t cnt[64];
-    if (threadIdx.x < 64) cnt[threadIdx.x] = 0;
-    __syncthreads();
-    const uint32_t nn = node_count(n_nodes, node_cap);
-    const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < nn) {
-        const Node nd = nodes[n];
-        if (!(nd.lvl & 256u)) atomicAdd(&cnt[node_bucket(nd)], 1u);  // leaves are summed by tiles
-    }
-    __syncthreads();
-    if (threadIdx.x < 64 && cnt[threadIdx.x]) atomicAdd(&lvl[threadIdx.x], cnt[threadIdx.x]);
-}
-
-__global__ void k_level_scan(uint32_t *lvl)
-{
-    const uint32_t lane = threadIdx.x;
-    const uint32_t v0 = lvl[lane], v1 = lvl[32 + lane];
-    uint32_t x0 = v0, x1 = v1;
+    if (threadIdx.x < 32) {
+        const uint32_t v = lvl[threadIdx.x];
+        uint32_t x = v;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
-        if (lane >= (uint32_t)o) {
-            x0 += y0;
-            x1 += y1;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (threadIdx.x >= (uint32_t)o) x += y;
         }
+        start[threadIdx.x] = x - v;
     }
-    const uint32_t tot0 = __shfl_sync(0xffffffffu, x0, 31);
-    lvl[64 + lane] = lvl[128 + lane] = x0 - v0;
-    lvl[96 + lane] = lvl[160 + lane] = tot0 + x1 - v1;
 }
 
-// Places every node in its bucket: a slot within the block from a shared-memory counter,
-// then one global atomic per bucket and block.  The order within a bucket is free (its
-// nodes are summed independently).
+// Places every internal node in its level's stretch of inodes: a slot within the block from
+// a shared-memory counter, then one global atomic per level and block.  The order within a
+// level is free (its nodes are summed independently).
 __global__ void __launch_bounds__(256) k_level_scatter(const Node *__restrict__ nodes,
                                                        const uint32_t *__restrict__ n_nodes, uint32_t node_cap,
                                                        uint32_t *__restrict__ lvl, uint32_t *__restrict__ inodes)
 {
-    __shared__ uint32_t cnt[64], base[64];
-    if (threadIdx.x < 64) cnt[threadIdx.x] = 0;
+    __shared__ uint32_t cnt[32], base[32], start[32];
+    if (threadIdx.x < 32) cnt[threadIdx.x] = 0;
+    level_starts(lvl, start);
     __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x < 32) lvl[32 + threadIdx.x] = start[threadIdx.x];
     const uint32_t nn = node_count(n_nodes, node_cap);
     const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t key = 0, slot = 0;
     bool inner = false;
     if (n < nn) {
-        const Node nd = nodes[n];
-        inner = !(nd.lvl & 256u);  // leaves are summed by tiles
+        const uint32_t l = nodes[n].lvl;
+        inner = !(l & 256u);  // leaves are summed by tiles
         if (inner) {
-            key = node_bucket(nd);
+            key = l & 255u;
             slot = atomicAdd(&cnt[key], 1u);
         }
     }
     __syncthreads();
-    if (threadIdx.x < 64 && cnt[threadIdx.x]) base[threadIdx.x] = atomicAdd(&lvl[128 + threadIdx.x], cnt[threadIdx.x]);
+    if (threadIdx.x < 32 && cnt[threadIdx.x])
+        base[threadIdx.x] = start[threadIdx.x] + atomicAdd(&lvl[64 + threadIdx.x], cnt[threadIdx.x]);
     __syncthreads();
     if (inner) inodes[base[key] + slot] = n;
 }
@@ -428,43 +417,112 @@ __global__ void __launch_bounds__(256) k_moments_leaf_tiled(const Node *__restri
     }
 }
 
+// The raw moments of internal node p: its children's, in child order.
+__device__ __forceinline__ void sum_children(uint32_t p, const uint32_t *__restrict__ kids, Dbl4 *raw)
+{
+    const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
+    const uint4 k0 = kp[0], k1 = kp[1];
+    const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+    Dbl4 a = make_dbl4(0.0, 0.0, 0.0, 0.0);
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+        if (kk[q] == kNone) break;
+        const Dbl4 r = raw[kk[q]];
+        a.x += r.x;
+        a.y += r.y;
+        a.z += r.z;
+        a.w += r.w;
+    }
+    raw[p] = a;
+}
+
 __global__ void __launch_bounds__(256) k_moments_level(int level, const uint32_t *__restrict__ lvl,
                                                        const uint32_t *__restrict__ inodes,
-                                                       const uint32_t *__restrict__ kids, Dbl4 *__restrict__ raw)
+                                                       const uint32_t *__restrict__ kids, Dbl4 *raw)
 {
-    const uint32_t b = lvl[64 + level], e = b + lvl[level];
-    for (uint32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x) {
-        const uint32_t p = inodes[i];
-        const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
-        const uint4 k0 = kp[0], k1 = kp[1];
-        const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-        Dbl4 a = make_dbl4(0.0, 0.0, 0.0, 0.0);
-#pragma unroll
-        for (int q = 0; q < 8; q++) {
-            if (kk[q] == kNone) break;
-            const Dbl4 r = raw[kk[q]];
-            a.x += r.x;
-            a.y += r.y;
-            a.z += r.z;
-            a.w += r.w;
-        }
-        raw[p] = a;
+    const uint32_t b = lvl[32 + level], e = b + lvl[level];
+    for (uint32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x)
+        sum_children(inodes[i], kids, raw);
+}
+
+// Every level in one launch, for smaller trees: one cluster of blocks goes through the
+// levels, deepest first, with a hardware cluster barrier after each that holds nodes (the
+// 21 launches of the form above cost more than their sums).  Its 16 blocks have a tenth of
+// the GPU's FP64 rate, which sets the line kClusterMax.
+constexpr int kClusterCtas = 16;
+constexpr int kClusterThreads = 512;
+
+template <class F>
+__device__ __forceinline__ void cluster_levels(const uint32_t *__restrict__ lvl, const uint32_t *__restrict__ inodes,
+                                               F &&f)
+{
+    const auto cl = cooperative_groups::this_cluster();
+    __shared__ uint32_t cnt[32], start[32];
+    if (threadIdx.x < 32) {
+        cnt[threadIdx.x] = lvl[threadIdx.x];
+        start[threadIdx.x] = lvl[32 + threadIdx.x];
+    }
+    __syncthreads();
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    for (int level = kMaxLevel - 1; level >= 0; level--) {
+        const uint32_t c = cnt[level];
+        if (!c) continue;  // the same in every block
+        for (uint32_t i = t; i < c; i += nt) f(inodes[start[level] + i], level);
+        cl.sync();
     }
 }
+
+__global__ void __launch_bounds__(kClusterThreads) k_moments_cluster(const uint32_t *__restrict__ lvl,
+                                                                     const uint32_t *__restrict__ inodes,
+                                                                     const uint32_t *__restrict__ kids, Dbl4 *raw)
+{
+    cluster_levels(lvl, inodes, [&](uint32_t p, int) { sum_children(p, kids, raw); });
+}
+
+// Launches a kernel as one cluster of kClusterCtas blocks (beyond the portable 8: an opt-in
+// per kernel and device, kept in `set`).
+template <class... P, class... A>
+static void launch_cluster(void (*kern)(P...), std::atomic<bool> *set, cudaStream_t s, A... args)
+{
+    const int dev = current_device_index();
+    if (dev < 0 || !set[dev].load()) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (dev >= 0) set[dev].store(true);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = kClusterCtas;
+    cfg.blockDim = kClusterThreads;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kClusterCtas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, P(args)...);
+    g_launches++;
+}
+
+// The line between the two forms, in particles.  Tree stage with launches / with a cluster
+// (replayed calls): 4 k 0.082 / 0.057 ms, 32 k 0.087 / 0.071, 100 k 0.132 / 0.119, 300 k
+// 0.154 / 0.138, 500 k (not replayed) 0.215 / 0.170, 1 M 0.233 / 0.232 and second moments
+// 0.123 / 0.150, 2 M 0.334 / 0.360.
+constexpr uint32_t kClusterMax = 700000;
 
 void launch_moments(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *kids,
                     const uint32_t *base, uint32_t N, const double *xs, const double *ys, const double *zs,
                     const float *ms, Dbl4 *raw, uint32_t *lvl, uint32_t *inodes, cudaStream_t s, int nsm)
 {
-    (void)nsm;
-    cudaMemsetAsync(lvl, 0, 192 * sizeof(uint32_t), s);
     const unsigned grid = (node_cap + 255) / 256;
-    k_node_buckets<<<grid, 256, 0, s>>>(nodes, n_nodes, node_cap, lvl);
-    k_level_scan<<<1, 32, 0, s>>>(lvl);
     k_level_scatter<<<grid, 256, 0, s>>>(nodes, n_nodes, node_cap, lvl, inodes);
     k_moments_leaf_tiled<<<(N + kLeafTile - 1) / kLeafTile, 256, 0, s>>>(nodes, n_nodes, node_cap, base, N, xs, ys,
                                                                        zs, ms, raw);
-    g_launches += 4;
+    g_launches += 2;
+    if (N <= kClusterMax) {
+        static std::atomic<bool> set[kMaxDevices];
+        launch_cluster(k_moments_cluster, set, s, lvl, inodes, kids, raw);
+        return;
+    }
     for (int level = kMaxLevel - 1; level >= 0; level--) {
         k_moments_level<<<nsm * 4, 256, 0, s>>>(level, lvl, inodes, kids, raw);
         g_launches++;
@@ -508,54 +566,77 @@ __global__ void __launch_bounds__(256) k_quad_leaf(const Node *__restrict__ node
     }
 }
 
+// The second moments of internal node p of the given level from its children's.
+__device__ __forceinline__ void quad_children(uint32_t p, int level, const Node *__restrict__ nodes,
+                                              const uint32_t *__restrict__ kids, const float4 *__restrict__ noff,
+                                              const uint32_t *__restrict__ box_off, int nbox,
+                                              const BoxPar *__restrict__ bps, float4 *quad)
+{
+    const Node np = nodes[p];
+    const float kf = bps[box_of(np.begin, box_off, nbox)].k_f;
+    const int hp = 1 << (kMaxLevel - level);
+    const float4 cp = noff[p];
+    float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
+    const uint4 k0 = kp[0], k1 = kp[1];
+    const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+#pragma unroll
+    for (int t = 0; t < 8; t++) {
+        const uint32_t c = kk[t];
+        if (c == kNone) break;
+        const Node nc = nodes[c];
+        const int hc = hp >> 1;
+        const float4 cc = noff[c];
+        // child COM - node COM: cell-centre difference (exact integer in u) and COM offsets
+        const float dx = fmaf((float)(2 * ((int)nc.ix - (int)np.ix) + hc - hp), kf, cc.x - cp.x);
+        const float dy = fmaf((float)(2 * ((int)nc.iy - (int)np.iy) + hc - hp), kf, cc.y - cp.y);
+        const float dz = fmaf((float)(2 * ((int)nc.iz - (int)np.iz) + hc - hp), kf, cc.z - cp.z);
+        const float4 q0 = quad[2 * (size_t)c], q1 = quad[2 * (size_t)c + 1];
+        const float mx = cc.w * dx, my = cc.w * dy, mz = cc.w * dz;
+        q[0] += fmaf(mx, dx, q0.x);
+        q[1] += fmaf(my, dy, q0.y);
+        q[2] += fmaf(mz, dz, q0.z);
+        q[3] += fmaf(mx, dy, q0.w);
+        q[4] += fmaf(mx, dz, q1.x);
+        q[5] += fmaf(my, dz, q1.y);
+    }
+    quad_store(quad, p, q);
+}
+
 __global__ void __launch_bounds__(256) k_quad_level(int level, const uint32_t *__restrict__ lvl,
                                                     const uint32_t *__restrict__ inodes,
                                                     const Node *__restrict__ nodes, const uint32_t *__restrict__ kids,
                                                     const float4 *__restrict__ noff,
                                                     const uint32_t *__restrict__ box_off, int nbox,
-                                                    const BoxPar *__restrict__ bps, float4 *__restrict__ quad)
+                                                    const BoxPar *__restrict__ bps, float4 *quad)
 {
-    const uint32_t b = lvl[64 + level], e = b + lvl[level];
-    for (uint32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x) {
-        const uint32_t p = inodes[i];
-        const Node np = nodes[p];
-        const float kf = bps[box_of(np.begin, box_off, nbox)].k_f;
-        const int hp = 1 << (kMaxLevel - level);
-        const float4 cp = noff[p];
-        float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
-        const uint4 k0 = kp[0], k1 = kp[1];
-        const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-#pragma unroll
-        for (int t = 0; t < 8; t++) {
-            const uint32_t c = kk[t];
-            if (c == kNone) break;
-            const Node nc = nodes[c];
-            const int hc = hp >> 1;
-            const float4 cc = noff[c];
-            // child COM - node COM: cell-centre difference (exact integer in u) and COM offsets
-            const float dx = fmaf((float)(2 * ((int)nc.ix - (int)np.ix) + hc - hp), kf, cc.x - cp.x);
-            const float dy = fmaf((float)(2 * ((int)nc.iy - (int)np.iy) + hc - hp), kf, cc.y - cp.y);
-            const float dz = fmaf((float)(2 * ((int)nc.iz - (int)np.iz) + hc - hp), kf, cc.z - cp.z);
-            const float4 q0 = quad[2 * (size_t)c], q1 = quad[2 * (size_t)c + 1];
-            const float mx = cc.w * dx, my = cc.w * dy, mz = cc.w * dz;
-            q[0] += fmaf(mx, dx, q0.x);
-            q[1] += fmaf(my, dy, q0.y);
-            q[2] += fmaf(mz, dz, q0.z);
-            q[3] += fmaf(mx, dy, q0.w);
-            q[4] += fmaf(mx, dz, q1.x);
-            q[5] += fmaf(my, dz, q1.y);
-        }
-        quad_store(quad, p, q);
-    }
+    const uint32_t b = lvl[32 + level], e = b + lvl[level];
+    for (uint32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x)
+        quad_children(inodes[i], level, nodes, kids, noff, box_off, nbox, bps, quad);
+}
+
+__global__ void __launch_bounds__(kClusterThreads) k_quad_cluster(
+    const uint32_t *__restrict__ lvl, const uint32_t *__restrict__ inodes, const Node *__restrict__ nodes,
+    const uint32_t *__restrict__ kids, const float4 *__restrict__ noff, const uint32_t *__restrict__ box_off, int nbox,
+    const BoxPar *__restrict__ bps, float4 *quad)
+{
+    cluster_levels(lvl, inodes, [&](uint32_t p, int level) {
+        quad_children(p, level, nodes, kids, noff, box_off, nbox, bps, quad);
+    });
 }
 
 void launch_quadrupoles(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *kids,
                         const float4 *poff, const float4 *noff, const uint32_t *lvl, const uint32_t *inodes,
-                        const uint32_t *box_off, int nbox, const BoxPar *bps, float4 *quad, cudaStream_t s, int nsm)
+                        uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps, float4 *quad, cudaStream_t s,
+                        int nsm)
 {
     k_quad_leaf<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, node_cap, poff, noff, quad);
     g_launches++;
+    if (N <= kClusterMax) {
+        static std::atomic<bool> set[kMaxDevices];
+        launch_cluster(k_quad_cluster, set, s, lvl, inodes, nodes, kids, noff, box_off, nbox, bps, quad);
+        return;
+    }
     for (int level = kMaxLevel - 1; level >= 0; level--) {
         k_quad_level<<<nsm * 4, 256, 0, s>>>(level, lvl, inodes, nodes, kids, noff, box_off, nbox, bps, quad);
         g_launches++;
