@@ -58,7 +58,7 @@ struct greem_ctx {
     DBuf<float> ms;
     // S3-S4
     DBuf<uint8_t> d8, K8;
-    DBuf<uint32_t> own, base, ctr, gflag, gidx;
+    DBuf<uint32_t> own, base, ctr, gstat;
     DBuf<Node> nodes;
     DBuf<Dbl4> raw, mom64;
     DBuf<float4> noff, poff, irel;
@@ -469,8 +469,7 @@ static int size_buffers(greem_ctx *c, const RunCfg &r)
     ENS(mom64, nc);
     ENS(noff, nc);
     ENS(lbox, nc);
-    ENS(gflag, nc);
-    ENS(gidx, nc + 1);
+    ENS(gstat, group_status_words(nc));
     ENS(groups, nc);
     ENS(gbox, nc * 2);
     if (r.quad) {
@@ -481,6 +480,7 @@ static int size_buffers(greem_ctx *c, const RunCfg &r)
     }
     ENS(kids, nc * 8);
     ENS(lvl, kLvlWords);
+    ENS(bins, kBinWords);
     ENS(bps, (size_t)r.nbox);
     ENS(box_off, (size_t)r.nbox + 1);
     ENS(st, 1);
@@ -490,7 +490,6 @@ static int size_buffers(greem_ctx *c, const RunCfg &r)
         ENS(llen, nc);
         ENS(lraw, nc);
         ENS(order, nc);
-        ENS(bins, 128);
         ENS(stack, (size_t)c->nsm * kListBlocksPerSM * kListWarps * c->stack_cap);
         ENS(flist, c->list_cap);
         if (r.index_lists) ENS(ilist, c->list_cap);
@@ -525,11 +524,13 @@ struct InlineBoxes {
     int nbox;
 };
 
-// Also clears the status word (a memset could sit on a copy engine too).
+// Also clears the status word and the sort's counters (a memset could sit on a copy engine
+// too).
 __global__ void k_set_boxes(InlineBoxes ib, BoxPar *__restrict__ bps, uint32_t *__restrict__ box_off,
-                            DevStatus *__restrict__ st)
+                            DevStatus *__restrict__ st, uint32_t *__restrict__ hist, uint32_t n_hist)
 {
     const int t = threadIdx.x;
+    for (uint32_t i = t; i < n_hist; i += blockDim.x) hist[i] = 0u;
     if (t < ib.nbox) bps[t] = ib.b[t];
     if (t <= ib.nbox) box_off[t] = ib.off[t];
     uint32_t *w = reinterpret_cast<uint32_t *>(st);
@@ -544,18 +545,20 @@ __global__ void k_status_out(const DevStatus *__restrict__ src, DevStatus *dst)
 }
 
 // Clears the status word and uploads the per-box constants.
-static void upload_boxes(greem_ctx *c, int nbox, cudaStream_t s)
+static void upload_boxes(greem_ctx *c, uint32_t N, int nbox, cudaStream_t s)
 {
+    const uint32_t n_hist = (uint32_t)radix_hist_elems(N);
     if (nbox <= kInlineBoxes) {
         InlineBoxes ib;
         memset(&ib, 0, sizeof(ib));
         ib.nbox = nbox;
         for (int b = 0; b < nbox; b++) ib.b[b] = c->bps_host[b];
         for (int b = 0; b <= nbox; b++) ib.off[b] = c->box_off_host[b];
-        k_set_boxes<<<1, 32, 0, s>>>(ib, c->bps.p, c->box_off.p, c->st.p);
+        k_set_boxes<<<1, 512, 0, s>>>(ib, c->bps.p, c->box_off.p, c->st.p, c->hist.p, n_hist);
         greem::g_launches++;
     } else {
         cudaMemsetAsync(c->st.p, 0, sizeof(DevStatus), s);
+        cudaMemsetAsync(c->hist.p, 0, sizeof(uint32_t) * n_hist, s);
         cudaMemcpyAsync(c->bps.p, c->bps_host, sizeof(BoxPar) * nbox, cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(c->box_off.p, c->box_off_host, sizeof(uint32_t) * (nbox + 1), cudaMemcpyHostToDevice, s);
     }
@@ -604,11 +607,16 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     const int nbox = r.nbox;
     const int nsm = c->nsm;
     const uint32_t ncap = (uint32_t)std::min<size_t>(c->node_cap, 0xFFFFFFF0u);
-    upload_boxes(c, nbox, s);
+    upload_boxes(c, N, nbox, s);
     ev_record(c, r, ev, 0);
-    launch_keys(r.pos, N, c->box_off.p, nbox, c->bps.p, c->k0.p, c->st.p, s);
-    ev_record(c, r, ev, 1);
     const int box_passes = nbox <= 1 ? 0 : (nbox <= 256 ? 1 : 2);
+    ZeroList zk = {};  // the sort's look-back words and the first scan's
+    zk.p[0] = reinterpret_cast<uint32_t *>(c->rs_status.p);
+    zk.n[0] = (uint32_t)(2 * radix_status_used(N, radix_key_passes() + box_passes));
+    zk.p[1] = c->scratch.p;
+    zk.n[1] = (uint32_t)scan_zero_words(N);
+    launch_keys(r.pos, N, c->box_off.p, nbox, c->bps.p, c->k0.p, box_passes, c->hist.p, zk, c->st.p, s, nsm);
+    ev_record(c, r, ev, 1);
     uint64_t *ks = nullptr;
     uint32_t *perm = nullptr;
     radix_sort(c->k0.p, c->k1.p, c->v0.p, c->v1.p, N, radix_key_passes(), box_passes, c->box_off.p, nbox, c->hist.p,
@@ -616,8 +624,15 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     launch_gather(r.pos, r.mass, perm, N, c->box_off.p, nbox, c->bps.p, c->xs.p, c->ys.p, c->zs.p, c->ms.p, c->st.p,
                   s);
     ev_record(c, r, ev, 2);
-    launch_tree_prep(ks, N, c->box_off.p, nbox, c->bps.p, c->d8.p, c->K8.p, c->own.p, c->lvl.p, s);
-    scan_u32(c->own.p, c->base.p, N, c->scratch.p, s);
+    ZeroList zt = {};  // the level counts, the group selection's look-back words, the work-order bins
+    zt.p[0] = c->lvl.p;
+    zt.n[0] = kLvlWords;
+    zt.p[1] = c->gstat.p;
+    zt.n[1] = (uint32_t)group_status_words(ncap);
+    zt.p[2] = c->bins.p;
+    zt.n[2] = kBinWords;
+    launch_tree_prep(ks, N, c->box_off.p, nbox, c->bps.p, c->d8.p, c->K8.p, c->own.p, zt, s);
+    scan_u32(c->own.p, c->base.p, N, c->scratch.p, c->st.p, s, nullptr, true);
     const uint32_t *n_nodes = c->base.p + N;
     launch_tree_fill(ks, N, c->box_off.p, nbox, c->d8.p, c->K8.p, c->base.p, c->nodes.p, ncap, c->st.p, s, nsm);
     launch_tree_links(c->nodes.p, n_nodes, ncap, c->kids.p, c->lvl.p, s, nsm);
@@ -628,15 +643,15 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     cudaStreamWaitEvent(s2, c->ev_fork, 0);
     launch_leaf_offsets(ks, c->K8.p, N, c->box_off.p, nbox, c->bps.p, c->xs.p, c->ys.p, c->zs.p, c->ms.p, c->poff.p,
                         c->pcell.p, s2);
-    launch_group_flags(c->nodes.p, n_nodes, ncap, c->box_off.p, nbox, c->bps.p, c->gflag.p, s2, nsm);
-    scan_u32(c->gflag.p, c->gidx.p, ncap, c->scratch.p, s2);
-    const uint32_t *n_groups = c->gidx.p + ncap;
-    launch_group_fill(c->nodes.p, n_nodes, ncap, c->gflag.p, c->gidx.p, c->box_off.p, nbox, c->groups.p, s2, nsm);
+    uint32_t *n_groups = c->lvl.p + 96;
+    launch_group_select(c->nodes.p, n_nodes, ncap, c->box_off.p, nbox, c->bps.p, c->groups.p, n_groups, c->gstat.p,
+                        c->st.p, s2);
     launch_group_box(c->groups.p, n_groups, c->pcell.p, c->gbox.p, s2, nsm);
     launch_leaf_boxes(c->nodes.p, n_nodes, ncap, c->pcell.p, c->lbox.p, s2, nsm);
-    launch_record_counts(n_nodes, n_groups, c->st.p, ncap, s2);
-    if (r.lists_force)
+    if (r.lists_force) {
+        launch_force_order(c->groups.p, n_groups, c->bps.p, c->bins.p, c->order.p, s2, nsm);
         launch_start_table(c->nodes.p, c->kids.p, c->base.p, c->bps.p, nbox, c->tbl_kmax, c->tbl.p, c->st.p, s2);
+    }
     cudaEventRecord(c->ev_join, s2);
     launch_moments(c->nodes.p, n_nodes, ncap, c->kids.p, c->base.p, N, c->xs.p, c->ys.p, c->zs.p, c->ms.p, c->raw.p,
                    c->lvl.p,
@@ -672,14 +687,12 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
         la.llen = c->llen.p;
         la.lraw = c->lraw.p;
         la.qcnt = r.quad ? c->qcnt.p : nullptr;
-        if (r.quad) cudaMemsetAsync(c->qcnt.p, 0, sizeof(uint32_t) * ncap, s);
         la.cap = c->list_cap;
         la.page = c->page;
         la.tbl = c->tbl.p;
         la.st = c->st.p;
         launch_lists(la, s, nsm);
         ev_record(c, r, ev, 5);
-        launch_force_order(c->groups.p, n_groups, c->bps.p, c->bins.p, c->order.p, s, nsm);
         ForceArgs fa = {};
         fa.wait_polls1 = c->wait_polls1;
         fa.groups = c->groups.p;
@@ -706,7 +719,7 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
         if (r.precision == GREEM_F64) launch_force_f64(fa, s, nsm);
         else launch_force_f32(fa, s, nsm, r.soft);
         if (r.quad) {
-            scan_u32(c->qcnt.p, c->qoff.p, ncap, c->scratch.p, s);
+            scan_u32(c->qcnt.p, c->qoff.p, ncap, c->scratch.p, c->st.p, s, n_groups);
             fa.qoff = c->qoff.p;
             fa.qcnt = c->qcnt.p;
             fa.qlist = c->qlist.p;
@@ -956,7 +969,7 @@ void greem_destroy(greem_ctx *c)
     release(c->rs_status); release(c->rs_runs);
     release(c->xs); release(c->ys); release(c->zs); release(c->ms);
     release(c->d8); release(c->K8); release(c->own); release(c->base); release(c->ctr);
-    release(c->gflag); release(c->gidx); release(c->nodes); release(c->raw); release(c->mom64); release(c->noff);
+    release(c->gstat); release(c->nodes); release(c->raw); release(c->mom64); release(c->noff);
     release(c->poff); release(c->pcell); release(c->lbox); release(c->irel); release(c->groups); release(c->gbox); release(c->quad);
     release(c->flist); release(c->ilist); release(c->loff);
     release(c->llen); release(c->lraw); release(c->kids); release(c->stack); release(c->order); release(c->bins);
@@ -1833,7 +1846,7 @@ int greem_domain_pack(greem_ctx *c, const double *pos, const float *mass, const 
         !cuda_ok(cudaMemcpyAsync(c->dom_boxes.p, boxes, sizeof(int32_t) * 6 * ndom, cudaMemcpyHostToDevice, s)))
         return GREEM_ERR_CUDA;
     launch_dom_count(pos, n, L, bp.pow2_e, c->dom_boxes.p, ndom, c->dom.p, c->dom_cnt.p, c->st.p, s);
-    scan_u32(c->dom_cnt.p, c->dom_cnt.p, ncnt, c->scratch.p, s);
+    scan_u32(c->dom_cnt.p, c->dom_cnt.p, ncnt, c->scratch.p, c->st.p, s);
     launch_dom_scatter(pos, mass, ids, n, L, c->dom.p, c->dom_cnt.p, ndom, pos_out, mass_out, ids_out, s);
     std::vector<uint32_t> off(ncnt + 1);
     unsigned flags = 0;
@@ -1891,7 +1904,7 @@ int greem_let_export(greem_ctx *c, const int32_t *boxes, int ndom, int self, int
         const int nb = std::min(kLetChunk, nrecv - j0);
         launch_let_count(c->nodes.p, n_nodes, ncap, lb.data() + j0, nb, c->bps.p, c->pcell.p, c->let_flag.p,
                          c->let_cnt.p, s, c->nsm);
-        scan_u32(c->let_cnt.p, c->let_cnt.p, run * nb, c->scratch.p, s);
+        scan_u32(c->let_cnt.p, c->let_cnt.p, run * nb, c->scratch.p, c->st.p, s);
         launch_let_ends(c->let_cnt.p, ncap, nb, c->let_ends.p, s);
         uint32_t ends[kLetChunk + 1];
         if (!cuda_ok(cudaGetLastError()) ||

@@ -165,20 +165,75 @@ __device__ __forceinline__ int box_of(uint32_t i, const uint32_t *__restrict__ b
     return lo;
 }
 
-// ---------------------------------------------------------------- host launchers
-struct ScanScratch {
-    uint32_t *buf = nullptr;  // block sums for every level
-    size_t cap = 0;
+// Words that a kernel zeroes on the side for kernels after it (counters, look-back words):
+// one launch less than a memset each.
+struct ZeroList {
+    uint32_t *p[3];
+    uint32_t n[3];
 };
-size_t scan_scratch_elems(size_t n);
-// out[0..n] = exclusive prefix sums of in[0..n), out[n] = total.  in may alias out.
-void scan_u32(const uint32_t *in, uint32_t *out, size_t n, uint32_t *scratch, cudaStream_t s);
+__device__ __forceinline__ void zero_words(const ZeroList &z, uint32_t t, uint32_t threads)
+{
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+        for (uint32_t i = t; i < z.n[k]; i += threads) z.p[k][i] = 0u;
+}
+
+__device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned long long v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long *p)
+{
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Single-pass prefix sums over tiles (decoupled look-back, Merrill & Garland 2016): the sum
+// over the tiles before `tile`, whose own sum is tot; status: one zeroed word per tile.  By
+// one whole warp, 32 predecessors at a time.  Tiles are taken by ticket, so a block waits
+// only on blocks that started before it; the wait is bounded (ST_TIMEOUT, and the sum is
+// then too small, never too large).
+constexpr unsigned long long kTileAgg = 1ull << 62, kTilePrefix = 2ull << 62;
+__device__ __forceinline__ uint32_t tile_prefix(unsigned long long *status, uint32_t tile, uint32_t tot, DevStatus *st)
+{
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) st_relaxed_u64(status + tile, (tile == 0 ? kTilePrefix : kTileAgg) | tot);
+    if (tile == 0) return 0;
+    uint32_t excl = 0, polls = 0;
+    for (long long j = (long long)tile - 1;;) {
+        const unsigned long long w = j - lane >= 0 ? ld_relaxed_u64(status + (j - lane)) : kTilePrefix;
+        const unsigned have = __ballot_sync(0xffffffffu, (w >> 62) != 0), pre = __ballot_sync(0xffffffffu, (w >> 62) == 2);
+        const int last = pre ? __ffs(pre) - 1 : 31;  // the nearest published prefix, or the whole window
+        const unsigned need = 0xffffffffu >> (31 - last);
+        if ((have & need) != need) {
+            if (++polls < kWaitPolls) continue;
+            if (lane == 0) atomicOr(&st->flags, ST_TIMEOUT);
+            break;
+        }
+        excl += __reduce_add_sync(0xffffffffu, lane <= last ? (uint32_t)w : 0u);
+        if (pre) break;
+        j -= 32;
+    }
+    if (lane == 0) st_relaxed_u64(status + tile, kTilePrefix | (excl + tot));
+    return excl;
+}
+
+// ---------------------------------------------------------------- host launchers
+size_t scan_scratch_elems(size_t n);  // the first scan_zero_words(n) of them are zeroed for the scan
+size_t scan_zero_words(size_t n);
+// out[0..n] = exclusive prefix sums of in[0..n), out[n] = total.  in may alias out.  n_dev:
+// the number of elements on the device (at most n), or null.  zeroed: the scratch is zero.
+void scan_u32(const uint32_t *in, uint32_t *out, size_t n, uint32_t *scratch, DevStatus *st, cudaStream_t s,
+              const uint32_t *n_dev = nullptr, bool zeroed = false);
 
 // S1-S2 (keys_sort.cu)
 void launch_keys(const double *pos, uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps,
-                 uint64_t *keys, DevStatus *st, cudaStream_t s);
+                 uint64_t *keys, int box_passes, uint32_t *hist, const ZeroList &zero, DevStatus *st, cudaStream_t s,
+                 int nsm);
 size_t radix_hist_elems(uint32_t n);
 size_t radix_status_elems(uint32_t n);
+size_t radix_status_used(uint32_t n, int passes);  // of them, the words that must be zero
 size_t radix_runs_elems(uint32_t n);
 int radix_key_passes();
 void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t n, int key_passes, int box_passes,
@@ -189,9 +244,9 @@ void launch_gather(const double *pos, const float *mass, const uint32_t *perm, u
                    cudaStream_t s);
 
 // S3-S4 (tree.cu)
-constexpr int kLvlWords = 96;  // words of lvl: see launch_moments
+constexpr int kLvlWords = 128;  // words of lvl: see launch_moments; [96]: the number of groups
 void launch_tree_prep(const uint64_t *keys, uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps,
-                      uint8_t *d8, uint8_t *K8, uint32_t *own, uint32_t *lvl, cudaStream_t s);
+                      uint8_t *d8, uint8_t *K8, uint32_t *own, const ZeroList &zero, cudaStream_t s);
 void launch_tree_fill(const uint64_t *keys, uint32_t N, const uint32_t *box_off, int nbox, const uint8_t *d8,
                       const uint8_t *K8, const uint32_t *base, Node *nodes, uint32_t node_cap, DevStatus *st,
                       cudaStream_t s, int nsm);
@@ -212,16 +267,12 @@ void launch_leaf_offsets(const uint64_t *keys, const uint8_t *K8, uint32_t N, co
 void launch_node_finish(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const Dbl4 *raw,
                         const uint32_t *box_off, int nbox, const BoxPar *bps, Dbl4 *mom64, float4 *noff,
                         cudaStream_t s, int nsm);
-void launch_group_flags(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *box_off,
-                        int nbox, const BoxPar *bps, uint32_t *flag, cudaStream_t s, int nsm);
-void launch_group_fill(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *flag,
-                       const uint32_t *gidx, const uint32_t *box_off, int nbox, Group *groups, cudaStream_t s,
-                       int nsm);
+size_t group_status_words(size_t node_cap);
+void launch_group_select(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *box_off, int nbox,
+                         const BoxPar *bps, Group *groups, uint32_t *n_groups, uint32_t *status, DevStatus *st,
+                         cudaStream_t s);
 void launch_group_box(const Group *groups, const uint32_t *n_groups, const unsigned long long *pcell, int4 *gbox,
                       cudaStream_t s, int nsm);
-void launch_record_counts(const uint32_t *n_nodes, const uint32_t *n_groups, DevStatus *st, uint32_t node_cap,
-                          cudaStream_t s);
-
 // S5 (lists.cu)
 struct ListArgs {
     const Node *nodes;
@@ -288,6 +339,7 @@ struct ForceArgs {
     // lowers it, through greem_debug_set
     uint32_t wait_polls1 = 0;
 };
+constexpr int kBinWords = 128;  // zeroed before launch_force_order
 void launch_force_order(const Group *groups, const uint32_t *n_groups, const BoxPar *bps, uint32_t *bins,
                         uint32_t *order, cudaStream_t s, int nsm);
 uint32_t force_pass_cap(uint32_t n, int n_crit);

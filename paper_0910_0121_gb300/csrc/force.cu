@@ -827,28 +827,27 @@ __global__ void __launch_bounds__(256) k_bin_count(const Group *__restrict__ gro
     if (threadIdx.x < 64 && sb[threadIdx.x]) atomicAdd(&bins[threadIdx.x], sb[threadIdx.x]);
 }
 
-__global__ void k_bin_scan(uint32_t *bins)
-{
-    const uint32_t lane = threadIdx.x;
-    const uint32_t v0 = bins[lane], v1 = bins[32 + lane];
-    uint32_t x0 = v0, x1 = v1;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
-        if (lane >= (uint32_t)o) {
-            x0 += y0;
-            x1 += y1;
-        }
-    }
-    const uint32_t tot0 = __shfl_sync(0xffffffffu, x0, 31);
-    bins[64 + lane] = x0 - v0;        // cursors
-    bins[96 + lane] = tot0 + x1 - v1;
-}
-
 __global__ void __launch_bounds__(256) k_bin_scatter(const Group *__restrict__ groups, const uint32_t *n_groups,
                                                      const BoxPar *__restrict__ bps,
                                                      uint32_t *__restrict__ bins, uint32_t *__restrict__ order)
 {
+    __shared__ uint32_t start[64];
+    if (threadIdx.x < 32) {  // the bins' first places, from their counts
+        const uint32_t v0 = bins[threadIdx.x], v1 = bins[32 + threadIdx.x];
+        uint32_t x0 = v0, x1 = v1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
+            if (threadIdx.x >= (uint32_t)o) {
+                x0 += y0;
+                x1 += y1;
+            }
+        }
+        const uint32_t tot0 = __shfl_sync(0xffffffffu, x0, 31);
+        start[threadIdx.x] = x0 - v0;
+        start[32 + threadIdx.x] = tot0 + x1 - v1;
+    }
+    __syncthreads();
     const uint32_t G = *n_groups;
     const int lane = threadIdx.x & 31;
     const uint32_t stride = gridDim.x * blockDim.x;
@@ -859,7 +858,7 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const Group *__restrict__ g
         const unsigned peers = __match_any_sync(0xffffffffu, key);
         const int leader = __ffs(peers) - 1;
         uint32_t base = 0;
-        if (g < G && lane == leader) base = atomicAdd(&bins[64 + key], (uint32_t)__popc(peers));
+        if (g < G && lane == leader) base = start[key] + atomicAdd(&bins[64 + key], (uint32_t)__popc(peers));
         base = __shfl_sync(0xffffffffu, base, leader);
         if (g < G) order[base + __popc(peers & ((1u << lane) - 1u))] = g;
     }
@@ -868,11 +867,9 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const Group *__restrict__ g
 void launch_force_order(const Group *groups, const uint32_t *n_groups, const BoxPar *bps, uint32_t *bins,
                         uint32_t *order, cudaStream_t s, int nsm)
 {
-    cudaMemsetAsync(bins, 0, 128 * sizeof(uint32_t), s);
     k_bin_count<<<nsm * 4, 256, 0, s>>>(groups, n_groups, bps, bins);
-    k_bin_scan<<<1, 32, 0, s>>>(bins);
     k_bin_scatter<<<nsm * 4, 256, 0, s>>>(groups, n_groups, bps, bins, order);
-    g_launches += 3;
+    g_launches += 2;
 }
 
 // Per device: the shared-memory opt-in of each force-kernel instantiation, and its

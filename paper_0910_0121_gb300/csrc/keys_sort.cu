@@ -5,6 +5,7 @@
 // to 2^21-1, and the three indices are bit-interleaved with x as the high bit of each
 // 3-bit digit.  Every FP64 step uses explicit round-to-nearest intrinsics so that no
 // multiply-add is fused: the key is a pure function of the IEEE inputs.
+#include <algorithm>
 #include <atomic>
 
 #include "cells.cuh"
@@ -23,14 +24,10 @@ __device__ __forceinline__ uint64_t spread3(uint32_t v)
     return x;
 }
 
-__global__ void __launch_bounds__(256) k_keys(const double *__restrict__ pos, uint32_t N,
-                                              const uint32_t *__restrict__ box_off, int nbox,
-                                              const BoxPar *__restrict__ bps, uint64_t *__restrict__ keys,
-                                              DevStatus *st)
+// The key of particle i (0 with the status set for a non-finite position).
+__device__ __forceinline__ uint64_t particle_key(const double *__restrict__ pos, uint32_t i, const BoxPar &bp,
+                                                 DevStatus *st)
 {
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const BoxPar &bp = bps[box_of(i, box_off, nbox)];
     const double L = bp.L, invL = bp.inv_L;
     double x = pos[3 * (size_t)i], y = pos[3 * (size_t)i + 1], z = pos[3 * (size_t)i + 2];
     // finite test on the exponent bits (integer pipe)
@@ -39,8 +36,7 @@ __global__ void __launch_bounds__(256) k_keys(const double *__restrict__ pos, ui
     };
     if (nonfinite(x) || nonfinite(y) || nonfinite(z)) {
         atomicOr(&st->flags, ST_NONFINITE);
-        keys[i] = 0;
-        return;
+        return 0;
     }
     uint32_t cx, cy, cz;
     if (bp.pow2_e != kNotPow2) {
@@ -53,14 +49,7 @@ __global__ void __launch_bounds__(256) k_keys(const double *__restrict__ pos, ui
         cy = c.y;
         cz = c.z;
     }
-    keys[i] = (spread3(cx) << 2) | (spread3(cy) << 1) | spread3(cz);
-}
-
-void launch_keys(const double *pos, uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps,
-                 uint64_t *keys, DevStatus *st, cudaStream_t s)
-{
-    k_keys<<<(N + 255) / 256, 256, 0, s>>>(pos, N, box_off, nbox, bps, keys, st);
-    g_launches++;
+    return (spread3(cx) << 2) | (spread3(cy) << 1) | spread3(cz);
 }
 
 // ------------------------------------------------------------------ radix sort
@@ -107,9 +96,9 @@ constexpr size_t kRsSmem = (size_t)kRsTile * (sizeof(uint64_t) + sizeof(uint32_t
 
 static inline uint32_t rs_tiles(uint32_t n) { return (n + kRsTile - 1) / kRsTile; }
 
-// u32 words: [passes][256] digit counts, [passes][256] digit starts, [passes] tickets, then
-// phase B's counts of long and middle runs and their work counters
-size_t radix_hist_elems(uint32_t) { return (size_t)kRsMaxPasses * 512 + kRsMaxPasses + 4; }
+// u32 words: [passes][256] digit counts, [passes] tickets, then phase B's counts of long and
+// middle runs and their work counters
+size_t radix_hist_elems(uint32_t) { return (size_t)kRsMaxPasses * 256 + kRsMaxPasses + 4; }
 // phase B's lists of runs: (start, end) pairs of kShortRun + 1 .. kWarpRun pairs (sorted
 // by a warp), then of more (sorted by a block)
 constexpr int kWarpRun = 64;
@@ -119,6 +108,7 @@ size_t radix_runs_elems(uint32_t n) { return 2 * ((size_t)mid_cap(n) + runs_cap(
 int radix_key_passes() { return kRsKeyPasses; }
 // u64 look-back words: [passes][tiles][256]
 size_t radix_status_elems(uint32_t n) { return (size_t)kRsMaxPasses * rs_tiles(n) * 256; }
+size_t radix_status_used(uint32_t n, int passes) { return (size_t)passes * rs_tiles(n) * 256; }
 
 // SRC 0: digit = key bits [shift, shift+8); SRC 1: digit = bits of the box of the value.
 template <int SRC>
@@ -141,28 +131,36 @@ __device__ __forceinline__ unsigned digit_peers(uint32_t d)
     return peers;
 }
 
-// All digit histograms in one pass over the unsorted keys (the box digits from the box
-// of each input index).  A warp whose lanes share a digit adds it with one shared
-// atomic (the usual case for the high digits of spatially ordered input); otherwise
-// every lane adds its own.
-__global__ void __launch_bounds__(256) k_rs_hist_all(const uint64_t *__restrict__ key, uint32_t n, int key_passes,
-                                                     int box_passes, const uint32_t *__restrict__ box_off, int nbox,
-                                                     uint32_t *__restrict__ hist, int kshift0)
+// S1, and on the way what the sort needs: all digit histograms (the box digits from the box
+// of each input index), counted from the keys in registers, and zeroed look-back words.  A
+// warp whose lanes share a digit adds it with one shared atomic (the usual case for the high
+// digits of spatially ordered input); otherwise every lane adds its own.  The blocks stay
+// for the whole array, so that each adds its counts to the global ones once (hist is zero
+// on entry).
+__global__ void __launch_bounds__(256) k_keys(const double *__restrict__ pos, uint32_t n,
+                                              const uint32_t *__restrict__ box_off, int nbox,
+                                              const BoxPar *__restrict__ bps, uint64_t *__restrict__ keys,
+                                              int box_passes, uint32_t *__restrict__ hist, ZeroList zero, DevStatus *st)
 {
     __shared__ uint32_t h[kRsMaxPasses][256];
-    const int passes = key_passes + box_passes;
+    const int passes = kRsKeyPasses + box_passes;
     for (int d = threadIdx.x; d < passes * 256; d += blockDim.x) (&h[0][0])[d] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const uint32_t stride = gridDim.x * blockDim.x;
+    zero_words(zero, blockIdx.x * blockDim.x + threadIdx.x, stride);
     for (uint32_t i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {
         const uint32_t i = i0 + (uint32_t)lane;
         const bool ok = i < n;
-        const uint64_t k = ok ? key[i] : 0ull;
-        const uint32_t b = (ok && box_passes) ? (uint32_t)box_of(i, box_off, nbox) : 0u;
+        const uint32_t b = ok ? (uint32_t)box_of(i, box_off, nbox) : 0u;
+        uint64_t k = 0;
+        if (ok) {
+            k = particle_key(pos, i, bps[b], st);
+            keys[i] = k;
+        }
         for (int p = 0; p < passes; p++) {
-            const uint32_t d = ok ? (p < key_passes ? (uint32_t)(k >> (kshift0 + 8 * p)) & 255u
-                                                    : (b >> (8 * (p - key_passes))) & 255u)
+            const uint32_t d = ok ? (p < kRsKeyPasses ? (uint32_t)(k >> (kRsLowBits + 8 * p)) & 255u
+                                                      : (b >> (8 * (p - kRsKeyPasses))) & 255u)
                                   : 256u;
             const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
             if (__all_sync(0xffffffffu, d == d0)) {
@@ -177,43 +175,20 @@ __global__ void __launch_bounds__(256) k_rs_hist_all(const uint64_t *__restrict_
         if ((&h[0][0])[d]) atomicAdd(&hist[d], (&h[0][0])[d]);
 }
 
-// Exclusive scan of each pass's 256 counts into its digit starts (one warp per pass).
-__global__ void k_rs_digit_starts(uint32_t *hist, int passes)
+void launch_keys(const double *pos, uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps,
+                 uint64_t *keys, int box_passes, uint32_t *hist, const ZeroList &zero, DevStatus *st, cudaStream_t s,
+                 int nsm)
 {
-    const int p = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (p >= passes) return;
-    const uint32_t *c = hist + p * 256;
-    uint32_t *o = hist + kRsMaxPasses * 256 + p * 256;
-    uint32_t carry = 0;
-    for (int b = 0; b < 256; b += 32) {
-        const uint32_t v = c[b + lane];
-        uint32_t x = v;
-#pragma unroll
-        for (int q = 1; q < 32; q <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, q);
-            if (lane >= q) x += y;
-        }
-        o[b + lane] = carry + x - v;
-        carry += __shfl_sync(0xffffffffu, x, 31);
-    }
-}
-
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned long long v)
-{
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long *p)
-{
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
+    const unsigned grid = std::min<unsigned>((N + 255) / 256, (unsigned)nsm * 8);
+    k_keys<<<grid, 256, 0, s>>>(pos, N, box_off, nbox, bps, keys, box_passes, hist, zero, st);
+    g_launches++;
 }
 
 template <int SRC>
 __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const uint64_t *__restrict__ kin,
                                                              const uint32_t *__restrict__ vin,
                                                              uint64_t *__restrict__ kout, uint32_t *__restrict__ vout,
-                                                             uint32_t n, int shift, const uint32_t *__restrict__ dstart,
+                                                             uint32_t n, int shift, const uint32_t *__restrict__ counts,
                                                              unsigned long long *status, uint32_t *ticket,
                                                              const uint32_t *__restrict__ box_off, int nbox,
                                                              DevStatus *st)
@@ -224,7 +199,7 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
     __shared__ uint32_t wcnt[kRsWarps][256];
     __shared__ uint32_t lstart[256];
     __shared__ uint32_t gbase[256];
-    __shared__ uint32_t wsum[kRsWarps];
+    __shared__ uint32_t wsum[kRsWarps], dsum[kRsWarps];
     __shared__ uint32_t s_tile;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     for (int d = tid; d < kRsWarps * 256; d += kRsThreads) (&wcnt[0][0])[d] = 0;
@@ -274,11 +249,26 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
         const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
-    if (lane == 31) wsum[w] = x;
+    // and the digits' first places in the whole output, from the counts of the whole input
+    const uint32_t dcount = counts[tid];
+    uint32_t dx = dcount;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, dx, o);
+        if (lane >= o) dx += y;
+    }
+    if (lane == 31) {
+        wsum[w] = x;
+        dsum[w] = dx;
+    }
     __syncthreads();
-    uint32_t wb = 0;
-    for (int ww = 0; ww < w; ww++) wb += wsum[ww];
+    uint32_t wb = 0, db = 0;
+    for (int ww = 0; ww < w; ww++) {
+        wb += wsum[ww];
+        db += dsum[ww];
+    }
     lstart[tid] = wb + x - tot;
+    const uint32_t dstart = db + dx - dcount;
     __syncthreads();
 #pragma unroll
     for (int t = 0; t < kRsItems; t++) {
@@ -293,7 +283,7 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
     // the tile sits in shared memory in digit order; look back for the exclusive prefix
     // of each digit over the earlier tiles
     if (tile == 0) {
-        gbase[tid] = dstart[tid];
+        gbase[tid] = dstart;
     } else {
         // look back over windows of up to kRsLook predecessors, loaded together: add
         // published counts from the nearest one backwards until a published prefix (done)
@@ -332,7 +322,7 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
             }
         }
         st_relaxed_u64(my, kRsPrefix | (excl + tot));
-        gbase[tid] = dstart[tid] + (uint32_t)excl;
+        gbase[tid] = dstart + (uint32_t)excl;
     }
     __syncthreads();
     const uint32_t tbase = tile * kRsTile;
@@ -385,8 +375,8 @@ static __device__ __noinline__ void sort_short_run(uint64_t *__restrict__ key, u
 
 // One thread per pair; the thread at the head of a run of two or more sorts a run of up
 // to kShortRun pairs itself and lists a longer one, its end found by binary search (the
-// top bits are sorted within a box): up to kWarpRun pairs for k_runs_warp (mid, n_mid),
-// more for k_runs_long (runs, n_long).  Other threads only read the top bits of pairs that
+// top bits are sorted within a box): up to kWarpRun pairs (mid, n_mid), more
+// (runs, n_long): both for k_runs_rest.  Other threads only read the top bits of pairs that
 // runs permute among themselves, so the concurrent sorts do not disturb them.
 __global__ void __launch_bounds__(256) k_runs_short(uint64_t *__restrict__ key, uint32_t *__restrict__ val, uint32_t n,
                                                     const uint32_t *__restrict__ box_off, int nbox,
@@ -436,7 +426,7 @@ __global__ void __launch_bounds__(256) k_runs_short(uint64_t *__restrict__ key, 
 // and l + 32; a 64-element bitonic network sorts the unique keys (low bits << 14 |
 // position), the step between the two halves inside each lane, the others by shuffles;
 // then every lane fetches the pairs its sorted keys name.
-__global__ void __launch_bounds__(256) k_runs_warp(uint64_t *__restrict__ key, uint32_t *__restrict__ val,
+static __device__ __forceinline__ void sort_mid_runs(uint64_t *__restrict__ key, uint32_t *__restrict__ val,
                                                    const uint32_t *__restrict__ mid, uint32_t mid_cap_,
                                                    const uint32_t *__restrict__ n_mid, uint32_t *__restrict__ ctr)
 {
@@ -489,16 +479,20 @@ __global__ void __launch_bounds__(256) k_runs_warp(uint64_t *__restrict__ key, u
     }
 }
 
-// The listed runs, one block each: up to kRunCap pairs by a bitonic sort in shared memory
+// The middle runs, then the long ones, one block each: up to kRunCap pairs by a bitonic sort in shared memory
 // of (low bits << 14 | position in the run), unique keys whose order is the stable one;
 // longer runs by one warp, three stable 9-bit LSD passes over the low 27 bits through the
 // other ping-pong buffer (tkey, tval) at the same positions, then copied back.
-__global__ void __launch_bounds__(kRunThreads) k_runs_long(uint64_t *__restrict__ key, uint32_t *__restrict__ val,
+__global__ void __launch_bounds__(kRunThreads) k_runs_rest(uint64_t *__restrict__ key, uint32_t *__restrict__ val,
                                                            uint64_t *__restrict__ tkey, uint32_t *__restrict__ tval,
                                                            const uint32_t *__restrict__ runs, uint32_t run_cap,
                                                            const uint32_t *__restrict__ n_long,
-                                                           uint32_t *__restrict__ ctr)
+                                                           uint32_t *__restrict__ ctr,
+                                                           const uint32_t *__restrict__ mid, uint32_t mid_cap_,
+                                                           const uint32_t *__restrict__ n_mid,
+                                                           uint32_t *__restrict__ mid_ctr)
 {
+    sort_mid_runs(key, val, mid, mid_cap_, n_mid, mid_ctr);
     extern __shared__ __align__(16) unsigned char run_smem[];
     uint64_t *comp = reinterpret_cast<uint64_t *>(run_smem);
     uint32_t *vals = reinterpret_cast<uint32_t *>(run_smem + (size_t)kRunCap * sizeof(uint64_t));
@@ -604,6 +598,7 @@ __global__ void __launch_bounds__(kRunThreads) k_runs_long(uint64_t *__restrict_
     }
 }
 
+// k_keys has counted the digits (hist) and zeroed the rest of hist and the status words.
 void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t n, int key_passes, int box_passes,
                 const uint32_t *box_off, int nbox, uint32_t *hist, unsigned long long *status, uint32_t *runs,
                 DevStatus *st, uint64_t **k_out, uint32_t **v_out, cudaStream_t s, int nsm)
@@ -614,24 +609,19 @@ void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t
     if (dev < 0 || !attr_set[dev].load()) {
         cudaFuncSetAttribute(k_rs_onesweep<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRsSmem);
         cudaFuncSetAttribute(k_rs_onesweep<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRsSmem);
-        cudaFuncSetAttribute(k_runs_long, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunSmem);
+        cudaFuncSetAttribute(k_runs_rest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunSmem);
         if (dev >= 0) attr_set[dev].store(true);
     }
     const uint32_t ntile = rs_tiles(n);
     const int passes = key_passes + box_passes;
-    cudaMemsetAsync(hist, 0, sizeof(uint32_t) * radix_hist_elems(n), s);
-    cudaMemsetAsync(status, 0, sizeof(unsigned long long) * (size_t)passes * ntile * 256, s);
-    k_rs_hist_all<<<nsm * 4, 256, 0, s>>>(k0, n, key_passes, box_passes, box_off, nbox, hist, kRsLowBits);
-    k_rs_digit_starts<<<1, 32 * passes, 0, s>>>(hist, passes);
-    g_launches += 2;
     uint64_t *ki = k0, *ko = k1;
     uint32_t *vi = nullptr, *vo = v1;  // first pass generates the identity values
     uint32_t *vfree = v0;
     for (int p = 0; p < passes; p++) {
         const bool boxp = p >= key_passes;
         const int shift = boxp ? 8 * (p - key_passes) : kRsLowBits + 8 * p;
-        const uint32_t *ds = hist + kRsMaxPasses * 256 + p * 256;
-        uint32_t *tk = hist + kRsMaxPasses * 512 + p;
+        const uint32_t *ds = hist + p * 256;
+        uint32_t *tk = hist + kRsMaxPasses * 256 + p;
         unsigned long long *sw = status + (size_t)p * ntile * 256;
         if (boxp) {
             k_rs_onesweep<1><<<ntile, kRsThreads, kRsSmem, s>>>(ki, vi, ko, vo, n, shift, ds, sw, tk, box_off, nbox, st);
@@ -649,13 +639,13 @@ void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t
     }
     // phase B: each run of equal top bits by its low bits, in place in (ki, vi); ko and vo
     // hold nothing that is still needed and serve the one-warp path as scratch
-    uint32_t *n_long = hist + kRsMaxPasses * 512 + kRsMaxPasses;  // n_long, long work, n_mid, mid work
+    uint32_t *n_long = hist + kRsMaxPasses * 256 + kRsMaxPasses;  // n_long, long work, n_mid, mid work
     uint32_t *mid = runs + 2 * (size_t)runs_cap(n);
     k_runs_short<<<(n + 255) / 256, 256, 0, s>>>(ki, vi, n, box_off, nbox, runs, runs_cap(n), n_long, mid, mid_cap(n),
                                                   n_long + 2);
-    k_runs_warp<<<nsm * 4, 256, 0, s>>>(ki, vi, mid, mid_cap(n), n_long + 2, n_long + 3);
-    k_runs_long<<<nsm, kRunThreads, kRunSmem, s>>>(ki, vi, ko, vo, runs, runs_cap(n), n_long, n_long + 1);
-    g_launches += 3;
+    k_runs_rest<<<nsm * 2, kRunThreads, kRunSmem, s>>>(ki, vi, ko, vo, runs, runs_cap(n), n_long, n_long + 1, mid,
+                                                       mid_cap(n), n_long + 2, n_long + 3);
+    g_launches += 2;
     *k_out = ki;
     *v_out = vi;
 }

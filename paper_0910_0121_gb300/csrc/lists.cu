@@ -603,6 +603,7 @@ __global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(Lis
                 a.loff[g] = 0;
                 a.llen[g] = 0;
                 a.lraw[g] = 0;
+                if (a.qcnt) a.qcnt[g] = 0;
             }
             continue;
         }
@@ -612,6 +613,7 @@ __global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(Lis
                     a.loff[g] = 0;
                     a.llen[g] = 0;
                     a.lraw[g] = 0;
+                    if (a.qcnt) a.qcnt[g] = 0;
                 }
                 continue;
             }

@@ -50,9 +50,9 @@ __global__ void __launch_bounds__(256) k_tree_prep(const uint64_t *__restrict__ 
                                                    const uint32_t *__restrict__ box_off, int nbox,
                                                    const BoxPar *__restrict__ bps, uint8_t *__restrict__ d8,
                                                    uint8_t *__restrict__ K8, uint32_t *__restrict__ own,
-                                                   uint32_t *__restrict__ lvl)
+                                                   ZeroList zero)
 {
-    if (blockIdx.x == 0 && threadIdx.x < kLvlWords) lvl[threadIdx.x] = 0;  // counted by k_tree_links
+    zero_words(zero, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
     __shared__ int8_t ws[256 + kPrepHalo];
     const long long i0 = (long long)blockIdx.x * 256;
     for (int k = threadIdx.x; k < 256 + kPrepHalo; k += 256) {
@@ -96,9 +96,9 @@ __global__ void __launch_bounds__(256) k_tree_prep(const uint64_t *__restrict__ 
 }
 
 void launch_tree_prep(const uint64_t *keys, uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps,
-                      uint8_t *d8, uint8_t *K8, uint32_t *own, uint32_t *lvl, cudaStream_t s)
+                      uint8_t *d8, uint8_t *K8, uint32_t *own, const ZeroList &zero, cudaStream_t s)
 {
-    k_tree_prep<<<(N + 255) / 256, 256, 0, s>>>(keys, N, box_off, nbox, bps, d8, K8, own, lvl);
+    k_tree_prep<<<(N + 255) / 256, 256, 0, s>>>(keys, N, box_off, nbox, bps, d8, K8, own, zero);
     g_launches++;
 }
 
@@ -803,43 +803,70 @@ __device__ __forceinline__ bool group_cond(const Node &nd, const BoxPar &bp)
     return k >= bp.lmin && ((int)(nd.end - nd.begin) <= bp.n_crit || (nd.lvl & 256u));
 }
 
-__global__ void __launch_bounds__(256) k_group_flags(const Node *__restrict__ nodes,
-                                                     const uint32_t *__restrict__ n_nodes, uint32_t node_cap,
-                                                     const uint32_t *__restrict__ box_off, int nbox,
-                                                     const BoxPar *__restrict__ bps, uint32_t *__restrict__ flag)
+// The groups in preorder, in one pass over the nodes: tiles of kSelTile nodes find their
+// groups, look back for the number before them (tile_prefix) and write them.  Also records
+// the counts for the host.  status: the ticket, a pad, then a look-back word per tile, all
+// zero.
+constexpr uint32_t kSelItems = 4, kSelTile = 256 * kSelItems;
+size_t group_status_words(size_t node_cap) { return 2 + 2 * ((node_cap + kSelTile - 1) / kSelTile + 1); }
+
+__global__ void __launch_bounds__(256) k_group_select(const Node *__restrict__ nodes,
+                                                      const uint32_t *__restrict__ n_nodes, uint32_t node_cap,
+                                                      const uint32_t *__restrict__ box_off, int nbox,
+                                                      const BoxPar *__restrict__ bps, Group *__restrict__ groups,
+                                                      uint32_t *__restrict__ n_groups, uint32_t *status, DevStatus *st)
 {
-    const uint32_t nn = node_count(n_nodes, node_cap);
-    for (uint32_t n = blockIdx.x * blockDim.x + threadIdx.x; n < node_cap; n += gridDim.x * blockDim.x) {
-        uint32_t f = 0;
+    __shared__ uint32_t s_tile, s_excl, wcnt[8 * kSelItems];
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    if (tid == 0) s_tile = atomicAdd(status, 1u);
+    __syncthreads();
+    const uint32_t tile = s_tile, nn = node_count(n_nodes, node_cap);
+    const uint32_t n0 = tile * kSelTile;
+    if (n0 >= nn) return;
+    bool f[kSelItems];
+    unsigned m[kSelItems];
+#pragma unroll
+    for (uint32_t t = 0; t < kSelItems; t++) {
+        const uint32_t n = n0 + t * 256u + (uint32_t)tid;
+        f[t] = false;
         if (n < nn) {
             const Node nd = nodes[n];
             const BoxPar &bp = bps[box_of(nd.begin, box_off, nbox)];
-            if (group_cond(nd, bp)) f = (nd.parent == kNone || !group_cond(nodes[nd.parent], bp)) ? 1u : 0u;
+            if (group_cond(nd, bp)) f[t] = nd.parent == kNone || !group_cond(nodes[nd.parent], bp);
         }
-        flag[n] = f;
+        m[t] = __ballot_sync(0xffffffffu, f[t]);
+        if (lane == 0) wcnt[t * 8 + w] = __popc(m[t]);
     }
-}
-
-void launch_group_flags(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *box_off,
-                        int nbox, const BoxPar *bps, uint32_t *flag, cudaStream_t s, int nsm)
-{
-    k_group_flags<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, node_cap, box_off, nbox, bps, flag);
-    g_launches++;
-}
-
-__global__ void __launch_bounds__(256) k_group_fill(const Node *__restrict__ nodes,
-                                                    const uint32_t *__restrict__ n_nodes, uint32_t node_cap,
-                                                    const uint32_t *__restrict__ flag,
-                                                    const uint32_t *__restrict__ gidx,
-                                                    const uint32_t *__restrict__ box_off, int nbox,
-                                                    Group *__restrict__ groups)
-{
-    const uint32_t nn = node_count(n_nodes, node_cap);
-    for (uint32_t n = blockIdx.x * blockDim.x + threadIdx.x; n < nn; n += gridDim.x * blockDim.x) {
-        if (!flag[n]) continue;
+    __syncthreads();
+    if (tid < 32) {
+        const uint32_t v = wcnt[tid];  // in node order
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (tid >= o) x += y;
+        }
+        wcnt[tid] = x - v;
+        const uint32_t tot = __shfl_sync(0xffffffffu, x, 31);
+        const uint32_t excl = tile_prefix(reinterpret_cast<unsigned long long *>(status + 2), tile, tot, st);
+        if (tid == 0) {
+            s_excl = excl;
+            if (nn - n0 <= kSelTile) {  // the last tile
+                *n_groups = excl + tot;
+                st->n_nodes = *n_nodes;
+                st->n_groups = excl + tot;
+                if (*n_nodes > node_cap) atomicOr(&st->flags, ST_NODE_CAP);
+            }
+        }
+    }
+    __syncthreads();
+    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+    for (uint32_t t = 0; t < kSelItems; t++) {
+        if (!f[t]) continue;
+        const uint32_t n = n0 + t * 256u + (uint32_t)tid;
         const Node nd = nodes[n];
-        const int k = nd.lvl & 255u;
-        const int32_t h = 1 << (kMaxLevel - k);
+        const int32_t h = 1 << (kMaxLevel - (int)(nd.lvl & 255u));
         Group g;
         g.node = n;
         g.begin = nd.begin;
@@ -849,14 +876,16 @@ __global__ void __launch_bounds__(256) k_group_fill(const Node *__restrict__ nod
         g.cy = 2 * (int32_t)nd.iy + h;
         g.cz = 2 * (int32_t)nd.iz + h;
         g.hg = h;
-        groups[gidx[n]] = g;
+        groups[s_excl + wcnt[t * 8 + w] + __popc(m[t] & lt)] = g;
     }
 }
 
-void launch_group_fill(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *flag,
-                       const uint32_t *gidx, const uint32_t *box_off, int nbox, Group *groups, cudaStream_t s, int nsm)
+void launch_group_select(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *box_off, int nbox,
+                         const BoxPar *bps, Group *groups, uint32_t *n_groups, uint32_t *status, DevStatus *st,
+                         cudaStream_t s)
 {
-    k_group_fill<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, node_cap, flag, gidx, box_off, nbox, groups);
+    k_group_select<<<(node_cap + kSelTile - 1) / kSelTile, 256, 0, s>>>(nodes, n_nodes, node_cap, box_off, nbox, bps,
+                                                                        groups, n_groups, status, st);
     g_launches++;
 }
 
@@ -904,20 +933,6 @@ void launch_group_box(const Group *groups, const uint32_t *n_groups, const unsig
                       cudaStream_t s, int nsm)
 {
     k_group_box<<<nsm * 8, 256, 0, s>>>(groups, n_groups, pcell, gbox);
-    g_launches++;
-}
-
-__global__ void k_record_counts(const uint32_t *n_nodes, const uint32_t *n_groups, DevStatus *st, uint32_t node_cap)
-{
-    st->n_nodes = *n_nodes;
-    st->n_groups = n_groups ? *n_groups : 0;
-    if (*n_nodes > node_cap) atomicOr(&st->flags, ST_NODE_CAP);
-}
-
-void launch_record_counts(const uint32_t *n_nodes, const uint32_t *n_groups, DevStatus *st, uint32_t node_cap,
-                          cudaStream_t s)
-{
-    k_record_counts<<<1, 1, 0, s>>>(n_nodes, n_groups, st, node_cap);
     g_launches++;
 }
 
