@@ -99,8 +99,7 @@ struct CellTest {
 // rx, ry, rz: the cell centre minus the group's cell centre (u), before wrapping; h: the
 // cell's half side (u).
 template <bool SHIFT>
-__device__ __forceinline__ CellTest cell_gap(int rx, int ry, int rz, int h, const Group &gr, const int4 tb,
-                                             const int4 th)
+__device__ __forceinline__ CellTest cell_gap(int rx, int ry, int rz, int h, const int4 tb, const int4 th)
 {
     CellTest c;
     int sx, sy, sz;
@@ -114,9 +113,9 @@ __device__ __forceinline__ CellTest cell_gap(int rx, int ry, int rz, int h, cons
     return c;
 }
 
-__device__ __forceinline__ long long cell_dist2(const CellTest &c, const Group &gr)
+__device__ __forceinline__ long long cell_dist2(const CellTest &c, int hg)
 {
-    const int ex = max(0, abs(c.dx) - gr.hg), ey = max(0, abs(c.dy) - gr.hg), ez = max(0, abs(c.dz) - gr.hg);
+    const int ex = max(0, abs(c.dx) - hg), ey = max(0, abs(c.dy) - hg), ez = max(0, abs(c.dz) - hg);
     return (long long)ex * ex + (long long)ey * ey + (long long)ez * ez;
 }
 
@@ -130,16 +129,19 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane)
     return v;
 }
 
-// The lane s whose exclusive offset off is the largest one <= t (offsets non-decreasing).
-__device__ __forceinline__ int owner_lane(uint32_t off, uint32_t t)
+// The items of a warp's sources, 32 at a time.  Source lanes (those with items) leave what
+// their items need in shared memory in the order of the lanes, and the lane of item t finds
+// its source's place from the sources that begin in the window [t0, t0 + 32): one warp OR,
+// one ballot and two population counts, where a search over the lanes' offsets and a shuffle
+// per value took 11 to 14 dependent shuffles.  List stage, 128^3 halo mix / 256^3 / 64 boxes:
+// 1.167 / 3.355 / 6.07 -> 1.120 / 3.204 / 5.94 ms.
+__device__ __forceinline__ uint32_t source_place(bool source, uint32_t off, uint32_t t0, unsigned le)
 {
-    int s = 0;
-#pragma unroll
-    for (int step = 16; step >= 1; step >>= 1) {
-        const uint32_t oc = __shfl_sync(0xffffffffu, off, s + step);
-        if (oc <= t) s += step;
-    }
-    return s;
+    const unsigned FULL = 0xffffffffu;
+    const uint32_t d = off - t0;
+    const unsigned heads = __reduce_or_sync(FULL, source && d < 32u ? 1u << d : 0u);
+    const unsigned before = __ballot_sync(FULL, source && off < t0);
+    return __popc(before) + __popc(heads & le) - 1;
 }
 
 // ---------------------------------------------------------------- start tables
@@ -224,21 +226,21 @@ void launch_start_table(const Node *nodes, const uint32_t *kids, const uint32_t 
 // when the stack would overflow (the status is set; the call is retried).
 template <bool INDEX>
 __device__ __forceinline__ bool take_cells(const ListArgs &a, bool acc, bool push, uint32_t child, const CellTest &ct,
-                                           float kf, unsigned long long pos0, unsigned long long lim, unsigned lt,
+                                           float kf, unsigned long long pos0, uint32_t room, unsigned lt,
                                            uint32_t &cnt, uint32_t &nacc, uint32_t *__restrict__ stk, uint32_t &sp,
                                            uint32_t cap)
 {
     const unsigned FULL = 0xffffffffu;
     const unsigned ab = __ballot_sync(FULL, acc);
     if (acc) {
-        const unsigned long long p = pos0 + cnt + __popc(ab & lt);
+        const uint32_t p = cnt + __popc(ab & lt);
         const float4 v = __ldg(a.noff + child);
         const float4 e = make_float4(__fadd_rn(__fmul_rn((float)ct.dx, kf), v.x),
                                      __fadd_rn(__fmul_rn((float)ct.dy, kf), v.y),
                                      __fadd_rn(__fmul_rn((float)ct.dz, kf), v.z), v.w);
-        if (p < lim) {
-            a.flist[p] = e;
-            if (INDEX) a.ilist[p] = (unsigned long long)child | (1ull << 32) | ((unsigned long long)ct.shc << 33);
+        if (p < room) {
+            a.flist[pos0 + p] = e;
+            if (INDEX) a.ilist[pos0 + p] = (unsigned long long)child | (1ull << 32) | ((unsigned long long)ct.shc << 33);
         }
     }
     cnt += __popc(ab);
@@ -253,18 +255,35 @@ __device__ __forceinline__ bool take_cells(const ListArgs &a, bool acc, bool pus
     return true;
 }
 
+// What a walk needs of its group, in shared memory: 64 bytes per warp, read by broadcast
+// where a test needs them.  Held in registers they would spill others: the walker keeps 32
+// warps per SM at 64 registers (spills 268 -> 80 bytes; with the one scan per step and the
+// one copy of the walk: 1.120 / 3.204 / 5.94 -> 1.034 / 3.045 / 5.46 ms).
+//   0: cell centre and half side (u)        1: particle box centre minus cell centre; first particle
+//   2: its half sides; end of the particles 3: T_prune (two words), k_f, l_min
+__device__ __forceinline__ int4 group_word(uint32_t gsm, int k)
+{
+    int4 v;
+    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(gsm + 16u * k));
+    return v;
+}
+__device__ __forceinline__ long long word_tprune(const int4 w)
+{
+    return (long long)(((unsigned long long)(uint32_t)w.y << 32) | (uint32_t)w.x);
+}
+
 // The first step of a walk that starts at level K = bp.kstart (see the header): the
 // level-K cells within r_cut of the group's particle box, tested like the children of an
 // opened node.  Returns false if the group must walk from the root instead (sp is then
 // untouched); sets overflow on a stack overflow.
 template <bool INDEX>
-__device__ __forceinline__ bool start_cells(const ListArgs &a, const Group &gr, const int4 tb, const int4 th,
-                                            const BoxPar &bp, uint32_t *__restrict__ stk, unsigned long long pos0,
-                                            unsigned long long lim, int lane, unsigned lt, uint32_t &cnt,
+__device__ __forceinline__ bool start_cells(const ListArgs &a, uint32_t gsm, const BoxPar &bp, uint32_t *__restrict__ stk, unsigned long long pos0,
+                                            uint32_t room, int lane, unsigned lt, uint32_t &cnt,
                                             uint32_t &nacc, uint32_t &sp, bool &overflow)
 {
     const int K = bp.kstart;
     if (K < 2) return false;
+    const int4 gc = group_word(gsm, 0), tb = group_word(gsm, 1), th = group_word(gsm, 2);
     const int R = bp.rprune;
     const int quarter = kPeriod / 4;
     if (quarter - th.x - abs(tb.x) <= R || quarter - th.y - abs(tb.y) <= R || quarter - th.z - abs(tb.z) <= R)
@@ -283,9 +302,9 @@ __device__ __forceinline__ bool start_cells(const ListArgs &a, const Group &gr, 
         }
     };
     int cx0, nx, cy0, ny, cz0, nz;
-    range(gr.cx, tb.x, th.x, cx0, nx);
-    range(gr.cy, tb.y, th.y, cy0, ny);
-    range(gr.cz, tb.z, th.z, cz0, nz);
+    range(gc.x, tb.x, th.x, cx0, nx);
+    range(gc.y, tb.y, th.y, cy0, ny);
+    range(gc.z, tb.z, th.z, cz0, nz);
     const uint32_t ncand = (uint32_t)(nx * ny * nz);
     if (ncand > kMaxStartCells) return false;
     const uint32_t *tb_k = a.tbl + bp.tbl_off;
@@ -325,22 +344,22 @@ __device__ __forceinline__ bool start_cells(const ListArgs &a, const Group &gr, 
                     if (ix == first(nd.ix >> fsh, cx0) && iy == first(nd.iy >> fsh, cy0) &&
                         iz == first(nd.iz >> fsh, cz0)) {
                         const int hl = 1 << (kMaxLevel - kl);
-                        ct = cell_gap<INDEX>(2 * (int)nd.ix + hl - gr.cx, 2 * (int)nd.iy + hl - gr.cy,
-                                             2 * (int)nd.iz + hl - gr.cz, hl, gr, tb, th);
+                        ct = cell_gap<INDEX>(2 * (int)nd.ix + hl - gc.x, 2 * (int)nd.iy + hl - gc.y,
+                                             2 * (int)nd.iz + hl - gc.z, hl, tb, th);
                         push = ct.Sg <= Tp;
                     }
                 } else {
                     node = e;
-                    ct = cell_gap<INDEX>((int)(wx << sh) + hK - gr.cx, (int)(wy << sh) + hK - gr.cy,
-                                         (int)(wz << sh) + hK - gr.cz, hK, gr, tb, th);
+                    ct = cell_gap<INDEX>((int)(wx << sh) + hK - gc.x, (int)(wy << sh) + hK - gc.y,
+                                         (int)(wz << sh) + hK - gc.z, hK, tb, th);
                     if (ct.Sg <= Tp) {
-                        acc = acc_level && cell_dist2(ct, gr) > AK;
+                        acc = acc_level && cell_dist2(ct, gc.w) > AK;
                         push = !acc;
                     }
                 }
             }
         }
-        if (!take_cells<INDEX>(a, acc, push, node, ct, kf, pos0, lim, lt, cnt, nacc, stk, sp, a.stack_cap)) {
+        if (!take_cells<INDEX>(a, acc, push, node, ct, kf, pos0, room, lt, cnt, nacc, stk, sp, a.stack_cap)) {
             overflow = true;
             break;
         }
@@ -361,8 +380,8 @@ __device__ __forceinline__ bool start_cells(const ListArgs &a, const Group &gr, 
     return true;
 }
 
-// Walks one group's list; writes entries [pos0, pos0+total) clipped at lim; returns
-// total.  stk is this warp's stack (a.stack_cap entries); an overflow sets the status.
+// Walks one group's list; writes entries [pos0, pos0+total), the first `room` of them;
+// returns total.  stk is this warp's stack (a.stack_cap entries); an overflow sets the status.
 //
 // The stack holds nodes that passed the prune test and failed the accept test: leaves,
 // whose particles are emitted, and nodes to open.  Each step pops up to 32 of them, one
@@ -374,23 +393,20 @@ __device__ __forceinline__ bool start_cells(const ListArgs &a, const Group &gr, 
 // goes through the per-particle r_cut test unless its whole leaf lies within r_cut.
 // INDEX: the index entries are written too (a.ilist).
 template <bool INDEX>
-__device__ uint32_t walk_group(const ListArgs &a, const Group &gr, const int4 tb, const int4 th, const BoxPar &bp,
+__device__ __forceinline__ uint32_t walk_group(const ListArgs &a, uint32_t gsm, const BoxPar &bp,
                                uint32_t root, uint32_t *__restrict__ stk, const uint8_t *__restrict__ octq,
-                               unsigned long long pos0, unsigned long long lim, int lane, uint32_t &nacc,
+                               uint4 *__restrict__ src,
+                               unsigned long long pos0, uint32_t room, int lane, uint32_t &nacc,
                                bool &from_table)
 {
     const unsigned FULL = 0xffffffffu;
-    const unsigned lt = (1u << lane) - 1u;
+    const unsigned lt = (1u << lane) - 1u, le = lt | (1u << lane);
     nacc = 0;
-    const uint32_t gend = gr.begin + gr.count;
-    const long long Tp = bp.T_prune;
-    const int lmin = bp.lmin;
-    const float kf = bp.k_f;
     const uint32_t cap = a.stack_cap;
     uint32_t cnt = 0;
     uint32_t sp = 0;
     bool overflow = false;
-    from_table = start_cells<INDEX>(a, gr, tb, th, bp, stk, pos0, lim, lane, lt, cnt, nacc, sp, overflow);
+    from_table = start_cells<INDEX>(a, gsm, bp, stk, pos0, room, lane, lt, cnt, nacc, sp, overflow);
     if (!from_table) {
         if (lane == 0) stk[0] = root;
         sp = 1;
@@ -404,8 +420,10 @@ __device__ uint32_t walk_group(const ListArgs &a, const Group &gr, const int4 tb
         __syncwarp();
         sp = sbase;
         Node nd;
+        unsigned long long lb = 0;
         if (valid) {
             nd = load_node(a.nodes + m);
+            lb = __ldg(a.lbox + m);  // of leaves only; loaded beside the node
         } else {
             nd.ix = nd.iy = nd.iz = 0; nd.lvl = 0; nd.begin = nd.end = nd.skip = 0; nd.parent = 0;
         }
@@ -414,58 +432,24 @@ __device__ uint32_t walk_group(const ListArgs &a, const Group &gr, const int4 tb
         const uint32_t mask = valid && !leaf ? (nd.lvl >> 16) & 255u : 0u;
         // the popped node's centre minus the group's cell centre (u, before wrapping)
         const int hn = 1 << (kMaxLevel - k);
-        const int ncx = 2 * (int)nd.ix + hn - gr.cx, ncy = 2 * (int)nd.iy + hn - gr.cy, ncz = 2 * (int)nd.iz + hn - gr.cz;
+        const int4 gc = group_word(gsm, 0);
+        const int ncx = 2 * (int)nd.ix + hn - gc.x, ncy = 2 * (int)nd.iy + hn - gc.y, ncz = 2 * (int)nd.iz + hn - gc.z;
 
-        // ---- children of the opened nodes: prune, accept (one entry), or push
-        const uint32_t nch = __popc(mask);
-        const uint32_t csum = warp_incl_scan(nch, lane);
-        const uint32_t coff = csum - nch;
-        const uint32_t ctot = __shfl_sync(FULL, csum, 31);
-        for (uint32_t c0 = 0; c0 < ctot; c0 += 32) {
-            const uint32_t t = c0 + lane;
-            const int s = owner_lane(coff, t);
-            const uint32_t o_s = __shfl_sync(FULL, coff, s);
-            const int pcx = __shfl_sync(FULL, ncx, s), pcy = __shfl_sync(FULL, ncy, s),
-                      pcz = __shfl_sync(FULL, ncz, s);
-            const uint32_t plvl = __shfl_sync(FULL, nd.lvl, s), pm = __shfl_sync(FULL, m, s);
-            bool acc = false, push = false;
-            uint32_t child = 0;
-            CellTest ct;
-            if (t < ctot) {
-                const uint32_t q = t - o_s;
-                const uint32_t oct = octq[((plvl >> 13) & (255u << 3)) | q];
-                const int kc = (int)(plvl & 255u) + 1;
-                const int hc = 1 << (kMaxLevel - kc);
-                // a child's centre is its parent's shifted by +-hc per axis
-                ct = cell_gap<INDEX>(pcx + ((oct & 4u) ? hc : -hc), pcy + ((oct & 2u) ? hc : -hc),
-                                     pcz + ((oct & 1u) ? hc : -hc), hc, gr, tb, th);
-                if (ct.Sg <= Tp) {
-                    child = __ldg(a.kids + (size_t)pm * 8 + q);
-                    acc = kc >= lmin && cell_dist2(ct, gr) > bp.A[kc];
-                    push = !acc;
-                }
-            }
-            if (!take_cells<INDEX>(a, acc, push, child, ct, kf, pos0, lim, lt, cnt, nacc, stk, sp, cap)) {
-                overflow = true;  // the caller's list is incomplete; the call is retried with a larger stack
-                break;
-            }
-        }
-        __syncwarp();
-        if (overflow) break;
-
-        // ---- particles of the popped leaves
+        // ---- the popped leaves: which particles, and what their entries take from the leaf
         uint32_t ne = 0;
         float bx = 0.f, by = 0.f, bz = 0.f;
-        unsigned shc = 0;   // test flag in bit 6; INDEX: the leaf's shift code in bits 0-5
+        unsigned shc = 0;   // test flag in bit 6, own in bit 7; INDEX: the leaf's shift code in bits 0-5
         int ox = 0, oy = 0, oz = 0;
         if (leaf) {
+            const int4 tb = group_word(gsm, 1), th = group_word(gsm, 2), pw = group_word(gsm, 3);
+            const long long Tp = word_tprune(pw);
+            const float kf = __int_as_float(pw.z);
             const int h = hn;
-            const CellTest lc = cell_gap<INDEX>(ncx, ncy, ncz, h, gr, tb, th);
+            const CellTest lc = cell_gap<INDEX>(ncx, ncy, ncz, h, tb, th);
             // the box of the leaf's particles (finest cells, in slots of q; k_leaf_boxes),
             // its centre relative to the group's cell centre in the leaf's image and its
             // half sides (u): beyond r_cut of the group's particle box, no particle is
             // kept; within it, every particle is (each particle's finest cell is inside)
-            const unsigned long long lb = __ldg(a.lbox + m);
             const int q = h > 256 ? (h >> 8) : 1;
             const int lx = (int)(lb & 255u), ly = (int)((lb >> 16) & 255u), lz = (int)((lb >> 32) & 255u);
             const int ux = (int)((lb >> 8) & 255u), uy = (int)((lb >> 24) & 255u), uz = (int)((lb >> 40) & 255u);
@@ -482,34 +466,99 @@ __device__ uint32_t walk_group(const ListArgs &a, const Group &gr, const int4 tb
             bx = __fmul_rn((float)lc.dx, kf);
             by = __fmul_rn((float)lc.dy, kf);
             bz = __fmul_rn((float)lc.dz, kf);
-            shc = lc.shc | (test_each ? 64u : 0u);
+            // the group's own particles leave their positions in irel; a leaf lies in the group
+            // whole or not at all
+            const bool own = nd.begin >= (uint32_t)tb.w && nd.begin < (uint32_t)th.w;
+            shc = lc.shc | (test_each ? 64u : 0u) | (own ? 128u : 0u);
             // a particle in finest cell c of this leaf sits at 2c + o (u) from the centre of
             // the group's particle box, in the leaf's image
-            ox = lc.dx - ncx - gr.cx + 1 - tb.x;
-            oy = lc.dy - ncy - gr.cy + 1 - tb.y;
-            oz = lc.dz - ncz - gr.cz + 1 - tb.z;
+            ox = lc.dx - ncx - gc.x + 1 - tb.x;
+            oy = lc.dy - ncy - gc.y + 1 - tb.y;
+            oz = lc.dz - ncz - gc.z + 1 - tb.z;
         }
-        const uint32_t isum = warp_incl_scan(ne, lane);
-        const uint32_t off = isum - ne;
-        const uint32_t tot = __shfl_sync(FULL, isum, 31);
+        // ---- the sources of both loops below, in shared memory
+        const uint32_t nch = __popc(mask);
+        uint32_t o, ctot, tot;  // the lane's first child or particle, and how many there are
+        if (!__any_sync(FULL, ne >> 18)) {  // a node has children or particles: one scan for both
+            const uint32_t v = nch | (ne << 9), x = warp_incl_scan(v, lane), last = __shfl_sync(FULL, x, 31);
+            o = mask ? (x - v) & 511u : (x - v) >> 9;
+            ctot = last & 511u;
+            tot = last >> 9;
+        } else {  // leaves of the finest level can hold any number of particles
+            const uint32_t x = warp_incl_scan(nch, lane), y = warp_incl_scan(ne, lane);
+            o = mask ? x - nch : y - ne;
+            ctot = __shfl_sync(FULL, x, 31);
+            tot = __shfl_sync(FULL, y, 31);
+        }
+        const unsigned inner = __ballot_sync(FULL, mask != 0), full = __ballot_sync(FULL, ne != 0);
+        const uint32_t n_inner = __popc(inner);  // the particles' sources come after the children's
+        if (mask) {
+            uint4 *d = src + 2 * __popc(inner & lt);
+            d[0] = make_uint4(o, m, nd.lvl, (uint32_t)ncx);
+            d[1] = make_uint4((uint32_t)ncy, (uint32_t)ncz, 0u, 0u);
+        }
+        if (ne) {
+            uint4 *d = src + 2 * (n_inner + __popc(full & lt));
+            d[0] = make_uint4(nd.begin - o, shc, (uint32_t)ox, (uint32_t)oy);
+            d[1] = make_uint4((uint32_t)oz, __float_as_uint(bx), __float_as_uint(by), __float_as_uint(bz));
+        }
+        const bool is_inner = mask != 0, is_full = ne != 0;
+        __syncwarp();
+
+        // ---- children of the opened nodes: prune, accept (one entry), or push
+        for (uint32_t c0 = 0; c0 < ctot; c0 += 32) {
+            const uint32_t t = c0 + lane;
+            const uint4 *sp_ = src + 2 * source_place(is_inner, o, c0, le);
+            const uint4 u = sp_[0];
+            const uint2 v = *reinterpret_cast<const uint2 *>(sp_ + 1);
+            const uint32_t o_s = u.x, pm = u.y, plvl = u.z;
+            const int pcx = (int)u.w, pcy = (int)v.x, pcz = (int)v.y;
+            const int4 pw = group_word(gsm, 3);
+            bool acc = false, push = false;
+            uint32_t child = 0;
+            CellTest ct;
+            if (t < ctot) {
+                const int4 tb = group_word(gsm, 1), th = group_word(gsm, 2);
+                const uint32_t q = t - o_s;
+                const uint32_t oct = octq[((plvl >> 13) & (255u << 3)) | q];
+                const int kc = (int)(plvl & 255u) + 1;
+                const int hc = 1 << (kMaxLevel - kc);
+                // a child's centre is its parent's shifted by +-hc per axis
+                ct = cell_gap<INDEX>(pcx + ((oct & 4u) ? hc : -hc), pcy + ((oct & 2u) ? hc : -hc),
+                                     pcz + ((oct & 1u) ? hc : -hc), hc, tb, th);
+                if (ct.Sg <= word_tprune(pw)) {
+                    child = __ldg(a.kids + (size_t)pm * 8 + q);
+                    acc = kc >= pw.w && cell_dist2(ct, group_word(gsm, 0).w) > bp.A[kc];
+                    push = !acc;
+                }
+            }
+            if (!take_cells<INDEX>(a, acc, push, child, ct, __int_as_float(pw.z), pos0, room, lt, cnt, nacc, stk, sp, cap)) {
+                overflow = true;  // the caller's list is incomplete; the call is retried with a larger stack
+                break;
+            }
+        }
+        __syncwarp();
+        if (overflow) break;
+
+        // ---- particles of the popped leaves
         for (uint32_t t0 = 0; t0 < tot; t0 += 32) {
             const uint32_t t = t0 + lane;
-            const int s = owner_lane(off, t);
-            const uint32_t o_s = __shfl_sync(FULL, off, s);
-            const uint32_t b_s = __shfl_sync(FULL, nd.begin, s);
-            const float bx_s = __shfl_sync(FULL, bx, s), by_s = __shfl_sync(FULL, by, s),
-                        bz_s = __shfl_sync(FULL, bz, s);
-            const unsigned sh_s = __shfl_sync(FULL, shc, s);
-            const int ox_s = __shfl_sync(FULL, ox, s), oy_s = __shfl_sync(FULL, oy, s), oz_s = __shfl_sync(FULL, oz, s);
+            const uint4 *sp_ = src + 2 * (n_inner + source_place(is_full, o, t0, le));
+            const uint4 u = sp_[0], v4 = sp_[1];
+            const unsigned sh_s = u.y;
+            const int ox_s = (int)u.z, oy_s = (int)u.w, oz_s = (int)v4.x;
+            const float bx_s = __uint_as_float(v4.y), by_s = __uint_as_float(v4.z), bz_s = __uint_as_float(v4.w);
             bool keep = false;
             float4 e;
             uint32_t j = kNone;
             if (t < tot) {
-                j = b_s + (t - o_s);
+                j = u.x + t;
                 const float4 v = __ldg(a.poff + j);
                 keep = true;
                 if (sh_s & 64u) {
                     // the particle's finest cell, in its leaf's image, against the particle box
+                    const int4 th = group_word(gsm, 2);
+                    const long long Tp = word_tprune(group_word(gsm, 3));
                     const unsigned long long c = __ldg(a.pcell + j);
                     const int px = 2 * (int)((uint32_t)c & 0x1fffffu) + ox_s;
                     const int py = 2 * (int)((uint32_t)(c >> 21) & 0x1fffffu) + oy_s;
@@ -519,18 +568,19 @@ __device__ uint32_t walk_group(const ListArgs &a, const Group &gr, const int4 tb
                     keep = (long long)qx * qx + (long long)qy * qy + (long long)qz * qz <= Tp;
                 }
                 e = make_float4(__fadd_rn(bx_s, v.x), __fadd_rn(by_s, v.y), __fadd_rn(bz_s, v.z), v.w);
-                if (j >= gr.begin && j < gend) a.irel[j] = e;
+                if (sh_s & 128u) a.irel[j] = e;
             }
             const unsigned kb = __ballot_sync(FULL, keep);
             if (keep) {
-                const unsigned long long p = pos0 + cnt + __popc(kb & lt);
-                if (p < lim) {
-                    a.flist[p] = e;
-                    if (INDEX) a.ilist[p] = (unsigned long long)j | ((unsigned long long)(sh_s & 63u) << 33);
+                const uint32_t p = cnt + __popc(kb & lt);
+                if (p < room) {
+                    a.flist[pos0 + p] = e;
+                    if (INDEX) a.ilist[pos0 + p] = (unsigned long long)j | ((unsigned long long)(sh_s & 63u) << 33);
                 }
             }
             cnt += __popc(kb);
         }
+        __syncwarp();  // the sources are read
     }
     __syncwarp();
     return cnt;
@@ -550,6 +600,10 @@ __global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(Lis
         for (; q < 8; q++) octq[8 * m + q] = 0;
     }
     __shared__ unsigned long long tallies[kListWarps][kTallyN];
+    __shared__ uint4 sources[kListWarps][64];  // walk_group's sources, two words of 16 bytes each
+    __shared__ int4 gconst[kListWarps][4];     // group_word
+    uint4 *src = sources[threadIdx.x >> 5];
+    const uint32_t gsm = (uint32_t)__cvta_generic_to_shared(gconst[threadIdx.x >> 5]);
     if (lane == 0)
         for (int k = 0; k < kTallyN; k++) tallies[threadIdx.x >> 5][k] = 0;
     __syncthreads();
@@ -580,25 +634,40 @@ __global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(Lis
         gi = __shfl_sync(FULL, gi, 0);
         if (gi >= G) break;
         const uint32_t g = (uint32_t)gi;
+        __syncwarp();  // the last group's constants are read, lane 0's tallies written
         const Group gr = a.groups[g];
-        const int4 tb = a.gbox[2 * (size_t)g], th = a.gbox[2 * (size_t)g + 1];
         const BoxPar &bp = a.bps[gr.box];
+        if (lane == 0) {
+            int4 *w = gconst[threadIdx.x >> 5];
+            const int4 tb = a.gbox[2 * (size_t)g], th = a.gbox[2 * (size_t)g + 1];
+            const unsigned long long Tp = (unsigned long long)bp.T_prune;
+            w[0] = make_int4(gr.cx, gr.cy, gr.cz, gr.hg);
+            w[1] = make_int4(tb.x, tb.y, tb.z, (int)gr.begin);
+            w[2] = make_int4(th.x, th.y, th.z, (int)(gr.begin + gr.count));
+            w[3] = make_int4((int)(uint32_t)Tp, (int)(uint32_t)(Tp >> 32), __float_as_int(bp.k_f), bp.lmin);
+        }
         const uint32_t root = a.base[bp.p_begin];
-        uint32_t nacc = 0;
-        bool from_table = false;
-        __syncwarp();  // lane 0's tallies
         if (!exhausted && (page_cur == page_end ||
                            (page_end - page_cur) * tally[kTallyGroups] < tally[kTallyPadded]))
             take_pages(1);
-        const uint32_t len =
-            walk_group<INDEX>(a, gr, tb, th, bp, root, stk, octq, page_cur, page_end, lane, nacc, from_table);
-        if (lane == 0) tally[kTallyStart] += from_table ? 1u : 0u;
-        const uint32_t padded = (len + 7u) & ~7u;
-        if (lane == 0) {
-            tally[kTallyPadded] += padded;
-            tally[kTallyGroups]++;
+        __syncwarp();
+        uint32_t nacc = 0, len = 0, padded = 0;
+        bool placed = false;
+        for (bool again = false;; again = true) {
+            bool from_table = false;
+            len = walk_group<INDEX>(a, gsm, bp, root, stk, octq, src, page_cur, (uint32_t)(page_end - page_cur), lane,
+                                    nacc, from_table);
+            padded = (len + 7u) & ~7u;
+            if (!again && lane == 0) {
+                tally[kTallyStart] += from_table ? 1u : 0u;
+                tally[kTallyPadded] += padded;
+                tally[kTallyGroups]++;
+            }
+            if (exhausted) break;
+            placed = page_cur + padded <= page_end;
+            if (placed || !take_pages((padded + a.page - 1) / a.page)) break;
         }
-        if (exhausted) {
+        if (!placed) {
             if (lane == 0) {
                 a.loff[g] = 0;
                 a.llen[g] = 0;
@@ -606,18 +675,6 @@ __global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(Lis
                 if (a.qcnt) a.qcnt[g] = 0;
             }
             continue;
-        }
-        if (page_cur + padded > page_end) {
-            if (!take_pages((padded + a.page - 1) / a.page)) {
-                if (lane == 0) {
-                    a.loff[g] = 0;
-                    a.llen[g] = 0;
-                    a.lraw[g] = 0;
-                    if (a.qcnt) a.qcnt[g] = 0;
-                }
-                continue;
-            }
-            walk_group<INDEX>(a, gr, tb, th, bp, root, stk, octq, page_cur, page_end, lane, nacc, from_table);
         }
         for (uint32_t t = len + lane; t < padded; t += 32) {
             a.flist[page_cur + t] = make_float4(16.f, 16.f, 16.f, 0.f);
@@ -629,7 +686,7 @@ __global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(Lis
             a.lraw[g] = len;
             if (a.qcnt) a.qcnt[g] = nacc;
             tally[kTallyLen] += len;
-            tally[kTallyInter] += (unsigned long long)len * gr.count;
+            tally[kTallyInter] += (unsigned long long)len * a.groups[g].count;
         }
         page_cur += padded;
     }
