@@ -81,8 +81,13 @@ constexpr int kRsWarps = kRsThreads / 32;
 #ifndef GREEM_RS_MINB
 #define GREEM_RS_MINB 3
 #endif
-constexpr int kRsItems = GREEM_RS_ITEMS;
-constexpr int kRsTile = kRsThreads * kRsItems;  // pairs per tile
+constexpr int kRsItems = GREEM_RS_ITEMS;        // pairs per thread
+// the same when the tiles are few: a pass then takes as long as one tile's chain of rankings
+// (sort stage at 12 / 4 / 3 / 2 pairs per thread: 4 k particles 0.045 / 0.033 / 0.031 / 0.030
+// ms, 32 k 0.047 / 0.037 / 0.035 / 0.037, 100 k 0.053 / 0.045 / 0.043 / 0.049, 300 k 0.063 /
+// 0.063 / 0.070 / -)
+constexpr int kRsItemsSmall = 3;
+constexpr uint32_t kRsSmallMax = 200000;        // pairs
 constexpr int kRsMaxPasses = 10;                // key digits + up to 2 box digits
 constexpr int kRsLowBits = 27;                  // bits left to phase B: levels 13-21
 constexpr int kRsKeyPasses = 5;                 // 8-bit digits over the top 36 bits
@@ -92,9 +97,10 @@ constexpr int kRunThreads = 256;
 constexpr size_t kRunSmem = (size_t)kRunCap * (sizeof(uint64_t) + sizeof(uint32_t));
 constexpr int kRsLook = 8;                      // predecessors loaded at once in the look-back
 constexpr unsigned long long kRsAgg = 1ull << 62, kRsPrefix = 2ull << 62, kRsValue = (1ull << 62) - 1;
-constexpr size_t kRsSmem = (size_t)kRsTile * (sizeof(uint64_t) + sizeof(uint32_t));
+constexpr size_t rs_smem(int items) { return (size_t)kRsThreads * items * (sizeof(uint64_t) + sizeof(uint32_t)); }
 
-static inline uint32_t rs_tiles(uint32_t n) { return (n + kRsTile - 1) / kRsTile; }
+static inline int rs_items(uint32_t n) { return n <= kRsSmallMax ? kRsItemsSmall : kRsItems; }
+static inline uint32_t rs_tiles(uint32_t n) { const uint32_t t = kRsThreads * rs_items(n); return (n + t - 1) / t; }
 
 // u32 words: [passes][256] digit counts, [passes] tickets, then phase B's counts of long and
 // middle runs and their work counters
@@ -184,7 +190,7 @@ void launch_keys(const double *pos, uint32_t N, const uint32_t *box_off, int nbo
     g_launches++;
 }
 
-template <int SRC>
+template <int SRC, int ITEMS>
 __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const uint64_t *__restrict__ kin,
                                                              const uint32_t *__restrict__ vin,
                                                              uint64_t *__restrict__ kout, uint32_t *__restrict__ vout,
@@ -193,9 +199,10 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
                                                              const uint32_t *__restrict__ box_off, int nbox,
                                                              DevStatus *st)
 {
-    extern __shared__ __align__(16) unsigned char rs_smem[];
-    uint64_t *sk = reinterpret_cast<uint64_t *>(rs_smem);
-    uint32_t *sv = reinterpret_cast<uint32_t *>(rs_smem + (size_t)kRsTile * sizeof(uint64_t));
+    constexpr uint32_t TILE = kRsThreads * ITEMS;  // pairs per tile
+    extern __shared__ __align__(16) unsigned char rs_buf[];
+    uint64_t *sk = reinterpret_cast<uint64_t *>(rs_buf);
+    uint32_t *sv = reinterpret_cast<uint32_t *>(rs_buf + (size_t)TILE * sizeof(uint64_t));
     __shared__ uint32_t wcnt[kRsWarps][256];
     __shared__ uint32_t lstart[256];
     __shared__ uint32_t gbase[256];
@@ -207,19 +214,19 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
     __syncthreads();
     const uint32_t tile = s_tile;
 
-    uint64_t k[kRsItems];
-    uint32_t v[kRsItems], rk[kRsItems];
-    const uint32_t wbase = tile * kRsTile + w * (kRsItems * 32);
+    uint64_t k[ITEMS];
+    uint32_t v[ITEMS], rk[ITEMS];
+    const uint32_t wbase = tile * TILE + w * (ITEMS * 32);
     const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
-    for (int t = 0; t < kRsItems; t++) {
+    for (int t = 0; t < ITEMS; t++) {
         const uint32_t i = wbase + t * 32 + lane;
         k[t] = i < n ? kin[i] : 0ull;
         v[t] = i < n ? (vin ? vin[i] : i) : 0u;
     }
     // rank within the warp's run of pairs, in input order
 #pragma unroll
-    for (int t = 0; t < kRsItems; t++) {
+    for (int t = 0; t < ITEMS; t++) {
         const bool valid = wbase + t * 32 + lane < n;
         const uint32_t d = valid ? rs_digit<SRC>(k[t], v[t], shift, box_off, nbox) : 256u;
         const unsigned peers = digit_peers(d);
@@ -271,7 +278,7 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
     const uint32_t dstart = db + dx - dcount;
     __syncthreads();
 #pragma unroll
-    for (int t = 0; t < kRsItems; t++) {
+    for (int t = 0; t < ITEMS; t++) {
         if (rk[t] != 0xffffffffu) {
             const uint32_t d = rs_digit<SRC>(k[t], v[t], shift, box_off, nbox);
             const uint32_t lp = lstart[d] + wcnt[w][d] + rk[t];
@@ -325,8 +332,8 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
         gbase[tid] = dstart + (uint32_t)excl;
     }
     __syncthreads();
-    const uint32_t tbase = tile * kRsTile;
-    const uint32_t cnt = min((uint32_t)kRsTile, n - tbase);
+    const uint32_t tbase = tile * TILE;
+    const uint32_t cnt = min(TILE, n - tbase);
     for (uint32_t j = tid; j < cnt; j += kRsThreads) {
         const uint64_t kk = sk[j];
         const uint32_t vv = sv[j];
@@ -607,8 +614,10 @@ void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t
     static std::atomic<bool> attr_set[kMaxDevices];
     const int dev = current_device_index();
     if (dev < 0 || !attr_set[dev].load()) {
-        cudaFuncSetAttribute(k_rs_onesweep<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRsSmem);
-        cudaFuncSetAttribute(k_rs_onesweep<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRsSmem);
+        cudaFuncSetAttribute(k_rs_onesweep<0, kRsItems>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)rs_smem(kRsItems));
+        cudaFuncSetAttribute(k_rs_onesweep<1, kRsItems>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)rs_smem(kRsItems));
         cudaFuncSetAttribute(k_runs_rest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunSmem);
         if (dev >= 0) attr_set[dev].store(true);
     }
@@ -623,11 +632,10 @@ void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t
         const uint32_t *ds = hist + p * 256;
         uint32_t *tk = hist + kRsMaxPasses * 256 + p;
         unsigned long long *sw = status + (size_t)p * ntile * 256;
-        if (boxp) {
-            k_rs_onesweep<1><<<ntile, kRsThreads, kRsSmem, s>>>(ki, vi, ko, vo, n, shift, ds, sw, tk, box_off, nbox, st);
-        } else {
-            k_rs_onesweep<0><<<ntile, kRsThreads, kRsSmem, s>>>(ki, vi, ko, vo, n, shift, ds, sw, tk, box_off, nbox, st);
-        }
+        const bool small = rs_items(n) == kRsItemsSmall;
+        const auto kern = boxp ? (small ? k_rs_onesweep<1, kRsItemsSmall> : k_rs_onesweep<1, kRsItems>)
+                               : (small ? k_rs_onesweep<0, kRsItemsSmall> : k_rs_onesweep<0, kRsItems>);
+        kern<<<ntile, kRsThreads, rs_smem(rs_items(n)), s>>>(ki, vi, ko, vo, n, shift, ds, sw, tk, box_off, nbox, st);
         g_launches++;
         // ping-pong
         uint64_t *kt = ki;

@@ -10,8 +10,8 @@
 namespace greem {
 
 constexpr int kScanThreads = 256;
-constexpr int kScanItems = 8;
-constexpr int kScanTile = kScanThreads * kScanItems;  // 2048
+constexpr int kScanItems = 16;  // 8 in single words: tree stage of 16.8 M particles 1.646 ms, 16 by 16-byte loads 1.535
+constexpr int kScanTile = kScanThreads * kScanItems;
 
 static inline size_t ceil_div(size_t a, size_t b) { return (a + b - 1) / b; }
 
@@ -61,12 +61,22 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t *in, size_
     const size_t base = tbase + (size_t)threadIdx.x * kScanItems;
     uint32_t v[kScanItems];
     uint32_t s = 0;
+    const bool whole = base + kScanItems <= n;  // 16-byte loads and stores (in and out are 16-byte aligned)
+    if (whole) {
 #pragma unroll
-    for (int t = 0; t < kScanItems; t++) {
-        size_t i = base + t;
-        v[t] = i < n ? in[i] : 0;
-        s += v[t];
+        for (int t = 0; t < kScanItems; t += 4) {
+            const uint4 u = *reinterpret_cast<const uint4 *>(in + base + t);
+            v[t] = u.x;
+            v[t + 1] = u.y;
+            v[t + 2] = u.z;
+            v[t + 3] = u.w;
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < kScanItems; t++) v[t] = base + t < n ? in[base + t] : 0;
     }
+#pragma unroll
+    for (int t = 0; t < kScanItems; t++) s += v[t];
     uint32_t tot;
     uint32_t run = block_exclusive_scan(s, &tot);
     if (threadIdx.x < 32) {
@@ -77,9 +87,18 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t *in, size_
     run += s_excl;
 #pragma unroll
     for (int t = 0; t < kScanItems; t++) {
-        size_t i = base + t;
-        if (i < n) out[i] = run;
-        run += v[t];
+        const uint32_t x = v[t];
+        v[t] = run;
+        run += x;
+    }
+    if (whole) {
+#pragma unroll
+        for (int t = 0; t < kScanItems; t += 4)
+            *reinterpret_cast<uint4 *>(out + base + t) = make_uint4(v[t], v[t + 1], v[t + 2], v[t + 3]);
+    } else {
+#pragma unroll
+        for (int t = 0; t < kScanItems; t++)
+            if (base + t < n) out[base + t] = v[t];
     }
     // the thread holding element n-1 also writes the total at out[n]
     if (base < n && n - 1 < base + kScanItems) out[n] = run;

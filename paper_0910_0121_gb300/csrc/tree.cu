@@ -418,20 +418,19 @@ __global__ void __launch_bounds__(256) k_moments_leaf_tiled(const Node *__restri
 }
 
 // The raw moments of internal node p: its children's, in child order.
-__device__ __forceinline__ void sum_children(uint32_t p, const uint32_t *__restrict__ kids, Dbl4 *raw)
+__device__ __forceinline__ void sum_children(uint32_t p, const uint32_t (&kk)[8], Dbl4 *raw)
 {
-    const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
-    const uint4 k0 = kp[0], k1 = kp[1];
-    const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-    Dbl4 a = make_dbl4(0.0, 0.0, 0.0, 0.0);
+    Dbl4 a = make_dbl4(0.0, 0.0, 0.0, 0.0), r[8];
+#pragma unroll
+    for (int q = 0; q < 8; q++)  // all loads before the first sum
+        r[q] = kk[q] != kNone ? raw[kk[q]] : a;
 #pragma unroll
     for (int q = 0; q < 8; q++) {
         if (kk[q] == kNone) break;
-        const Dbl4 r = raw[kk[q]];
-        a.x += r.x;
-        a.y += r.y;
-        a.z += r.z;
-        a.w += r.w;
+        a.x += r[q].x;
+        a.y += r[q].y;
+        a.z += r[q].z;
+        a.w += r[q].w;
     }
     raw[p] = a;
 }
@@ -441,8 +440,13 @@ __global__ void __launch_bounds__(256) k_moments_level(int level, const uint32_t
                                                        const uint32_t *__restrict__ kids, Dbl4 *raw)
 {
     const uint32_t b = lvl[32 + level], e = b + lvl[level];
-    for (uint32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x)
-        sum_children(inodes[i], kids, raw);
+    for (uint32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x) {
+        const uint32_t p = inodes[i];
+        const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
+        const uint4 k0 = kp[0], k1 = kp[1];
+        const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+        sum_children(p, kk, raw);
+    }
 }
 
 // Every level in one launch, for smaller trees: one cluster of blocks goes through the
@@ -450,11 +454,14 @@ __global__ void __launch_bounds__(256) k_moments_level(int level, const uint32_t
 // 21 launches of the form above cost more than their sums).  Its 16 blocks have a tenth of
 // the GPU's FP64 rate, which sets the line kClusterMax.
 constexpr int kClusterCtas = 16;
-constexpr int kClusterThreads = 512;
+constexpr int kClusterThreads = 256;  // 512: tree stage of 100 k particles 0.113 ms, 256: 0.098, 128: 0.092 (300 k: the same)
 
+// f(p, level, kids of p) for every internal node.  A thread loads its first node of a level
+// and its child table before the barrier that ends the level below: neither depends on it,
+// and the level's chain of memory round trips shortens to the children's moments.
 template <class F>
 __device__ __forceinline__ void cluster_levels(const uint32_t *__restrict__ lvl, const uint32_t *__restrict__ inodes,
-                                               F &&f)
+                                               const uint32_t *__restrict__ kids, F &&f)
 {
     const auto cl = cooperative_groups::this_cluster();
     __shared__ uint32_t cnt[32], start[32];
@@ -464,10 +471,29 @@ __device__ __forceinline__ void cluster_levels(const uint32_t *__restrict__ lvl,
     }
     __syncthreads();
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    for (int level = kMaxLevel - 1; level >= 0; level--) {
-        const uint32_t c = cnt[level];
-        if (!c) continue;  // the same in every block
-        for (uint32_t i = t; i < c; i += nt) f(inodes[start[level] + i], level);
+    auto below = [&](int level) {
+        do level--;
+        while (level >= 0 && cnt[level] == 0);
+        return level;  // the same in every block
+    };
+    uint32_t p = 0;
+    uint4 k0 = make_uint4(0, 0, 0, 0), k1 = k0;
+    auto load = [&](int level, uint32_t i) {
+        p = inodes[start[level] + i];
+        const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
+        k0 = kp[0];
+        k1 = kp[1];
+    };
+    int level = below(kMaxLevel);
+    if (level >= 0 && t < cnt[level]) load(level, t);
+    while (level >= 0) {
+        for (uint32_t i = t; i < cnt[level]; i += nt) {
+            if (i != t) load(level, i);
+            const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+            f(p, level, kk);
+        }
+        level = below(level);
+        if (level >= 0 && t < cnt[level]) load(level, t);
         cl.sync();
     }
 }
@@ -476,7 +502,7 @@ __global__ void __launch_bounds__(kClusterThreads) k_moments_cluster(const uint3
                                                                      const uint32_t *__restrict__ inodes,
                                                                      const uint32_t *__restrict__ kids, Dbl4 *raw)
 {
-    cluster_levels(lvl, inodes, [&](uint32_t p, int) { sum_children(p, kids, raw); });
+    cluster_levels(lvl, inodes, kids, [&](uint32_t p, int, const uint32_t (&kk)[8]) { sum_children(p, kk, raw); });
 }
 
 // Launches a kernel as one cluster of kClusterCtas blocks (beyond the portable 8: an opt-in
@@ -504,9 +530,9 @@ static void launch_cluster(void (*kern)(P...), std::atomic<bool> *set, cudaStrea
 }
 
 // The line between the two forms, in particles.  Tree stage with launches / with a cluster
-// (replayed calls): 4 k 0.082 / 0.057 ms, 32 k 0.087 / 0.071, 100 k 0.132 / 0.119, 300 k
-// 0.154 / 0.138, 500 k (not replayed) 0.215 / 0.170, 1 M 0.233 / 0.232 and second moments
-// 0.123 / 0.150, 2 M 0.334 / 0.360.
+// (replayed calls): 4 k 0.082 / 0.045 ms, 32 k 0.087 / 0.055, 100 k 0.132 / 0.098, 300 k
+// 0.154 / 0.115, 500 k (not replayed) 0.215 / 0.148, 1 M 0.217 / 0.225 and second moments
+// 0.119 / 0.156, 2 M 0.309 / 0.344.
 constexpr uint32_t kClusterMax = 700000;
 
 void launch_moments(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *kids,
@@ -567,8 +593,8 @@ __global__ void __launch_bounds__(256) k_quad_leaf(const Node *__restrict__ node
 }
 
 // The second moments of internal node p of the given level from its children's.
-__device__ __forceinline__ void quad_children(uint32_t p, int level, const Node *__restrict__ nodes,
-                                              const uint32_t *__restrict__ kids, const float4 *__restrict__ noff,
+__device__ __forceinline__ void quad_children(uint32_t p, int level, const uint32_t (&kk)[8],
+                                              const Node *__restrict__ nodes, const float4 *__restrict__ noff,
                                               const uint32_t *__restrict__ box_off, int nbox,
                                               const BoxPar *__restrict__ bps, float4 *quad)
 {
@@ -577,9 +603,6 @@ __device__ __forceinline__ void quad_children(uint32_t p, int level, const Node 
     const int hp = 1 << (kMaxLevel - level);
     const float4 cp = noff[p];
     float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
-    const uint4 k0 = kp[0], k1 = kp[1];
-    const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
 #pragma unroll
     for (int t = 0; t < 8; t++) {
         const uint32_t c = kk[t];
@@ -611,8 +634,13 @@ __global__ void __launch_bounds__(256) k_quad_level(int level, const uint32_t *_
                                                     const BoxPar *__restrict__ bps, float4 *quad)
 {
     const uint32_t b = lvl[32 + level], e = b + lvl[level];
-    for (uint32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x)
-        quad_children(inodes[i], level, nodes, kids, noff, box_off, nbox, bps, quad);
+    for (uint32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x) {
+        const uint32_t p = inodes[i];
+        const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
+        const uint4 k0 = kp[0], k1 = kp[1];
+        const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+        quad_children(p, level, kk, nodes, noff, box_off, nbox, bps, quad);
+    }
 }
 
 __global__ void __launch_bounds__(kClusterThreads) k_quad_cluster(
@@ -620,8 +648,8 @@ __global__ void __launch_bounds__(kClusterThreads) k_quad_cluster(
     const uint32_t *__restrict__ kids, const float4 *__restrict__ noff, const uint32_t *__restrict__ box_off, int nbox,
     const BoxPar *__restrict__ bps, float4 *quad)
 {
-    cluster_levels(lvl, inodes, [&](uint32_t p, int level) {
-        quad_children(p, level, nodes, kids, noff, box_off, nbox, bps, quad);
+    cluster_levels(lvl, inodes, kids, [&](uint32_t p, int level, const uint32_t (&kk)[8]) {
+        quad_children(p, level, kk, nodes, noff, box_off, nbox, bps, quad);
     });
 }
 

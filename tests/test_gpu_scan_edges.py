@@ -1,4 +1,5 @@
-"""The single-pass scans at the edges of their tiles (2048 counts, 1024 nodes) and the key
+"""The single-pass scans at the edges of their tiles (4096 counts, 1024 nodes), the sort on
+both sides of its two tile sizes (768 and 3072 pairs, the line at 200000) and the key
 kernel's digit counts: trees and groups against the oracle's, bit for bit, for particle
 numbers around the tile sizes, one box and several."""
 import numpy as np
@@ -25,7 +26,7 @@ def _check(ctx, pos, mass, n_crit, n_leaf):
     assert np.array_equal(ctx.dump(greem.DUMP_GROUPS), t.groups())
 
 
-@pytest.mark.parametrize("n", [1, 31, 255, 257, 2047, 2048, 2049, 4097, 65537])
+@pytest.mark.parametrize("n", [1, 31, 255, 257, 767, 769, 4095, 4096, 4097, 65537, 200000, 200001])
 @pytest.mark.parametrize("n_crit,n_leaf", [(1, 1), (64, 10)])
 def test_tree_and_groups(n, n_crit, n_leaf):
     rng = np.random.default_rng(n)
