@@ -752,6 +752,9 @@ __global__ void __launch_bounds__(GREEM_FORCE_THREADS, GREEM_FORCE_MINB) k_force
 // stretch [qoff[g], qoff[g] + qcnt[g]) of the quadrupole list (three float4 per entry:
 // the list entry, then the node's second moments, both in eta units).  One warp per group.  An overflow of
 // qcap entries records the total needed and the call is retried with a larger list.
+// Bound by the latency of its gathers: two chunks of 32 entries in flight per warp (1 M halo
+// particles: 178 -> 158 us; four chunks 174; stores staged in shared memory: the same).
+constexpr int kQFill = 2;
 __global__ void __launch_bounds__(256) k_qlist_fill(ForceArgs a, const float4 *__restrict__ quad, unsigned long long qcap)
 {
     const unsigned FULL = 0xffffffffu;
@@ -772,23 +775,38 @@ __global__ void __launch_bounds__(256) k_qlist_fill(ForceArgs a, const float4 *_
         const uint32_t len = a.lraw[g];
         const unsigned long long q0 = a.qoff[g];
         if (q0 + a.qcnt[g] > qcap) continue;
-        uint32_t k = 0;
-        for (uint32_t e0 = 0; e0 < len; e0 += 32) {
-            const uint32_t e = e0 + lane;
-            unsigned long long ie = 0;
-            if (e < len) ie = a.ilist[lo + e];
-            const bool node = e < len && ((ie >> 32) & 1ull) != 0;
-            const unsigned bal = __ballot_sync(FULL, node);
-            if (node) {
-                const uint32_t n = (uint32_t)(ie & 0xffffffffull);
-                float4 *d = const_cast<float4 *>(a.qlist) + 3ull * (q0 + k + __popc(bal & lt));
-                // r_cut units -> eta units (positions x2, second moments x4; exact)
-                const float4 f = a.flist[lo + e], q0 = quad[2 * (size_t)n], q1 = quad[2 * (size_t)n + 1];
-                d[0] = make_float4(2.0f * f.x, 2.0f * f.y, 2.0f * f.z, f.w);
-                d[1] = make_float4(4.0f * q0.x, 4.0f * q0.y, 4.0f * q0.z, 4.0f * q0.w);
-                d[2] = make_float4(4.0f * q1.x, 4.0f * q1.y, 4.0f * q1.z, 4.0f * q1.w);
+        float4 *out = const_cast<float4 *>(a.qlist) + 3ull * q0;
+        for (uint32_t e0 = 0; e0 < len; e0 += 32 * kQFill) {
+            uint32_t n[kQFill];
+            unsigned bal[kQFill];
+            float4 f[kQFill], qa[kQFill], qb[kQFill];
+#pragma unroll
+            for (int u = 0; u < kQFill; u++) {
+                const uint32_t e = e0 + 32 * u + lane;
+                unsigned long long ie = 0;
+                if (e < len) ie = a.ilist[lo + e];
+                n[u] = ((ie >> 32) & 1ull) ? (uint32_t)ie : 0xffffffffu;
             }
-            k += __popc(bal);
+#pragma unroll
+            for (int u = 0; u < kQFill; u++) {
+                bal[u] = __ballot_sync(FULL, n[u] != 0xffffffffu);
+                if (n[u] != 0xffffffffu) {
+                    f[u] = a.flist[lo + e0 + 32 * u + lane];
+                    qa[u] = quad[2 * (size_t)n[u]];
+                    qb[u] = quad[2 * (size_t)n[u] + 1];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kQFill; u++) {
+                if (n[u] != 0xffffffffu) {
+                    // r_cut units -> eta units (positions x2, second moments x4; exact)
+                    float4 *d = out + 3 * __popc(bal[u] & lt);
+                    d[0] = make_float4(2.0f * f[u].x, 2.0f * f[u].y, 2.0f * f[u].z, f[u].w);
+                    d[1] = make_float4(4.0f * qa[u].x, 4.0f * qa[u].y, 4.0f * qa[u].z, 4.0f * qa[u].w);
+                    d[2] = make_float4(4.0f * qb[u].x, 4.0f * qb[u].y, 4.0f * qb[u].z, 4.0f * qb[u].w);
+                }
+                out += 3 * __popc(bal[u]);
+            }
         }
     }
 }
