@@ -58,7 +58,7 @@ struct greem_ctx {
     DBuf<float> ms;
     // S3-S4
     DBuf<uint8_t> d8, K8;
-    DBuf<uint32_t> own, base, ctr, gstat;
+    DBuf<uint32_t> own, base, pend, gstat;
     DBuf<Node> nodes;
     DBuf<Dbl4> raw, mom64;
     DBuf<float4> noff, poff, irel;
@@ -71,7 +71,7 @@ struct greem_ctx {
     // S5-S6
     DBuf<float4> flist;
     DBuf<unsigned long long> ilist, loff;
-    DBuf<uint32_t> llen, lraw, kids, stack, order, bins, lvl;
+    DBuf<uint32_t> llen, lraw, kids, stack, order, bins, n_groups;
     DBuf<uint32_t> tbl;   // the list walk's start tables (k_start_table)
     int tbl_kmax = 0;     // the deepest start level of the current call's boxes
     int start_cap = 7;    // the deepest level a list walk may start at (greem_debug_set)
@@ -466,7 +466,7 @@ static int size_buffers(greem_ctx *c, const RunCfg &r)
     ENS(irel, N);
     const size_t nc = c->node_cap;
     ENS(nodes, nc);
-    ENS(ctr, nc);
+    ENS(pend, nc);
     ENS(raw, nc);
     ENS(mom64, nc);
     ENS(noff, nc);
@@ -481,7 +481,7 @@ static int size_buffers(greem_ctx *c, const RunCfg &r)
         ENS(qlist, c->qcap * 3);
     }
     ENS(kids, nc * 8);
-    ENS(lvl, kLvlWords);
+    ENS(n_groups, 1);
     ENS(bins, kBinWords);
     ENS(bps, (size_t)r.nbox);
     ENS(box_off, (size_t)r.nbox + 1);
@@ -626,9 +626,9 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     launch_gather(r.pos, r.mass, perm, N, c->box_off.p, nbox, c->bps.p, c->xs.p, c->ys.p, c->zs.p, c->ms.p, c->st.p,
                   s);
     ev_record(c, r, ev, 2);
-    ZeroList zt = {};  // the level counts, the group selection's look-back words, the work-order bins
-    zt.p[0] = c->lvl.p;
-    zt.n[0] = kLvlWords;
+    ZeroList zt = {};  // the number of groups, the group selection's look-back words, the work-order bins
+    zt.p[0] = c->n_groups.p;
+    zt.n[0] = 1;
     zt.p[1] = c->gstat.p;
     zt.n[1] = (uint32_t)group_status_words(ncap);
     zt.p[2] = c->bins.p;
@@ -637,7 +637,7 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     scan_u32(c->own.p, c->base.p, N, c->scratch.p, c->st.p, s, nullptr, true);
     const uint32_t *n_nodes = c->base.p + N;
     launch_tree_fill(ks, N, c->box_off.p, nbox, c->d8.p, c->K8.p, c->base.p, c->nodes.p, ncap, c->st.p, s, nsm);
-    launch_tree_links(c->nodes.p, n_nodes, ncap, c->kids.p, c->lvl.p, s, nsm);
+    launch_tree_links(c->nodes.p, n_nodes, ncap, c->kids.p, c->pend.p, s, nsm);
     // fork: the moments (FP64-bound) on s; the particle offsets and the groups (integer
     // work, reading only the tree) on the second stream
     cudaStream_t s2 = c->aux;
@@ -645,7 +645,7 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     cudaStreamWaitEvent(s2, c->ev_fork, 0);
     launch_leaf_offsets(ks, c->K8.p, N, c->box_off.p, nbox, c->bps.p, c->xs.p, c->ys.p, c->zs.p, c->ms.p, c->poff.p,
                         c->pcell.p, s2);
-    uint32_t *n_groups = c->lvl.p + 96;
+    uint32_t *n_groups = c->n_groups.p;
     launch_group_select(c->nodes.p, n_nodes, ncap, c->box_off.p, nbox, c->bps.p, c->groups.p, n_groups, c->gstat.p,
                         c->st.p, s2);
     launch_group_box(c->groups.p, n_groups, c->pcell.p, c->gbox.p, s2, nsm);
@@ -656,16 +656,14 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     }
     cudaEventRecord(c->ev_join, s2);
     launch_moments(c->nodes.p, n_nodes, ncap, c->kids.p, c->base.p, N, c->xs.p, c->ys.p, c->zs.p, c->ms.p, c->raw.p,
-                   c->lvl.p,
-                   c->ctr.p, s, nsm);
+                   c->pend.p, s, nsm);
     launch_node_finish(c->nodes.p, n_nodes, ncap, c->raw.p, c->box_off.p, nbox, c->bps.p, c->mom64.p, c->noff.p, s,
                        nsm);
     ev_record(c, r, ev, 3);
     // join: what the second stream still had to do counts as the groups stage
     cudaStreamWaitEvent(s, c->ev_join, 0);
     if (r.quad)
-        launch_quadrupoles(c->nodes.p, n_nodes, ncap, c->kids.p, c->poff.p, c->noff.p, c->lvl.p, c->ctr.p,
-                           N, c->box_off.p, nbox, c->bps.p, c->quad.p, s, nsm);
+        launch_quadrupoles(c->nodes.p, n_nodes, ncap, c->kids.p, c->poff.p, c->noff.p, c->pend.p, c->box_off.p, nbox, c->bps.p, c->quad.p, s, nsm);
     ev_record(c, r, ev, 4);
     if (r.lists_force) {
         ListArgs la;
@@ -970,12 +968,12 @@ void greem_destroy(greem_ctx *c)
     release(c->k0); release(c->k1); release(c->v0); release(c->v1); release(c->hist); release(c->scratch);
     release(c->rs_status); release(c->rs_runs);
     release(c->xs); release(c->ys); release(c->zs); release(c->ms);
-    release(c->d8); release(c->K8); release(c->own); release(c->base); release(c->ctr);
+    release(c->d8); release(c->K8); release(c->own); release(c->base); release(c->pend);
     release(c->gstat); release(c->nodes); release(c->raw); release(c->mom64); release(c->noff);
     release(c->poff); release(c->pcell); release(c->lbox); release(c->irel); release(c->groups); release(c->gbox); release(c->quad);
     release(c->flist); release(c->ilist); release(c->loff);
     release(c->llen); release(c->lraw); release(c->kids); release(c->stack); release(c->order); release(c->bins);
-    release(c->lvl); release(c->bps); release(c->box_off); release(c->small); release(c->st);
+    release(c->n_groups); release(c->bps); release(c->box_off); release(c->small); release(c->st);
     release(c->qlist); release(c->qcnt); release(c->qoff);
     release(c->dom_boxes); release(c->dom); release(c->dom_cnt); release(c->let_flag); release(c->let_cnt);
     release(c->let_ends); release(c->tbl);

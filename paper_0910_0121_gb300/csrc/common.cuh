@@ -244,21 +244,19 @@ void launch_gather(const double *pos, const float *mass, const uint32_t *perm, u
                    cudaStream_t s);
 
 // S3-S4 (tree.cu)
-constexpr int kLvlWords = 128;  // words of lvl: see launch_moments; [96]: the number of groups
 void launch_tree_prep(const uint64_t *keys, uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps,
                       uint8_t *d8, uint8_t *K8, uint32_t *own, const ZeroList &zero, cudaStream_t s);
 void launch_tree_fill(const uint64_t *keys, uint32_t N, const uint32_t *box_off, int nbox, const uint8_t *d8,
                       const uint8_t *K8, const uint32_t *base, Node *nodes, uint32_t node_cap, DevStatus *st,
                       cudaStream_t s, int nsm);
-void launch_tree_links(Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, uint32_t *kids, uint32_t *lvl,
+void launch_tree_links(Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, uint32_t *kids, uint32_t *pend,
                        cudaStream_t s, int nsm);
 void launch_moments(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *kids,
                     const uint32_t *base, uint32_t N, const double *xs, const double *ys, const double *zs,
-                    const float *ms, Dbl4 *raw, uint32_t *lvl, uint32_t *inodes, cudaStream_t s, int nsm);
+                    const float *ms, Dbl4 *raw, uint32_t *pend, cudaStream_t s, int nsm);
 void launch_quadrupoles(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *kids,
-                        const float4 *poff, const float4 *noff, const uint32_t *lvl, const uint32_t *inodes,
-                        uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps, float4 *quad, cudaStream_t s,
-                        int nsm);
+                        const float4 *poff, const float4 *noff, uint32_t *pend, const uint32_t *box_off, int nbox,
+                        const BoxPar *bps, float4 *quad, cudaStream_t s, int nsm);
 void launch_leaf_boxes(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap,
                        const unsigned long long *pcell, unsigned long long *lbox, cudaStream_t s, int nsm);
 void launch_leaf_offsets(const uint64_t *keys, const uint8_t *K8, uint32_t N, const uint32_t *box_off, int nbox,

@@ -14,7 +14,6 @@
 // prefix, so K_i comes from a sliding maximum over such windows.  Particle i then owns
 // the nodes (i, d_i) ... (i, K_i); an exclusive scan of the ownership counts numbers
 // the nodes in DFS preorder, because preorder is the order of (begin, level).
-#include <cooperative_groups.h>
 
 #include <algorithm>
 #include <atomic>
@@ -217,33 +216,32 @@ __device__ __forceinline__ uint32_t node_count(const uint32_t *n_nodes, uint32_t
     return n < cap ? n : cap;
 }
 
-// Parent links, child counts, the child table (up to 8 children per internal node,
-// unused slots kNone) and each node's child-octant mask (bits 16-23 of lvl; octant =
-// x<<2 | y<<1 | z of the child's cell within the parent's); the internal nodes of each
-// level are counted on the way (lvl[level]).  The children of an internal
+// Parent links, the child table (up to 8 children per internal node, unused slots kNone),
+// each node's child-octant mask (bits 16-23 of lvl; octant = x<<2 | y<<1 | z of the
+// child's cell within the parent's) and its word of `pend` (climb below): kNone for a leaf,
+// else n | n << 8, n its children that are internal nodes.  The children of an internal
 // node p are p+1 and then the skip chain while it stays inside p's particle range, in
 // Morton order, so slot q holds the child in the octant of the mask's (q+1)-th set bit.
 __global__ void __launch_bounds__(256) k_tree_links(Node *__restrict__ nodes, const uint32_t *__restrict__ n_nodes,
                                                     uint32_t node_cap, uint32_t *__restrict__ kids,
-                                                    uint32_t *__restrict__ lvl)
+                                                    uint32_t *__restrict__ pend)
 {
-    __shared__ uint32_t cnt_[32];
-    if (threadIdx.x < 32) cnt_[threadIdx.x] = 0;
-    __syncthreads();
     const uint32_t nn = node_count(n_nodes, node_cap);
     for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < nn; p += gridDim.x * blockDim.x) {
         const Node np = nodes[p];
         uint32_t slot[8];
 #pragma unroll
         for (int k = 0; k < 8; k++) slot[k] = kNone;
-        uint32_t cnt = 0, mask = 0;
+        uint32_t cnt = 0, mask = 0, wait = kNone;
         if (!(np.lvl & 256u)) {
             const int sh = kMaxLevel - 1 - (int)(np.lvl & 255u);  // child side in finest cells = 1 << sh
             uint32_t c = p + 1;
+            wait = 0;
             while (c < nn && nodes[c].begin < np.end && cnt < 8) {
                 const Node nc = nodes[c];
                 nodes[c].parent = p;
                 mask |= 1u << ((((nc.ix >> sh) & 1u) << 2) | (((nc.iy >> sh) & 1u) << 1) | ((nc.iz >> sh) & 1u));
+                wait += (nc.lvl & 256u) ? 0u : 0x101u;
 #pragma unroll
                 for (int k = 0; k < 8; k++)
                     if (k == (int)cnt) slot[k] = c;
@@ -251,20 +249,18 @@ __global__ void __launch_bounds__(256) k_tree_links(Node *__restrict__ nodes, co
                 c = nc.skip;
             }
             nodes[p].lvl = np.lvl | (mask << 16);
-            atomicAdd(&cnt_[np.lvl & 255u], 1u);
         }
         uint4 *kp = reinterpret_cast<uint4 *>(kids + (size_t)p * 8);
         kp[0] = make_uint4(slot[0], slot[1], slot[2], slot[3]);
         kp[1] = make_uint4(slot[4], slot[5], slot[6], slot[7]);
+        pend[p] = wait;
     }
-    __syncthreads();
-    if (threadIdx.x < 32 && cnt_[threadIdx.x]) atomicAdd(&lvl[threadIdx.x], cnt_[threadIdx.x]);
 }
 
-void launch_tree_links(Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, uint32_t *kids, uint32_t *lvl,
+void launch_tree_links(Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, uint32_t *kids, uint32_t *pend,
                        cudaStream_t s, int nsm)
 {
-    k_tree_links<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, node_cap, kids, lvl);
+    k_tree_links<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, node_cap, kids, pend);
     g_launches++;
 }
 
@@ -272,58 +268,70 @@ void launch_tree_links(Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, 
 // their particles in FP64 by tiles of consecutive particles (k_moments_leaf_tiled below:
 // coalesced loads, and within a tile the leaves taken in order of particle count, so the
 // lanes of a warp loop over equally many particles: an FP64 warp instruction costs the
-// same with idle lanes, and FP64 issue is expensive on this GPU).  Internal nodes are
-// bucketed by level and follow level by level, deepest first, each summing its
-// children's raw moments in child order.  Every sum has a fixed order, so the result
-// does not depend on scheduling.
-//
-// lvl[0..32): internal nodes per level (k_tree_links), lvl[32..64): each level's first place
-// in inodes, lvl[64..96): places taken so far.
+// same with idle lanes, and FP64 issue is expensive on this GPU).  Internal nodes follow
+// in one climb (k_moments_up), each summing its children's raw moments in child order.
+// Every sum has a fixed order, so the result does not depend on scheduling.
 
-// The exclusive prefix sums of the level counts, by the first warp of a block (smem start).
-__device__ __forceinline__ void level_starts(const uint32_t *__restrict__ lvl, uint32_t *start)
+// Calls f(p, has) for every internal node p after the calls for its internal children, in
+// one launch and without a wait: a node counts its finished internal children in pend, and
+// the warp that finishes the last of them takes the node on.  A warp keeps a queue of
+// nodes that are ready, first those with no internal child (found by a scan over pend),
+// then the parents its own nodes complete, and works on 32 / LANES of them at a time, LANES
+// lanes each, so that its lanes stay full.  UP: pend counts from 0 up to n (the second
+// climb of a tree), else from n down to 0.
+// What bounds it is the chain of a node's round trips (queue, child table, children, fence,
+// count: about 1 us a level) and, from a few million nodes, FP64 issue.  Moments of all
+// levels, against a launch per level (more than 700 k particles) or one cluster of 16 blocks
+// with its barriers, and the lists of each level's nodes that both of them need: tree stage
+// 100 k particles 0.098 -> 0.080 ms, 300 k 0.114 -> 0.092, 2 M 0.309 -> 0.250 and 0.330 ->
+// 0.235 (halos, one state of a step), 16.8 M 1.56 -> 1.47; second moments of 1 M 0.121 -> 0.061 ms.
+// f's stores are made before the count (fence, then atomic) and what it reads of the
+// children after it; it has to read them past the L1 cache (__ldcg).
+constexpr int kClimbWarps = 8;
+template <int LANES, bool UP, class F>
+__device__ __forceinline__ void climb(const Node *__restrict__ nodes, uint32_t nn, uint32_t *pend, F &&f)
 {
-    if (threadIdx.x < 32) {
-        const uint32_t v = lvl[threadIdx.x];
-        uint32_t x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (threadIdx.x >= (uint32_t)o) x += y;
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr uint32_t PER = 32 / LANES;
+    __shared__ uint32_t queue[kClimbWarps][64];  // at most PER - 1 + 32 before a step, then PER fewer and PER more
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const uint32_t sub = (uint32_t)lane / LANES;
+    uint32_t *q = queue[w];
+    uint32_t qn = 0;  // the same in every lane
+    const uint32_t nchunks = (nn + 31) / 32, nwarps = gridDim.x * kClimbWarps;
+    uint32_t ch = blockIdx.x * kClimbWarps + (uint32_t)w;
+    for (;;) {
+        while (qn < PER && ch < nchunks) {
+            const uint32_t n = ch * 32 + (uint32_t)lane;
+            // a word with n > 0 is never 0: the upper byte stays
+            const bool start = n < nn && pend[n] == 0u;
+            const unsigned m = __ballot_sync(FULL, start);
+            if (start) q[qn + __popc(m & lt)] = n;
+            qn += __popc(m);
+            ch += nwarps;
         }
-        start[threadIdx.x] = x - v;
-    }
-}
-
-// Places every internal node in its level's stretch of inodes: a slot within the block from
-// a shared-memory counter, then one global atomic per level and block.  The order within a
-// level is free (its nodes are summed independently).
-__global__ void __launch_bounds__(256) k_level_scatter(const Node *__restrict__ nodes,
-                                                       const uint32_t *__restrict__ n_nodes, uint32_t node_cap,
-                                                       uint32_t *__restrict__ lvl, uint32_t *__restrict__ inodes)
-{
-    __shared__ uint32_t cnt[32], base[32], start[32];
-    if (threadIdx.x < 32) cnt[threadIdx.x] = 0;
-    level_starts(lvl, start);
-    __syncthreads();
-    if (blockIdx.x == 0 && threadIdx.x < 32) lvl[32 + threadIdx.x] = start[threadIdx.x];
-    const uint32_t nn = node_count(n_nodes, node_cap);
-    const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t key = 0, slot = 0;
-    bool inner = false;
-    if (n < nn) {
-        const uint32_t l = nodes[n].lvl;
-        inner = !(l & 256u);  // leaves are summed by tiles
-        if (inner) {
-            key = l & 255u;
-            slot = atomicAdd(&cnt[key], 1u);
+        if (qn == 0) return;
+        __syncwarp();
+        const uint32_t take = min(qn, PER);
+        qn -= take;
+        const bool has = sub < take;
+        const uint32_t p = has ? q[qn + sub] : 0u;
+        const uint32_t parent = has ? nodes[p].parent : kNone;
+        f(p, has);
+        __threadfence();
+        __syncwarp();
+        bool ready = false;
+        if (parent != kNone && (uint32_t)lane % LANES == 0) {
+            const uint32_t old = atomicAdd(&pend[parent], UP ? 1u : ~0u);
+            ready = UP ? (old & 255u) + 1u == old >> 8 : (old & 255u) == 1u;
         }
+        __threadfence();
+        const unsigned m = __ballot_sync(FULL, ready);
+        if (ready) q[qn + __popc(m & lt)] = parent;
+        qn += __popc(m);
+        __syncwarp();
     }
-    __syncthreads();
-    if (threadIdx.x < 32 && cnt[threadIdx.x])
-        base[threadIdx.x] = start[threadIdx.x] + atomicAdd(&lvl[64 + threadIdx.x], cnt[threadIdx.x]);
-    __syncthreads();
-    if (inner) inodes[base[key] + slot] = n;
 }
 
 // Leaf moments by tiles of consecutive particles: a block takes the leaves that start in
@@ -417,142 +425,47 @@ __global__ void __launch_bounds__(256) k_moments_leaf_tiled(const Node *__restri
     }
 }
 
-// The raw moments of internal node p: its children's, in child order.
-__device__ __forceinline__ void sum_children(uint32_t p, const uint32_t (&kk)[8], Dbl4 *raw)
+// The raw moments of the internal nodes, four lanes a node: a lane sums one component of
+// its children's, in child order.
+__global__ void __launch_bounds__(32 * kClimbWarps) k_moments_up(const Node *__restrict__ nodes,
+                                                                 const uint32_t *__restrict__ n_nodes,
+                                                                 uint32_t node_cap, uint32_t *pend,
+                                                                 const uint32_t *__restrict__ kids, double *raw)
 {
-    Dbl4 a = make_dbl4(0.0, 0.0, 0.0, 0.0), r[8];
-#pragma unroll
-    for (int q = 0; q < 8; q++)  // all loads before the first sum
-        r[q] = kk[q] != kNone ? raw[kk[q]] : a;
-#pragma unroll
-    for (int q = 0; q < 8; q++) {
-        if (kk[q] == kNone) break;
-        a.x += r[q].x;
-        a.y += r[q].y;
-        a.z += r[q].z;
-        a.w += r[q].w;
-    }
-    raw[p] = a;
-}
-
-__global__ void __launch_bounds__(256) k_moments_level(int level, const uint32_t *__restrict__ lvl,
-                                                       const uint32_t *__restrict__ inodes,
-                                                       const uint32_t *__restrict__ kids, Dbl4 *raw)
-{
-    const uint32_t b = lvl[32 + level], e = b + lvl[level];
-    for (uint32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x) {
-        const uint32_t p = inodes[i];
+    const uint32_t c = threadIdx.x & 3u;
+    climb<4, false>(nodes, node_count(n_nodes, node_cap), pend, [&](uint32_t p, bool has) {
+        uint32_t kk[8];
         const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
-        const uint4 k0 = kp[0], k1 = kp[1];
-        const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-        sum_children(p, kk, raw);
-    }
-}
-
-// Every level in one launch, for smaller trees: one cluster of blocks goes through the
-// levels, deepest first, with a hardware cluster barrier after each that holds nodes (the
-// 21 launches of the form above cost more than their sums).  Its 16 blocks have a tenth of
-// the GPU's FP64 rate, which sets the line kClusterMax.
-constexpr int kClusterCtas = 16;
-constexpr int kClusterThreads = 256;  // 512: tree stage of 100 k particles 0.113 ms, 256: 0.098, 128: 0.092 (300 k: the same)
-
-// f(p, level, kids of p) for every internal node.  A thread loads its first node of a level
-// and its child table before the barrier that ends the level below: neither depends on it,
-// and the level's chain of memory round trips shortens to the children's moments.
-template <class F>
-__device__ __forceinline__ void cluster_levels(const uint32_t *__restrict__ lvl, const uint32_t *__restrict__ inodes,
-                                               const uint32_t *__restrict__ kids, F &&f)
-{
-    const auto cl = cooperative_groups::this_cluster();
-    __shared__ uint32_t cnt[32], start[32];
-    if (threadIdx.x < 32) {
-        cnt[threadIdx.x] = lvl[threadIdx.x];
-        start[threadIdx.x] = lvl[32 + threadIdx.x];
-    }
-    __syncthreads();
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    auto below = [&](int level) {
-        do level--;
-        while (level >= 0 && cnt[level] == 0);
-        return level;  // the same in every block
-    };
-    uint32_t p = 0;
-    uint4 k0 = make_uint4(0, 0, 0, 0), k1 = k0;
-    auto load = [&](int level, uint32_t i) {
-        p = inodes[start[level] + i];
-        const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
-        k0 = kp[0];
-        k1 = kp[1];
-    };
-    int level = below(kMaxLevel);
-    if (level >= 0 && t < cnt[level]) load(level, t);
-    while (level >= 0) {
-        for (uint32_t i = t; i < cnt[level]; i += nt) {
-            if (i != t) load(level, i);
-            const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-            f(p, level, kk);
+        const uint4 none = make_uint4(kNone, kNone, kNone, kNone), k0 = has ? kp[0] : none, k1 = has ? kp[1] : none;
+        kk[0] = k0.x; kk[1] = k0.y; kk[2] = k0.z; kk[3] = k0.w;
+        kk[4] = k1.x; kk[5] = k1.y; kk[6] = k1.z; kk[7] = k1.w;
+        double r[8], a = 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; q++)  // all loads before the first sum
+            r[q] = kk[q] != kNone ? __ldcg(raw + 4 * (size_t)kk[q] + c) : 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            if (!__any_sync(0xffffffffu, kk[q] != kNone)) break;
+            a += r[q];
         }
-        level = below(level);
-        if (level >= 0 && t < cnt[level]) load(level, t);
-        cl.sync();
-    }
+        if (has) raw[4 * (size_t)p + c] = a;
+    });
 }
 
-__global__ void __launch_bounds__(kClusterThreads) k_moments_cluster(const uint32_t *__restrict__ lvl,
-                                                                     const uint32_t *__restrict__ inodes,
-                                                                     const uint32_t *__restrict__ kids, Dbl4 *raw)
+static unsigned climb_grid(uint32_t node_cap, int nsm)
 {
-    cluster_levels(lvl, inodes, kids, [&](uint32_t p, int, const uint32_t (&kk)[8]) { sum_children(p, kk, raw); });
+    return (unsigned)std::min<size_t>(((size_t)node_cap + 32 * kClimbWarps - 1) / (32 * kClimbWarps), (size_t)nsm * 4);
 }
-
-// Launches a kernel as one cluster of kClusterCtas blocks (beyond the portable 8: an opt-in
-// per kernel and device, kept in `set`).
-template <class... P, class... A>
-static void launch_cluster(void (*kern)(P...), std::atomic<bool> *set, cudaStream_t s, A... args)
-{
-    const int dev = current_device_index();
-    if (dev < 0 || !set[dev].load()) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (dev >= 0) set[dev].store(true);
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = kClusterCtas;
-    cfg.blockDim = kClusterThreads;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kClusterCtas;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kern, P(args)...);
-    g_launches++;
-}
-
-// The line between the two forms, in particles.  Tree stage with launches / with a cluster
-// (replayed calls): 4 k 0.082 / 0.045 ms, 32 k 0.087 / 0.055, 100 k 0.132 / 0.098, 300 k
-// 0.154 / 0.115, 500 k (not replayed) 0.215 / 0.148, 1 M 0.217 / 0.225 and second moments
-// 0.119 / 0.156, 2 M 0.309 / 0.344.
-constexpr uint32_t kClusterMax = 700000;
 
 void launch_moments(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *kids,
                     const uint32_t *base, uint32_t N, const double *xs, const double *ys, const double *zs,
-                    const float *ms, Dbl4 *raw, uint32_t *lvl, uint32_t *inodes, cudaStream_t s, int nsm)
+                    const float *ms, Dbl4 *raw, uint32_t *pend, cudaStream_t s, int nsm)
 {
-    const unsigned grid = (node_cap + 255) / 256;
-    k_level_scatter<<<grid, 256, 0, s>>>(nodes, n_nodes, node_cap, lvl, inodes);
     k_moments_leaf_tiled<<<(N + kLeafTile - 1) / kLeafTile, 256, 0, s>>>(nodes, n_nodes, node_cap, base, N, xs, ys,
                                                                        zs, ms, raw);
+    k_moments_up<<<climb_grid(node_cap, nsm), 32 * kClimbWarps, 0, s>>>(nodes, n_nodes, node_cap, pend, kids,
+                                                                      reinterpret_cast<double *>(raw));
     g_launches += 2;
-    if (N <= kClusterMax) {
-        static std::atomic<bool> set[kMaxDevices];
-        launch_cluster(k_moments_cluster, set, s, lvl, inodes, kids, raw);
-        return;
-    }
-    for (int level = kMaxLevel - 1; level >= 0; level--) {
-        k_moments_level<<<nsm * 4, 256, 0, s>>>(level, lvl, inodes, kids, raw);
-        g_launches++;
-    }
 }
 
 // Second moments about the COM (the second-order terms of Sec. 4.1), FP32 in r_cut^2 units,
@@ -592,83 +505,54 @@ __global__ void __launch_bounds__(256) k_quad_leaf(const Node *__restrict__ node
     }
 }
 
-// The second moments of internal node p of the given level from its children's.
-__device__ __forceinline__ void quad_children(uint32_t p, int level, const uint32_t (&kk)[8],
-                                              const Node *__restrict__ nodes, const float4 *__restrict__ noff,
-                                              const uint32_t *__restrict__ box_off, int nbox,
-                                              const BoxPar *__restrict__ bps, float4 *quad)
+// The second moments of the internal nodes, eight lanes a node: each lane moves one child's,
+// and the sums are taken in child order.
+__global__ void __launch_bounds__(32 * kClimbWarps) k_quad_up(const Node *__restrict__ nodes,
+                                                              const uint32_t *__restrict__ n_nodes, uint32_t node_cap,
+                                                              uint32_t *pend, const uint32_t *__restrict__ kids,
+                                                              const float4 *__restrict__ noff,
+                                                              const uint32_t *__restrict__ box_off, int nbox,
+                                                              const BoxPar *__restrict__ bps, float4 *quad)
 {
-    const Node np = nodes[p];
-    const float kf = bps[box_of(np.begin, box_off, nbox)].k_f;
-    const int hp = 1 << (kMaxLevel - level);
-    const float4 cp = noff[p];
-    float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const uint32_t t = threadIdx.x & 7u;
+    climb<8, true>(nodes, node_count(n_nodes, node_cap), pend, [&](uint32_t p, bool has) {
+        const uint32_t c = has ? kids[(size_t)p * 8 + t] : kNone;
+        float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (c != kNone) {
+            const float4 q0 = __ldcg(quad + 2 * (size_t)c), q1 = __ldcg(quad + 2 * (size_t)c + 1);
+            const Node np = nodes[p], nc = nodes[c];
+            const float kf = bps[box_of(np.begin, box_off, nbox)].k_f;
+            const int hc = 1 << (kMaxLevel - (int)(nc.lvl & 255u)), hp = 2 * hc;
+            const float4 cp = noff[p], cc = noff[c];
+            // child COM - node COM: cell-centre difference (exact integer in u) and COM offsets
+            const float dx = fmaf((float)(2 * ((int)nc.ix - (int)np.ix) + hc - hp), kf, cc.x - cp.x);
+            const float dy = fmaf((float)(2 * ((int)nc.iy - (int)np.iy) + hc - hp), kf, cc.y - cp.y);
+            const float dz = fmaf((float)(2 * ((int)nc.iz - (int)np.iz) + hc - hp), kf, cc.z - cp.z);
+            const float mx = cc.w * dx, my = cc.w * dy, mz = cc.w * dz;
+            v[0] = fmaf(mx, dx, q0.x);
+            v[1] = fmaf(my, dy, q0.y);
+            v[2] = fmaf(mz, dz, q0.z);
+            v[3] = fmaf(mx, dy, q0.w);
+            v[4] = fmaf(mx, dz, q1.x);
+            v[5] = fmaf(my, dz, q1.y);
+        }
+        float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int t = 0; t < 8; t++) {
-        const uint32_t c = kk[t];
-        if (c == kNone) break;
-        const Node nc = nodes[c];
-        const int hc = hp >> 1;
-        const float4 cc = noff[c];
-        // child COM - node COM: cell-centre difference (exact integer in u) and COM offsets
-        const float dx = fmaf((float)(2 * ((int)nc.ix - (int)np.ix) + hc - hp), kf, cc.x - cp.x);
-        const float dy = fmaf((float)(2 * ((int)nc.iy - (int)np.iy) + hc - hp), kf, cc.y - cp.y);
-        const float dz = fmaf((float)(2 * ((int)nc.iz - (int)np.iz) + hc - hp), kf, cc.z - cp.z);
-        const float4 q0 = quad[2 * (size_t)c], q1 = quad[2 * (size_t)c + 1];
-        const float mx = cc.w * dx, my = cc.w * dy, mz = cc.w * dz;
-        q[0] += fmaf(mx, dx, q0.x);
-        q[1] += fmaf(my, dy, q0.y);
-        q[2] += fmaf(mz, dz, q0.z);
-        q[3] += fmaf(mx, dy, q0.w);
-        q[4] += fmaf(mx, dz, q1.x);
-        q[5] += fmaf(my, dz, q1.y);
-    }
-    quad_store(quad, p, q);
-}
-
-__global__ void __launch_bounds__(256) k_quad_level(int level, const uint32_t *__restrict__ lvl,
-                                                    const uint32_t *__restrict__ inodes,
-                                                    const Node *__restrict__ nodes, const uint32_t *__restrict__ kids,
-                                                    const float4 *__restrict__ noff,
-                                                    const uint32_t *__restrict__ box_off, int nbox,
-                                                    const BoxPar *__restrict__ bps, float4 *quad)
-{
-    const uint32_t b = lvl[32 + level], e = b + lvl[level];
-    for (uint32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x) {
-        const uint32_t p = inodes[i];
-        const uint4 *kp = reinterpret_cast<const uint4 *>(kids + (size_t)p * 8);
-        const uint4 k0 = kp[0], k1 = kp[1];
-        const uint32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-        quad_children(p, level, kk, nodes, noff, box_off, nbox, bps, quad);
-    }
-}
-
-__global__ void __launch_bounds__(kClusterThreads) k_quad_cluster(
-    const uint32_t *__restrict__ lvl, const uint32_t *__restrict__ inodes, const Node *__restrict__ nodes,
-    const uint32_t *__restrict__ kids, const float4 *__restrict__ noff, const uint32_t *__restrict__ box_off, int nbox,
-    const BoxPar *__restrict__ bps, float4 *quad)
-{
-    cluster_levels(lvl, inodes, kids, [&](uint32_t p, int level, const uint32_t (&kk)[8]) {
-        quad_children(p, level, kk, nodes, noff, box_off, nbox, bps, quad);
+        for (int k = 0; k < 8; k++)
+#pragma unroll
+            for (int i = 0; i < 6; i++) q[i] += __shfl_sync(0xffffffffu, v[i], k, 8);
+        if (has && t == 0) quad_store(quad, p, q);
     });
 }
 
 void launch_quadrupoles(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *kids,
-                        const float4 *poff, const float4 *noff, const uint32_t *lvl, const uint32_t *inodes,
-                        uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps, float4 *quad, cudaStream_t s,
-                        int nsm)
+                        const float4 *poff, const float4 *noff, uint32_t *pend, const uint32_t *box_off, int nbox,
+                        const BoxPar *bps, float4 *quad, cudaStream_t s, int nsm)
 {
     k_quad_leaf<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, node_cap, poff, noff, quad);
-    g_launches++;
-    if (N <= kClusterMax) {
-        static std::atomic<bool> set[kMaxDevices];
-        launch_cluster(k_quad_cluster, set, s, lvl, inodes, nodes, kids, noff, box_off, nbox, bps, quad);
-        return;
-    }
-    for (int level = kMaxLevel - 1; level >= 0; level--) {
-        k_quad_level<<<nsm * 4, 256, 0, s>>>(level, lvl, inodes, nodes, kids, noff, box_off, nbox, bps, quad);
-        g_launches++;
-    }
+    k_quad_up<<<climb_grid(node_cap, nsm), 32 * kClimbWarps, 0, s>>>(nodes, n_nodes, node_cap, pend, kids, noff,
+                                                                   box_off, nbox, bps, quad);
+    g_launches += 2;
 }
 
 // Each particle's offset from the centre of its leaf cell (level K_i) in r_cut units: the

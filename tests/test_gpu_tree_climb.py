@@ -1,6 +1,5 @@
-"""Moments and second moments summed level by level, by one cluster of blocks for smaller
-trees and by one launch per level above: shallow and deep trees on both sides of the line
-against sums over each node's particles."""
+"""Moments and second moments of every level in one climb from the deepest nodes: shallow and
+deep trees of all sizes against sums over each node's particles."""
 import numpy as np
 import pytest
 
