@@ -1,6 +1,7 @@
 // S5 Barnes (1990) grouped interaction lists (Sec. 2.2 steps 3 and 5; Sec. 3.1.2).
 //
-// One warp per group walks its box's tree from the root with a per-warp stack.  Every
+// One warp per group (a team of 2 or 4 when groups are few) walks its box's tree from the
+// root with a stack.  Every
 // node the recursive walk visits is tested, in this order:
 //   prune  -- the node's cell is farther than r_cut from the group's particle box (the
 //             box of finest-level cells that holds the group's particles; periodic
@@ -221,19 +222,61 @@ void launch_start_table(const Node *nodes, const uint32_t *kids, const uint32_t 
     g_launches++;
 }
 
+// The warps that walk one group together (W consecutive warps of a block; each chunk of 32
+// cells or particles goes to the next warp, and every warp keeps the walk's state).  A
+// chunk's entries and pushes go where one warp alone would put them: `mine` counts this
+// warp's, `before` those of the lower warps, `total` all of the team's.
+template <int W>
+struct Team {
+    uint32_t *slots = nullptr;  // two rows of W counts, used in turn: one barrier per exchange
+    uint32_t row = 0;
+    int wid = 0, bar = 0;       // warp within the team; the team's barrier
+    __device__ __forceinline__ void sync() const
+    {
+        if constexpr (W == 1) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(32 * W) : "memory");
+    }
+    __device__ __forceinline__ void place(uint32_t mine, int lane, uint32_t &before, uint32_t &total)
+    {
+        if constexpr (W == 1) {
+            before = 0;
+            total = mine;
+        } else {
+            const unsigned FULL = 0xffffffffu;
+            if (lane == 0) slots[row * W + wid] = mine;
+            sync();
+            const uint32_t v = lane < W ? slots[row * W + lane] : 0u;
+            row ^= 1u;
+            total = __reduce_add_sync(FULL, v);
+            before = __reduce_add_sync(FULL, lane < wid ? v : 0u);
+        }
+    }
+};
+
 // One tested cell per lane: an accepted node becomes one entry at its centre of mass
 // (acc), a node to open or a leaf to empty goes onto the stack (push).  Returns false
 // when the stack would overflow (the status is set; the call is retried).
-template <bool INDEX>
-__device__ __forceinline__ bool take_cells(const ListArgs &a, bool acc, bool push, uint32_t child, const CellTest &ct,
-                                           float kf, unsigned long long pos0, uint32_t room, unsigned lt,
-                                           uint32_t &cnt, uint32_t &nacc, uint32_t *__restrict__ stk, uint32_t &sp,
-                                           uint32_t cap)
+template <bool INDEX, int W>
+__device__ __forceinline__ bool take_cells(const ListArgs &a, Team<W> &team, bool acc, bool push, uint32_t child,
+                                           const CellTest &ct, float kf, unsigned long long pos0, uint32_t room,
+                                           int lane, unsigned lt, uint32_t &cnt, uint32_t &nacc,
+                                           uint32_t *__restrict__ stk, uint32_t &sp, uint32_t cap)
 {
     const unsigned FULL = 0xffffffffu;
     const unsigned ab = __ballot_sync(FULL, acc);
+    uint32_t na = __popc(ab), np = 0, a0 = 0, p0 = 0;
+    unsigned pb = 0;
+    if constexpr (W > 1) {
+        pb = __ballot_sync(FULL, push);
+        uint32_t before, total;
+        team.place(na | ((uint32_t)__popc(pb) << 16), lane, before, total);
+        a0 = before & 0xffffu;
+        p0 = before >> 16;
+        na = total & 0xffffu;
+        np = total >> 16;
+    }
     if (acc) {
-        const uint32_t p = cnt + __popc(ab & lt);
+        const uint32_t p = cnt + a0 + __popc(ab & lt);
         const float4 v = __ldg(a.noff + child);
         const float4 e = make_float4(__fadd_rn(__fmul_rn((float)ct.dx, kf), v.x),
                                      __fadd_rn(__fmul_rn((float)ct.dy, kf), v.y),
@@ -243,15 +286,18 @@ __device__ __forceinline__ bool take_cells(const ListArgs &a, bool acc, bool pus
             if (INDEX) a.ilist[pos0 + p] = (unsigned long long)child | (1ull << 32) | ((unsigned long long)ct.shc << 33);
         }
     }
-    cnt += __popc(ab);
-    nacc += __popc(ab);
-    const unsigned pb = __ballot_sync(FULL, push);
-    if (sp + __popc(pb) > cap) {
+    cnt += na;
+    nacc += na;
+    if constexpr (W == 1) {
+        pb = __ballot_sync(FULL, push);
+        np = __popc(pb);
+    }
+    if (sp + np > cap) {
         if (lt == 0u) atomicOr(&a.st->flags, ST_STACK);
         return false;
     }
-    if (push) stk[sp + __popc(pb & lt)] = child;
-    sp += __popc(pb);
+    if (push) stk[sp + p0 + __popc(pb & lt)] = child;
+    sp += np;
     return true;
 }
 
@@ -276,8 +322,8 @@ __device__ __forceinline__ long long word_tprune(const int4 w)
 // level-K cells within r_cut of the group's particle box, tested like the children of an
 // opened node.  Returns false if the group must walk from the root instead (sp is then
 // untouched); sets overflow on a stack overflow.
-template <bool INDEX>
-__device__ __forceinline__ bool start_cells(const ListArgs &a, uint32_t gsm, const BoxPar &bp, uint32_t *__restrict__ stk, unsigned long long pos0,
+template <bool INDEX, int W>
+__device__ __forceinline__ bool start_cells(const ListArgs &a, Team<W> &team, uint32_t gsm, const BoxPar &bp, uint32_t *__restrict__ stk, unsigned long long pos0,
                                             uint32_t room, int lane, unsigned lt, uint32_t &cnt,
                                             uint32_t &nacc, uint32_t &sp, bool &overflow)
 {
@@ -313,11 +359,12 @@ __device__ __forceinline__ bool start_cells(const ListArgs &a, uint32_t gsm, con
     const bool acc_level = K >= bp.lmin;
     const long long AK = bp.A[K];
     const float kf = bp.k_f;
-    // lane's candidate t = (ix ny + iy) nz + iz, advanced by 32 per chunk
-    int iz = lane % nz, iy = (lane / nz) % ny, ix = lane / (nz * ny);
-    const int sz = 32 % nz, qz = 32 / nz, sy = qz % ny, sx = qz / ny;
-    for (uint32_t c0 = 0; c0 < ncand; c0 += 32) {
-        const uint32_t t = c0 + (uint32_t)lane;
+    // lane's candidate t = (ix ny + iy) nz + iz, advanced by the team's chunks
+    const int l0 = 32 * team.wid + lane;
+    int iz = l0 % nz, iy = (l0 / nz) % ny, ix = l0 / (nz * ny);
+    const int sz = (32 * W) % nz, qz = (32 * W) / nz, sy = qz % ny, sx = qz / ny;
+    for (uint32_t c0 = 0; c0 < ncand; c0 += 32 * W) {
+        const uint32_t t = c0 + (uint32_t)l0;
         bool acc = false, push = false, node_coarse = false;
         uint32_t node = 0;
         CellTest ct;
@@ -359,7 +406,7 @@ __device__ __forceinline__ bool start_cells(const ListArgs &a, uint32_t gsm, con
                 }
             }
         }
-        if (!take_cells<INDEX>(a, acc, push, node, ct, kf, pos0, room, lt, cnt, nacc, stk, sp, a.stack_cap)) {
+        if (!take_cells<INDEX, W>(a, team, acc, push, node, ct, kf, pos0, room, lane, lt, cnt, nacc, stk, sp, a.stack_cap)) {
             overflow = true;
             break;
         }
@@ -392,8 +439,8 @@ __device__ __forceinline__ bool start_cells(const ListArgs &a, uint32_t gsm, con
 // pushed.  Last, the particles of the popped leaves are spread over the lanes and each
 // goes through the per-particle r_cut test unless its whole leaf lies within r_cut.
 // INDEX: the index entries are written too (a.ilist).
-template <bool INDEX>
-__device__ __forceinline__ uint32_t walk_group(const ListArgs &a, uint32_t gsm, const BoxPar &bp,
+template <bool INDEX, int W>
+__device__ __forceinline__ uint32_t walk_group(const ListArgs &a, Team<W> &team, uint32_t gsm, const BoxPar &bp,
                                uint32_t root, uint32_t *__restrict__ stk, const uint8_t *__restrict__ octq,
                                uint4 *__restrict__ src,
                                unsigned long long pos0, uint32_t room, int lane, uint32_t &nacc,
@@ -406,18 +453,18 @@ __device__ __forceinline__ uint32_t walk_group(const ListArgs &a, uint32_t gsm, 
     uint32_t cnt = 0;
     uint32_t sp = 0;
     bool overflow = false;
-    from_table = start_cells<INDEX>(a, gsm, bp, stk, pos0, room, lane, lt, cnt, nacc, sp, overflow);
+    from_table = start_cells<INDEX, W>(a, team, gsm, bp, stk, pos0, room, lane, lt, cnt, nacc, sp, overflow);
     if (!from_table) {
-        if (lane == 0) stk[0] = root;
+        if (team.wid == 0 && lane == 0) stk[0] = root;
         sp = 1;
     }
-    __syncwarp();
+    team.sync();
     while (sp > 0 && !overflow) {
         const uint32_t nb = min(sp, 32u);
         const uint32_t sbase = sp - nb;
         const bool valid = (uint32_t)lane < nb;
         const uint32_t m = valid ? stk[sbase + lane] : 0u;
-        __syncwarp();
+        __syncwarp();  // (a team's pushes come after its first exchange)
         sp = sbase;
         Node nd;
         unsigned long long lb = 0;
@@ -506,7 +553,7 @@ __device__ __forceinline__ uint32_t walk_group(const ListArgs &a, uint32_t gsm, 
         __syncwarp();
 
         // ---- children of the opened nodes: prune, accept (one entry), or push
-        for (uint32_t c0 = 0; c0 < ctot; c0 += 32) {
+        for (uint32_t c0 = 32 * team.wid; c0 < ctot + 32 * team.wid; c0 += 32 * W) {
             const uint32_t t = c0 + lane;
             const uint4 *sp_ = src + 2 * source_place(is_inner, o, c0, le);
             const uint4 u = sp_[0];
@@ -532,7 +579,7 @@ __device__ __forceinline__ uint32_t walk_group(const ListArgs &a, uint32_t gsm, 
                     push = !acc;
                 }
             }
-            if (!take_cells<INDEX>(a, acc, push, child, ct, __int_as_float(pw.z), pos0, room, lt, cnt, nacc, stk, sp, cap)) {
+            if (!take_cells<INDEX, W>(a, team, acc, push, child, ct, __int_as_float(pw.z), pos0, room, lane, lt, cnt, nacc, stk, sp, cap)) {
                 overflow = true;  // the caller's list is incomplete; the call is retried with a larger stack
                 break;
             }
@@ -541,7 +588,7 @@ __device__ __forceinline__ uint32_t walk_group(const ListArgs &a, uint32_t gsm, 
         if (overflow) break;
 
         // ---- particles of the popped leaves
-        for (uint32_t t0 = 0; t0 < tot; t0 += 32) {
+        for (uint32_t t0 = 32 * team.wid; t0 < tot + 32 * team.wid; t0 += 32 * W) {
             const uint32_t t = t0 + lane;
             const uint4 *sp_ = src + 2 * (n_inner + source_place(is_full, o, t0, le));
             const uint4 u = sp_[0], v4 = sp_[1];
@@ -571,74 +618,90 @@ __device__ __forceinline__ uint32_t walk_group(const ListArgs &a, uint32_t gsm, 
                 if (sh_s & 128u) a.irel[j] = e;
             }
             const unsigned kb = __ballot_sync(FULL, keep);
+            uint32_t before, total;
+            team.place(__popc(kb), lane, before, total);
             if (keep) {
-                const uint32_t p = cnt + __popc(kb & lt);
+                const uint32_t p = cnt + before + __popc(kb & lt);
                 if (p < room) {
                     a.flist[pos0 + p] = e;
                     if (INDEX) a.ilist[pos0 + p] = (unsigned long long)j | ((unsigned long long)(sh_s & 63u) << 33);
                 }
             }
-            cnt += __popc(kb);
+            cnt += total;
         }
-        __syncwarp();  // the sources are read
+        team.sync();  // the sources are read, the pushes made
     }
-    __syncwarp();
+    team.sync();
     return cnt;
 }
 
-template <bool INDEX>
-__global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(ListArgs a)
+// A block's shared memory.
+struct ListShared {
+    uint8_t octq[256 * 8];  // octq[8 mask + q]: the octant of the (q+1)-th set bit of an 8-bit child mask
+    unsigned long long tallies[kListWarps][kTallyN];
+    uint4 sources[kListWarps][64];  // walk_group's sources, two words of 16 bytes each
+    int4 gconst[kListWarps][4];     // group_word
+    uint32_t slots[2 * kListWarps];
+    unsigned long long word[kListWarps];
+};
+
+// The lists of all groups, W warps per group.
+template <bool INDEX, int W>
+__device__ __forceinline__ void build_lists(const ListArgs &a, ListShared &sm, uint32_t G)
 {
+    constexpr int BT = kListWarps / W;  // teams per block
     const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    // octq[8 mask + q]: the octant of the (q+1)-th set bit of an 8-bit child mask
-    __shared__ uint8_t octq[256 * 8];
-    for (uint32_t m = threadIdx.x; m < 256; m += blockDim.x) {
-        uint32_t q = 0;
-        for (uint32_t o = 0; o < 8; o++)
-            if (m & (1u << o)) octq[8 * m + q++] = (uint8_t)o;
-        for (; q < 8; q++) octq[8 * m + q] = 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tm = warp / W;  // team within the block
+    const uint8_t *octq = sm.octq;
+    uint4 *src = sm.sources[warp];
+    const uint32_t gsm = (uint32_t)__cvta_generic_to_shared(sm.gconst[tm]);
+    Team<W> team;
+    if constexpr (W > 1) {
+        team.slots = sm.slots + 2 * W * tm;
+        team.wid = warp % W;
+        team.bar = 1 + tm;
     }
-    __shared__ unsigned long long tallies[kListWarps][kTallyN];
-    __shared__ uint4 sources[kListWarps][64];  // walk_group's sources, two words of 16 bytes each
-    __shared__ int4 gconst[kListWarps][4];     // group_word
-    uint4 *src = sources[threadIdx.x >> 5];
-    const uint32_t gsm = (uint32_t)__cvta_generic_to_shared(gconst[threadIdx.x >> 5]);
-    if (lane == 0)
-        for (int k = 0; k < kTallyN; k++) tallies[threadIdx.x >> 5][k] = 0;
-    __syncthreads();
-    if (a.st->flags & ST_NODE_CAP) return;  // the tree was truncated: the call is retried
-    unsigned long long *tally = tallies[threadIdx.x >> 5];
-    const uint32_t G = *a.n_groups;
-    uint32_t *stk = a.stack + (size_t)(blockIdx.x * kListWarps + (threadIdx.x >> 5)) * a.stack_cap;
+    const bool first = team.wid == 0 && lane == 0;  // the team's first thread
+    // the first thread's value, for every thread of the team
+    auto share = [&](unsigned long long v) -> unsigned long long {
+        if constexpr (W == 1) return __shfl_sync(FULL, v, 0);
+        if (first) sm.word[tm] = v;
+        team.sync();
+        v = sm.word[tm];
+        team.sync();
+        return v;
+    };
+    unsigned long long *tally = sm.tallies[tm];
+    uint32_t *stk = a.stack + (size_t)(blockIdx.x * BT + tm) * a.stack_cap;
     unsigned long long page_cur = 0, page_end = 0;
     bool exhausted = false;  // the pool ran out: only count what the lists need
     // np fresh pages become the warp's current ones; false (and the status) past the pool
     auto take_pages = [&](unsigned long long np) -> bool {
-        unsigned long long first = 0;
-        if (lane == 0) first = atomicAdd(&a.st->list_pages, np);
-        first = __shfl_sync(FULL, first, 0);
-        if ((first + np) * a.page > a.cap) {
-            if (lane == 0) atomicOr(&a.st->flags, ST_LIST_CAP);
+        unsigned long long page0 = 0;
+        if (first) page0 = atomicAdd(&a.st->list_pages, np);
+        page0 = share(page0);
+        if ((page0 + np) * a.page > a.cap) {
+            if (first) atomicOr(&a.st->flags, ST_LIST_CAP);
             page_cur = page_end = 0;
             exhausted = true;
             return false;
         }
-        page_cur = first * a.page;
-        page_end = (first + np) * a.page;
+        page_cur = page0 * a.page;
+        page_end = (page0 + np) * a.page;
         return true;
     };
     for (;;) {
         unsigned long long gi = 0;
-        if (lane == 0) gi = atomicAdd(&a.st->work[0], 1ull);
-        gi = __shfl_sync(FULL, gi, 0);
+        if (first) gi = atomicAdd(&a.st->work[0], 1ull);
+        gi = share(gi);
         if (gi >= G) break;
         const uint32_t g = (uint32_t)gi;
-        __syncwarp();  // the last group's constants are read, lane 0's tallies written
+        if constexpr (W == 1) __syncwarp();  // the last group's constants are read, the tallies written
         const Group gr = a.groups[g];
         const BoxPar &bp = a.bps[gr.box];
-        if (lane == 0) {
-            int4 *w = gconst[threadIdx.x >> 5];
+        if (first) {
+            int4 *w = sm.gconst[tm];
             const int4 tb = a.gbox[2 * (size_t)g], th = a.gbox[2 * (size_t)g + 1];
             const unsigned long long Tp = (unsigned long long)bp.T_prune;
             w[0] = make_int4(gr.cx, gr.cy, gr.cz, gr.hg);
@@ -650,15 +713,15 @@ __global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(Lis
         if (!exhausted && (page_cur == page_end ||
                            (page_end - page_cur) * tally[kTallyGroups] < tally[kTallyPadded]))
             take_pages(1);
-        __syncwarp();
+        team.sync();
         uint32_t nacc = 0, len = 0, padded = 0;
         bool placed = false;
         for (bool again = false;; again = true) {
             bool from_table = false;
-            len = walk_group<INDEX>(a, gsm, bp, root, stk, octq, src, page_cur, (uint32_t)(page_end - page_cur), lane,
+            len = walk_group<INDEX, W>(a, team, gsm, bp, root, stk, octq, src, page_cur, (uint32_t)(page_end - page_cur), lane,
                                     nacc, from_table);
             padded = (len + 7u) & ~7u;
-            if (!again && lane == 0) {
+            if (!again && first) {
                 tally[kTallyStart] += from_table ? 1u : 0u;
                 tally[kTallyPadded] += padded;
                 tally[kTallyGroups]++;
@@ -668,7 +731,7 @@ __global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(Lis
             if (placed || !take_pages((padded + a.page - 1) / a.page)) break;
         }
         if (!placed) {
-            if (lane == 0) {
+            if (first) {
                 a.loff[g] = 0;
                 a.llen[g] = 0;
                 a.lraw[g] = 0;
@@ -676,11 +739,11 @@ __global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(Lis
             }
             continue;
         }
-        for (uint32_t t = len + lane; t < padded; t += 32) {
+        for (uint32_t t = len + lane; t < padded && team.wid == 0; t += 32) {
             a.flist[page_cur + t] = make_float4(16.f, 16.f, 16.f, 0.f);
             if (INDEX) a.ilist[page_cur + t] = ~0ull;
         }
-        if (lane == 0) {
+        if (first) {
             a.loff[g] = page_cur;
             a.llen[g] = padded;
             a.lraw[g] = len;
@@ -690,14 +753,37 @@ __global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(Lis
         }
         page_cur += padded;
     }
-    __syncwarp();
-    if (lane == 0) {
+    if (first) {
         DevStatus *st = a.st;
         if (tally[kTallyPadded]) atomicAdd(&st->sum_padded, tally[kTallyPadded]);
         if (tally[kTallyLen]) atomicAdd(&st->sum_len, tally[kTallyLen]);
         if (tally[kTallyInter]) atomicAdd(&st->sum_inter, tally[kTallyInter]);
         if (tally[kTallyStart]) atomicAdd(&st->sum_start, tally[kTallyStart]);
     }
+}
+
+template <bool INDEX>
+__global__ void __launch_bounds__(kListWarps * 32, kListBlocksPerSM) k_lists(ListArgs a)
+{
+    __shared__ ListShared sm;
+    for (uint32_t m = threadIdx.x; m < 256; m += blockDim.x) {
+        uint32_t q = 0;
+        for (uint32_t o = 0; o < 8; o++)
+            if (m & (1u << o)) sm.octq[8 * m + q++] = (uint8_t)o;
+        for (; q < 8; q++) sm.octq[8 * m + q] = 0;
+    }
+    if (threadIdx.x < kListWarps * kTallyN) (&sm.tallies[0][0])[threadIdx.x] = 0;
+    __syncthreads();
+    if (a.st->flags & ST_NODE_CAP) return;  // the tree was truncated: the call is retried
+    const uint32_t G = *a.n_groups, warps = gridDim.x * kListWarps;
+    // Few groups: several warps walk one together, as a walk is a chain of dependent round
+    // trips and most of the warps would have none.  A team's warps all pop and scan, so with
+    // enough groups for the warps one each is faster.  List stage with 1 / 2 / 4 warps per
+    // group, on 4864 warps (us): 512 groups 34.8 / 32.4 / 28.4, 963 57 / 47 / 41, 1630 67 /
+    // 53 / 57, 2657 73.5 / 67.3 / 77.5, 4096 71.4 / 75.8 / 104, 9923 146 / 199 / 252.
+    if (4 * (unsigned long long)G <= warps) build_lists<INDEX, 4>(a, sm, G);
+    else if (3 * (unsigned long long)G <= 2 * (unsigned long long)warps) build_lists<INDEX, 2>(a, sm, G);
+    else build_lists<INDEX, 1>(a, sm, G);
 }
 
 void launch_lists(const ListArgs &a, cudaStream_t s, int nsm)
