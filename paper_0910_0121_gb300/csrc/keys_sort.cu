@@ -76,12 +76,15 @@ __device__ __forceinline__ uint64_t particle_key(const double *__restrict__ pos,
 constexpr int kRsThreads = 256;
 constexpr int kRsWarps = kRsThreads / 32;
 #ifndef GREEM_RS_ITEMS
-#define GREEM_RS_ITEMS 12
+#define GREEM_RS_ITEMS 14
 #endif
 #ifndef GREEM_RS_MINB
 #define GREEM_RS_MINB 3
 #endif
-constexpr int kRsItems = GREEM_RS_ITEMS;        // pairs per thread
+// pairs per thread: sort stage at 10 / 12 / 14 / 16: 256^3 1.114 / 1.076 / 1.046 / 1.083 ms, 64
+// boxes 0.899 / 0.864 / 0.850 / 0.915, 2 M uniform 0.172 / 0.172 / 0.176 / 0.178 (with 12 and
+// ranking by ballots 1.141, 0.934, 0.213; all particles on a line, sorted, 0.360 -> 0.335)
+constexpr int kRsItems = GREEM_RS_ITEMS;
 // the same when the tiles are few: a pass then takes as long as one tile's chain of rankings
 // (sort stage at 12 / 4 / 3 / 2 pairs per thread: 4 k particles 0.045 / 0.033 / 0.031 / 0.030
 // ms, 32 k 0.047 / 0.037 / 0.035 / 0.037, 100 k 0.053 / 0.045 / 0.043 / 0.049, 300 k 0.063 /
@@ -122,19 +125,6 @@ __device__ __forceinline__ uint32_t rs_digit(uint64_t k, uint32_t v, int shift, 
 {
     if (SRC == 0) return (uint32_t)(k >> shift) & 255u;
     return ((uint32_t)box_of(v, box_off, nbox) >> shift) & 255u;
-}
-
-// Lanes of the warp whose 8-bit digit equals this lane's (d < 256; lanes with d = 256,
-// out of range, match only each other): one ballot per digit bit.
-__device__ __forceinline__ unsigned digit_peers(uint32_t d)
-{
-    unsigned peers = __ballot_sync(0xffffffffu, d >= 256u) ^ (d >= 256u ? 0u : 0xffffffffu);
-#pragma unroll
-    for (int b = 0; b < 8; b++) {
-        const unsigned bb = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-        peers &= ((d >> b) & 1u) ? bb : ~bb;
-    }
-    return peers;
 }
 
 // S1, and on the way what the sort needs: all digit histograms (the box digits from the box
@@ -204,12 +194,13 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
     uint64_t *sk = reinterpret_cast<uint64_t *>(rs_buf);
     uint32_t *sv = reinterpret_cast<uint32_t *>(rs_buf + (size_t)TILE * sizeof(uint64_t));
     __shared__ uint32_t wcnt[kRsWarps][256];
+    __shared__ uint32_t mask[kRsWarps][256];
     __shared__ uint32_t lstart[256];
     __shared__ uint32_t gbase[256];
     __shared__ uint32_t wsum[kRsWarps], dsum[kRsWarps];
     __shared__ uint32_t s_tile;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    for (int d = tid; d < kRsWarps * 256; d += kRsThreads) (&wcnt[0][0])[d] = 0;
+    for (int d = tid; d < kRsWarps * 256; d += kRsThreads) (&wcnt[0][0])[d] = (&mask[0][0])[d] = 0;
     if (tid == 0) s_tile = atomicAdd(ticket, 1u);
     __syncthreads();
     const uint32_t tile = s_tile;
@@ -229,10 +220,17 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
     for (int t = 0; t < ITEMS; t++) {
         const bool valid = wbase + t * 32 + lane < n;
         const uint32_t d = valid ? rs_digit<SRC>(k[t], v[t], shift, box_off, nbox) : 256u;
-        const unsigned peers = digit_peers(d);
-        const uint32_t before = d < 256u ? wcnt[w][d] : 0u;
+        // the lanes of the warp with the same digit leave their bits in the digit's mask (read
+        // and cleared before the next pairs): 3 instructions on shared memory, where a ballot
+        // per digit bit took about 30 on the ALU that bounded the pass
+        if (valid) atomicOr(&mask[w][d], 1u << lane);
         __syncwarp();
-        if (d < 256u && (peers & lt) == 0u) wcnt[w][d] = before + __popc(peers);
+        const uint32_t peers = valid ? mask[w][d] : 0u, before = valid ? wcnt[w][d] : 0u;
+        __syncwarp();
+        if (valid && (peers & lt) == 0u) {
+            wcnt[w][d] = before + __popc(peers);
+            mask[w][d] = 0u;
+        }
         __syncwarp();
         rk[t] = valid ? before + __popc(peers & lt) : 0xffffffffu;
     }

@@ -26,7 +26,7 @@ def _check(ctx, pos, mass, n_crit, n_leaf):
     assert np.array_equal(ctx.dump(greem.DUMP_GROUPS), t.groups())
 
 
-@pytest.mark.parametrize("n", [1, 31, 255, 257, 767, 769, 4095, 4096, 4097, 65537, 200000, 200001])
+@pytest.mark.parametrize("n", [1, 31, 255, 257, 767, 769, 4095, 4096, 4097, 65537, 200000, 200001, 204287, 204289])
 @pytest.mark.parametrize("n_crit,n_leaf", [(1, 1), (64, 10)])
 def test_tree_and_groups(n, n_crit, n_leaf):
     rng = np.random.default_rng(n)
