@@ -335,7 +335,7 @@ __device__ __forceinline__ void climb(const Node *__restrict__ nodes, uint32_t n
 }
 
 // Leaf moments by tiles of consecutive particles: a block takes the leaves that start in
-// its tile of kLeafTile sorted particles (the deepest node a particle owns is a leaf, so
+// its tile of TILE sorted particles (the deepest node a particle owns is a leaf, so
 // particle i starts leaf base[i+1] - 1 when it owns any node), stages the tile's
 // particles and a halo in shared memory with coalesced loads, and orders its leaves by
 // particle count, so that the lanes of a warp loop equally often (an FP64 warp
@@ -343,8 +343,13 @@ __device__ __forceinline__ void climb(const Node *__restrict__ nodes, uint32_t n
 // order, as a thread alone would.  Leaves reaching past the halo read the rest from
 // global memory.
 constexpr int kLeafTile = 1024;
+// the same where tiles of 1024 are fewer than two per SM: a block's FP64 sums take as long as
+// the kernel, so smaller tiles on more SMs are faster (tree stage at tiles of 1024 / 256: 4 k
+// particles 0.043 / 0.039 ms, 100 k 0.082 / 0.077, 262 k 0.092 / 0.090, 1 M 0.161 / 0.168)
+constexpr int kLeafTileSmall = 256;
 constexpr int kLeafHalo = 64;
 
+template <int TILE>
 __global__ void __launch_bounds__(256) k_moments_leaf_tiled(const Node *__restrict__ nodes,
                                                             const uint32_t *__restrict__ n_nodes, uint32_t node_cap,
                                                             const uint32_t *__restrict__ base, uint32_t N,
@@ -353,13 +358,13 @@ __global__ void __launch_bounds__(256) k_moments_leaf_tiled(const Node *__restri
                                                             const double *__restrict__ zs,
                                                             const float *__restrict__ ms, Dbl4 *__restrict__ raw)
 {
-    __shared__ double sx_[kLeafTile + kLeafHalo], sy_[kLeafTile + kLeafHalo], sz_[kLeafTile + kLeafHalo];
-    __shared__ float sm_[kLeafTile + kLeafHalo];
-    __shared__ uint32_t leaf_n[kLeafTile], leaf_b[kLeafTile], leaf_e[kLeafTile], order[kLeafTile];
+    __shared__ double sx_[TILE + kLeafHalo], sy_[TILE + kLeafHalo], sz_[TILE + kLeafHalo];
+    __shared__ float sm_[TILE + kLeafHalo];
+    __shared__ uint32_t leaf_n[TILE], leaf_b[TILE], leaf_e[TILE], order[TILE];
     __shared__ uint32_t cnt[33], start[33], nleaf;
     const uint32_t nn = node_count(n_nodes, node_cap);
-    const uint32_t p0 = blockIdx.x * kLeafTile;
-    const uint32_t pe = min(N, p0 + kLeafTile + kLeafHalo);
+    const uint32_t p0 = blockIdx.x * TILE;
+    const uint32_t pe = min(N, p0 + TILE + kLeafHalo);
     const int tid = threadIdx.x;
     if (tid < 33) cnt[tid] = 0;
     if (tid == 0) nleaf = 0;
@@ -371,7 +376,7 @@ __global__ void __launch_bounds__(256) k_moments_leaf_tiled(const Node *__restri
     }
     __syncthreads();
     // the leaves that start in the tile
-    const uint32_t pt = min(N, p0 + kLeafTile);
+    const uint32_t pt = min(N, p0 + TILE);
     for (uint32_t i = p0 + tid; i < pt; i += blockDim.x) {
         const uint32_t o0 = base[i], o1 = base[i + 1];
         if (o1 == o0) continue;
@@ -461,8 +466,9 @@ void launch_moments(const Node *nodes, const uint32_t *n_nodes, uint32_t node_ca
                     const uint32_t *base, uint32_t N, const double *xs, const double *ys, const double *zs,
                     const float *ms, Dbl4 *raw, uint32_t *pend, cudaStream_t s, int nsm)
 {
-    k_moments_leaf_tiled<<<(N + kLeafTile - 1) / kLeafTile, 256, 0, s>>>(nodes, n_nodes, node_cap, base, N, xs, ys,
-                                                                       zs, ms, raw);
+    const uint32_t tile = N <= 2u * (uint32_t)nsm * kLeafTile ? kLeafTileSmall : kLeafTile;
+    const auto leaf = tile == kLeafTile ? k_moments_leaf_tiled<kLeafTile> : k_moments_leaf_tiled<kLeafTileSmall>;
+    leaf<<<(N + tile - 1) / tile, 256, 0, s>>>(nodes, n_nodes, node_cap, base, N, xs, ys, zs, ms, raw);
     k_moments_up<<<climb_grid(node_cap, nsm), 32 * kClimbWarps, 0, s>>>(nodes, n_nodes, node_cap, pend, kids,
                                                                       reinterpret_cast<double *>(raw));
     g_launches += 2;

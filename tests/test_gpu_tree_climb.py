@@ -1,5 +1,6 @@
 """Moments and second moments of every level in one climb from the deepest nodes: shallow and
-deep trees of all sizes against sums over each node's particles."""
+deep trees of all sizes, on both sides of the line between the leaf pass's tiles, against
+sums over each node's particles."""
 import numpy as np
 import pytest
 
@@ -15,7 +16,8 @@ _build.build()
 from paper_0910_0121_gb300 import greem  # noqa: E402
 
 
-@pytest.mark.parametrize("n,depth", [(1, 0.1), (9, 1e-6), (4096, 0.1), (50000, 1e-6), (700000, 1e-4), (700001, 1e-4)])
+@pytest.mark.parametrize("n,depth", [(1, 0.1), (9, 1e-6), (257, 0.1), (4096, 0.1), (50000, 1e-6), (311296, 1e-3),
+                                     (311297, 1e-3), (700001, 1e-4)])
 def test_moments_of_every_node(n, depth):
     rng = np.random.default_rng(n)
     pos = rng.random((n, 3))
