@@ -484,8 +484,8 @@ static __device__ __forceinline__ void sort_mid_runs(uint64_t *__restrict__ key,
     }
 }
 
-// The middle runs, then the long ones, one block each: up to kRunCap pairs by a bitonic sort in shared memory
-// of (low bits << 14 | position in the run), unique keys whose order is the stable one;
+// The middle runs, then the long ones, one block each: up to cap pairs (kRunCap, or less
+// where the input is shorter) by a bitonic sort in shared memory of (low bits << 14 | position in the run), unique keys whose order is the stable one;
 // longer runs by one warp, three stable 9-bit LSD passes over the low 27 bits through the
 // other ping-pong buffer (tkey, tval) at the same positions, then copied back.
 __global__ void __launch_bounds__(kRunThreads) k_runs_rest(uint64_t *__restrict__ key, uint32_t *__restrict__ val,
@@ -495,12 +495,12 @@ __global__ void __launch_bounds__(kRunThreads) k_runs_rest(uint64_t *__restrict_
                                                            uint32_t *__restrict__ ctr,
                                                            const uint32_t *__restrict__ mid, uint32_t mid_cap_,
                                                            const uint32_t *__restrict__ n_mid,
-                                                           uint32_t *__restrict__ mid_ctr)
+                                                           uint32_t *__restrict__ mid_ctr, uint32_t cap)
 {
     sort_mid_runs(key, val, mid, mid_cap_, n_mid, mid_ctr);
     extern __shared__ __align__(16) unsigned char run_smem[];
     uint64_t *comp = reinterpret_cast<uint64_t *>(run_smem);
-    uint32_t *vals = reinterpret_cast<uint32_t *>(run_smem + (size_t)kRunCap * sizeof(uint64_t));
+    uint32_t *vals = reinterpret_cast<uint32_t *>(run_smem + (size_t)cap * sizeof(uint64_t));
     __shared__ uint32_t s_r;
     __shared__ uint64_t s_top;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(kRunThreads) k_runs_rest(uint64_t *__restrict_
         const uint32_t r = s_r;
         if (r >= nl) break;
         const uint32_t s = runs[2 * r], e = runs[2 * r + 1], len = e - s;
-        if (len <= (uint32_t)kRunCap) {
+        if (len <= cap) {
             uint32_t P = 1;
             while (P < len) P <<= 1;
             for (uint32_t j = tid; j < P; j += kRunThreads) {
@@ -649,8 +649,13 @@ void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t
     uint32_t *mid = runs + 2 * (size_t)runs_cap(n);
     k_runs_short<<<(n + 255) / 256, 256, 0, s>>>(ki, vi, n, box_off, nbox, runs, runs_cap(n), n_long, mid, mid_cap(n),
                                                   n_long + 2);
-    k_runs_rest<<<nsm * 2, kRunThreads, kRunSmem, s>>>(ki, vi, ko, vo, runs, runs_cap(n), n_long, n_long + 1, mid,
-                                                       mid_cap(n), n_long + 2, n_long + 3);
+    // no run is longer than the input: small calls ask for less shared memory and fewer blocks
+    // (sort stage of 4 k particles 0.0303 -> 0.0285 ms)
+    uint32_t cap = 512;  // at least the digit starts of the one-warp path
+    while (cap < (uint32_t)kRunCap && cap < n) cap *= 2;
+    const unsigned grid = std::min<unsigned>((n + 255) / 256, (unsigned)nsm * 2);
+    k_runs_rest<<<grid, kRunThreads, cap * (sizeof(uint64_t) + sizeof(uint32_t)), s>>>(
+        ki, vi, ko, vo, runs, runs_cap(n), n_long, n_long + 1, mid, mid_cap(n), n_long + 2, n_long + 3, cap);
     g_launches += 2;
     *k_out = ki;
     *v_out = vi;
