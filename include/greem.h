@@ -205,10 +205,11 @@ typedef struct greem_stats {
     int64_t kernel_launches;  /* kernels launched by the last call */
     int32_t l_min;            /* shallowest group level of box 0 */
     int32_t retries;          /* capacity retries of the last call */
-    /* with STAGE_TIMES, by events on the context's stream: keys; sort and gather; tree,
-     * moments and node COM offsets; groups (particle offsets and groups run on a second
-     * stream beside the moments: what remains of them after the moments, and the
-     * second-order moments); lists; force (and PM); total */
+    /* with STAGE_TIMES, by events on the context's stream: keys and the sort's digit counts;
+     * sort and gather; tree, moments and node COM offsets; groups (particle offsets, groups
+     * and the force kernel's work order run on a second stream beside the moments: what
+     * remains of them after the moments, and the second-order moments); lists; force (and
+     * PM); total */
     double ms_keys, ms_sort, ms_tree, ms_groups, ms_lists, ms_force, ms_total;
     /* list walks that started below the root, from the level-K cell table (Sec. 3.1.2
      * walk; the conditions under which the entries are the same are in lists.cu), and the
