@@ -273,6 +273,10 @@ int greem_debug_dump_group_lists(greem_ctx *ctx, const int64_t *groups, int64_t 
  *                             instead of the root (default 7; 0 or 1: every walk starts at
  *                             the root; value < 0 restores the default).  The lists hold the
  *                             same entries either way; for timing comparisons.  Stays in effect.
+ *   GREEM_DEBUG_LOOK_BACK     the prefix sums whose wait on earlier parts of the array gives up
+ *                             at once (default: after 2^22 polls), a sum of GREEM_LOOK_*: a call
+ *                             whose array has more than one part returns GREEM_ERR_TIMEOUT, and
+ *                             the context stays usable.  0 or less: none.  Stays in effect.
  * Every setting also drops the graph that repeated greem_short_force_ex calls replay.
  * Errors: INVALID_ARG (NULL ctx, unknown what, value out of range). */
 #define GREEM_DEBUG_WAIT_POLLS 0
@@ -282,6 +286,12 @@ int greem_debug_dump_group_lists(greem_ctx *ctx, const int64_t *groups, int64_t 
 #define GREEM_DEBUG_MAX_ATTEMPTS 4
 #define GREEM_DEBUG_START_LEVEL 5
 #define GREEM_DEBUG_REPLAY 6
+#define GREEM_DEBUG_LOOK_BACK 7
+#define GREEM_LOOK_SORT 1      /* a digit pass of the key sort */
+#define GREEM_LOOK_NODES 2     /* the node numbers */
+#define GREEM_LOOK_GROUPS 4    /* the group selection */
+#define GREEM_LOOK_SECOND 8    /* the places of the second-order lists */
+#define GREEM_LOOK_ALL 15
 int greem_debug_set(greem_ctx *ctx, int what, int64_t value);
 
 /* The FP32 list entries of selected groups exactly as the force kernel reads them, for

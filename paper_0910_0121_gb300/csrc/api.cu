@@ -71,7 +71,7 @@ struct greem_ctx {
     // S5-S6
     DBuf<float4> flist;
     DBuf<unsigned long long> ilist, loff;
-    DBuf<uint32_t> llen, lraw, kids, stack, order, bins, n_groups;
+    DBuf<uint32_t> llen, lraw, kids, stack, order, bins, n_nodes, n_groups;
     DBuf<uint32_t> tbl;   // the list walk's start tables (k_start_table)
     int tbl_kmax = 0;     // the deepest start level of the current call's boxes
     int start_cap = 7;    // the deepest level a list walk may start at (greem_debug_set)
@@ -96,6 +96,7 @@ struct greem_ctx {
     uint32_t next_stack_cap = 0;
     int max_attempts = 6;
     uint32_t wait_polls1 = 0;
+    unsigned look_back = 0;  // the look-backs that give up at once (GREEM_LOOK_*)
 
     // results of the last call
     uint64_t *ks = nullptr;
@@ -481,6 +482,7 @@ static int size_buffers(greem_ctx *c, const RunCfg &r)
         ENS(qlist, c->qcap * 3);
     }
     ENS(kids, nc * 8);
+    ENS(n_nodes, 1);
     ENS(n_groups, 1);
     ENS(bins, kBinWords);
     ENS(bps, (size_t)r.nbox);
@@ -600,6 +602,9 @@ static cudaEvent_t *stage_events(greem_ctx *c)
     return c->stage_ev;
 }
 
+// The limit of a look-back's waits (0: it gives up at once, a failure test).
+static uint32_t look_polls(const greem_ctx *c, unsigned which) { return (c->look_back & which) ? 0u : kWaitPolls; }
+
 static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
 {
     int rc = size_buffers(c, r);
@@ -622,7 +627,7 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     uint64_t *ks = nullptr;
     uint32_t *perm = nullptr;
     radix_sort(c->k0.p, c->k1.p, c->v0.p, c->v1.p, N, radix_key_passes(), box_passes, c->box_off.p, nbox, c->hist.p,
-               c->rs_status.p, c->rs_runs.p, c->st.p, &ks, &perm, s, nsm);
+               c->rs_status.p, c->rs_runs.p, c->st.p, &ks, &perm, s, nsm, look_polls(c, GREEM_LOOK_SORT));
     launch_gather(r.pos, r.mass, perm, N, c->box_off.p, nbox, c->bps.p, c->xs.p, c->ys.p, c->zs.p, c->ms.p, c->st.p,
                   s);
     ev_record(c, r, ev, 2);
@@ -634,9 +639,9 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     zt.p[2] = c->bins.p;
     zt.n[2] = kBinWords;
     launch_tree_prep(ks, N, c->box_off.p, nbox, c->bps.p, c->d8.p, c->K8.p, c->own.p, zt, s);
-    scan_u32(c->own.p, c->base.p, N, c->scratch.p, c->st.p, s, nullptr, true);
-    const uint32_t *n_nodes = c->base.p + N;
-    launch_tree_fill(ks, N, c->box_off.p, nbox, c->d8.p, c->K8.p, c->base.p, c->nodes.p, ncap, c->st.p, s, nsm);
+    scan_u32(c->own.p, c->base.p, N, c->scratch.p, c->st.p, s, nullptr, true, look_polls(c, GREEM_LOOK_NODES));
+    uint32_t *n_nodes = c->n_nodes.p;
+    launch_tree_fill(ks, N, c->box_off.p, nbox, c->d8.p, c->K8.p, c->base.p, c->nodes.p, ncap, n_nodes, c->st.p, s, nsm);
     launch_tree_links(c->nodes.p, n_nodes, ncap, c->kids.p, c->pend.p, s, nsm);
     // fork: the moments (FP64-bound) on s; the particle offsets and the groups (integer
     // work, reading only the tree) on the second stream
@@ -647,8 +652,8 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
                         c->pcell.p, s2);
     uint32_t *n_groups = c->n_groups.p;
     launch_group_select(c->nodes.p, n_nodes, ncap, c->box_off.p, nbox, c->bps.p, c->groups.p, n_groups, c->gstat.p,
-                        c->st.p, s2);
-    launch_group_box(c->groups.p, n_groups, c->pcell.p, c->gbox.p, s2, nsm);
+                        c->st.p, s2, look_polls(c, GREEM_LOOK_GROUPS));
+    launch_group_box(c->groups.p, n_groups, c->pcell.p, c->gbox.p, c->st.p, s2, nsm);
     launch_leaf_boxes(c->nodes.p, n_nodes, ncap, c->pcell.p, c->lbox.p, s2, nsm);
     if (r.lists_force) {
         launch_force_order(c->groups.p, n_groups, c->bps.p, c->bins.p, c->order.p, s2, nsm);
@@ -719,7 +724,8 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
         if (r.precision == GREEM_F64) launch_force_f64(fa, s, nsm);
         else launch_force_f32(fa, s, nsm, r.soft);
         if (r.quad) {
-            scan_u32(c->qcnt.p, c->qoff.p, ncap, c->scratch.p, c->st.p, s, n_groups);
+            scan_u32(c->qcnt.p, c->qoff.p, ncap, c->scratch.p, c->st.p, s, n_groups, false,
+                     look_polls(c, GREEM_LOOK_SECOND));
             fa.qoff = c->qoff.p;
             fa.qcnt = c->qcnt.p;
             fa.qlist = c->qlist.p;
@@ -973,7 +979,7 @@ void greem_destroy(greem_ctx *c)
     release(c->poff); release(c->pcell); release(c->lbox); release(c->irel); release(c->groups); release(c->gbox); release(c->quad);
     release(c->flist); release(c->ilist); release(c->loff);
     release(c->llen); release(c->lraw); release(c->kids); release(c->stack); release(c->order); release(c->bins);
-    release(c->n_groups); release(c->bps); release(c->box_off); release(c->small); release(c->st);
+    release(c->n_nodes); release(c->n_groups); release(c->bps); release(c->box_off); release(c->small); release(c->st);
     release(c->qlist); release(c->qcnt); release(c->qoff);
     release(c->dom_boxes); release(c->dom); release(c->dom_cnt); release(c->let_flag); release(c->let_cnt);
     release(c->let_ends); release(c->tbl);
@@ -1896,7 +1902,7 @@ int greem_let_export(greem_ctx *c, const int32_t *boxes, int ndom, int self, int
          (rc = ensure(c, c->let_ends, (size_t)kLetChunk + 1)) ||
          (rc = ensure(c, c->scratch, scan_scratch_elems(run * chunk + 1) + 64))))
         return rc;
-    const uint32_t *n_nodes = c->base.p + N;
+    const uint32_t *n_nodes = c->n_nodes.p;
     cudaStream_t s = c->stream;
     greem::g_launches = 0;
     int64_t run_items = 0;
@@ -1957,6 +1963,10 @@ int greem_debug_set(greem_ctx *c, int what, int64_t value)
     case GREEM_DEBUG_REPLAY:
         if (value < 0 || value > 1) return GREEM_ERR_INVALID_ARG;
         c->ag_enabled = value != 0;
+        return GREEM_OK;
+    case GREEM_DEBUG_LOOK_BACK:
+        if (value > GREEM_LOOK_ALL) return GREEM_ERR_INVALID_ARG;
+        c->look_back = value < 0 ? 0u : (unsigned)value;
         return GREEM_OK;
     default:
         return GREEM_ERR_INVALID_ARG;

@@ -192,22 +192,27 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
 // Single-pass prefix sums over tiles (decoupled look-back, Merrill & Garland 2016): the sum
 // over the tiles before `tile`, whose own sum is tot; status: one zeroed word per tile.  By
 // one whole warp, 32 predecessors at a time.  Tiles are taken by ticket, so a block waits
-// only on blocks that started before it; the wait is bounded (ST_TIMEOUT, and the sum is
-// then too small, never too large).
+// only on blocks that started before it; the wait is bounded: after `polls` of them
+// ST_TIMEOUT is set and the sum is too small, never too large (polls 0, a failure test:
+// every tile but the first gives up at once).  What such a sum numbers overlaps, and leaves
+// slots that nobody writes, so nothing may follow those numbers: the kernel after the scan
+// sets the count that later kernels go by to 0 (k_tree_fill for the nodes, k_group_box for
+// the groups), and the kernels that read single numbers look at the flag.
 constexpr unsigned long long kTileAgg = 1ull << 62, kTilePrefix = 2ull << 62;
-__device__ __forceinline__ uint32_t tile_prefix(unsigned long long *status, uint32_t tile, uint32_t tot, DevStatus *st)
+__device__ __forceinline__ uint32_t tile_prefix(unsigned long long *status, uint32_t tile, uint32_t tot, DevStatus *st,
+                                                uint32_t polls)
 {
     const int lane = threadIdx.x & 31;
     if (lane == 0) st_relaxed_u64(status + tile, (tile == 0 ? kTilePrefix : kTileAgg) | tot);
     if (tile == 0) return 0;
-    uint32_t excl = 0, polls = 0;
+    uint32_t excl = 0, polled = 0;
     for (long long j = (long long)tile - 1;;) {
         const unsigned long long w = j - lane >= 0 ? ld_relaxed_u64(status + (j - lane)) : kTilePrefix;
         const unsigned have = __ballot_sync(0xffffffffu, (w >> 62) != 0), pre = __ballot_sync(0xffffffffu, (w >> 62) == 2);
         const int last = pre ? __ffs(pre) - 1 : 31;  // the nearest published prefix, or the whole window
         const unsigned need = 0xffffffffu >> (31 - last);
-        if ((have & need) != need) {
-            if (++polls < kWaitPolls) continue;
+        if ((have & need) != need || polls == 0) {
+            if (++polled < polls) continue;
             if (lane == 0) atomicOr(&st->flags, ST_TIMEOUT);
             break;
         }
@@ -224,8 +229,9 @@ size_t scan_scratch_elems(size_t n);  // the first scan_zero_words(n) of them ar
 size_t scan_zero_words(size_t n);
 // out[0..n] = exclusive prefix sums of in[0..n), out[n] = total.  in may alias out.  n_dev:
 // the number of elements on the device (at most n), or null.  zeroed: the scratch is zero.
+// polls: tile_prefix's limit.
 void scan_u32(const uint32_t *in, uint32_t *out, size_t n, uint32_t *scratch, DevStatus *st, cudaStream_t s,
-              const uint32_t *n_dev = nullptr, bool zeroed = false);
+              const uint32_t *n_dev = nullptr, bool zeroed = false, uint32_t polls = kWaitPolls);
 
 // S1-S2 (keys_sort.cu)
 void launch_keys(const double *pos, uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps,
@@ -238,7 +244,7 @@ size_t radix_runs_elems(uint32_t n);
 int radix_key_passes();
 void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t n, int key_passes, int box_passes,
                 const uint32_t *box_off, int nbox, uint32_t *hist, unsigned long long *status, uint32_t *runs,
-                DevStatus *st, uint64_t **k_out, uint32_t **v_out, cudaStream_t s, int nsm);
+                DevStatus *st, uint64_t **k_out, uint32_t **v_out, cudaStream_t s, int nsm, uint32_t polls);
 void launch_gather(const double *pos, const float *mass, const uint32_t *perm, uint32_t N, const uint32_t *box_off,
                    int nbox, const BoxPar *bps, double *xs, double *ys, double *zs, float *ms, DevStatus *st,
                    cudaStream_t s);
@@ -247,8 +253,8 @@ void launch_gather(const double *pos, const float *mass, const uint32_t *perm, u
 void launch_tree_prep(const uint64_t *keys, uint32_t N, const uint32_t *box_off, int nbox, const BoxPar *bps,
                       uint8_t *d8, uint8_t *K8, uint32_t *own, const ZeroList &zero, cudaStream_t s);
 void launch_tree_fill(const uint64_t *keys, uint32_t N, const uint32_t *box_off, int nbox, const uint8_t *d8,
-                      const uint8_t *K8, const uint32_t *base, Node *nodes, uint32_t node_cap, DevStatus *st,
-                      cudaStream_t s, int nsm);
+                      const uint8_t *K8, const uint32_t *base, Node *nodes, uint32_t node_cap, uint32_t *n_nodes,
+                      DevStatus *st, cudaStream_t s, int nsm);
 void launch_tree_links(Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, uint32_t *kids, uint32_t *pend,
                        cudaStream_t s, int nsm);
 void launch_moments(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *kids,
@@ -268,9 +274,9 @@ void launch_node_finish(const Node *nodes, const uint32_t *n_nodes, uint32_t nod
 size_t group_status_words(size_t node_cap);
 void launch_group_select(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *box_off, int nbox,
                          const BoxPar *bps, Group *groups, uint32_t *n_groups, uint32_t *status, DevStatus *st,
-                         cudaStream_t s);
-void launch_group_box(const Group *groups, const uint32_t *n_groups, const unsigned long long *pcell, int4 *gbox,
-                      cudaStream_t s, int nsm);
+                         cudaStream_t s, uint32_t polls);
+void launch_group_box(const Group *groups, uint32_t *n_groups, const unsigned long long *pcell, int4 *gbox,
+                      const DevStatus *st, cudaStream_t s, int nsm);
 // S5 (lists.cu)
 struct ListArgs {
     const Node *nodes;

@@ -671,8 +671,8 @@ __global__ void __launch_bounds__(GREEM_FORCE_THREADS, GREEM_FORCE_MINB) k_force
     __syncwarp();
     if (a.st->flags & ST_NODE_CAP) return;  // the tree was truncated: the call is retried
     // the quadrupole lists are incomplete (and would be read past their end): the call is
-    // retried with larger lists
-    if (QUAD && (a.st->flags & (ST_LIST_CAP | ST_QLIST_CAP))) return;
+    // retried with larger lists; or a wait gave up (the scan that places them)
+    if (QUAD && (a.st->flags & (ST_LIST_CAP | ST_QLIST_CAP | ST_TIMEOUT))) return;
     const uint32_t G = *a.n_groups;
     const uint32_t share = CAP ? (uint32_t)a.share : 0u, others = (1u << share) - 1u;
     for (;;) {
@@ -760,7 +760,7 @@ __global__ void __launch_bounds__(256) k_qlist_fill(ForceArgs a, const float4 *_
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    if (a.st->flags & (ST_NODE_CAP | ST_LIST_CAP)) return;
+    if (a.st->flags & (ST_NODE_CAP | ST_LIST_CAP | ST_TIMEOUT)) return;
     const uint32_t G = *a.n_groups;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned long long need = a.qoff[G];

@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
                                                              uint32_t n, int shift, const uint32_t *__restrict__ counts,
                                                              unsigned long long *status, uint32_t *ticket,
                                                              const uint32_t *__restrict__ box_off, int nbox,
-                                                             DevStatus *st)
+                                                             DevStatus *st, uint32_t polls)
 {
     constexpr uint32_t TILE = kRsThreads * ITEMS;  // pairs per tile
     extern __shared__ __align__(16) unsigned char rs_buf[];
@@ -198,10 +198,13 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
     __shared__ uint32_t lstart[256];
     __shared__ uint32_t gbase[256];
     __shared__ uint32_t wsum[kRsWarps], dsum[kRsWarps];
-    __shared__ uint32_t s_tile;
+    __shared__ uint32_t s_tile, s_flags;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     for (int d = tid; d < kRsWarps * 256; d += kRsThreads) (&wcnt[0][0])[d] = (&mask[0][0])[d] = 0;
-    if (tid == 0) s_tile = atomicAdd(ticket, 1u);
+    if (tid == 0) {
+        s_tile = atomicAdd(ticket, 1u);
+        s_flags = st->flags;
+    }
     __syncthreads();
     const uint32_t tile = s_tile;
 
@@ -295,7 +298,8 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
         // or a tile that has not published yet (wait for it, then go on from there)
         unsigned long long excl = 0;
         int j = (int)tile - 1;
-        bool done = false, timeout = false;
+        bool done = false, timeout = polls == 0;  // 0: a failure test
+        if (timeout) atomicOr(&st->flags, ST_TIMEOUT);
         while (!done && !timeout) {
             unsigned long long sw[kRsLook];
 #pragma unroll
@@ -317,7 +321,7 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
                 const unsigned long long *w8 = status + (size_t)j * 256 + tid;
                 uint32_t it = 0;
                 while ((ld_relaxed_u64(w8) >> 62) == 0ull) {
-                    if (++it >= kWaitPolls) {
+                    if (++it >= polls) {
                         atomicOr(&st->flags, ST_TIMEOUT);
                         timeout = true;
                         break;
@@ -331,7 +335,9 @@ __global__ void __launch_bounds__(kRsThreads, GREEM_RS_MINB) k_rs_onesweep(const
     }
     __syncthreads();
     const uint32_t tbase = tile * TILE;
-    const uint32_t cnt = min(TILE, n - tbase);
+    // after an earlier pass that gave up the keys are not those that were counted, and the
+    // digits' places could lie past the end
+    const uint32_t cnt = (s_flags & ST_TIMEOUT) ? 0u : min(TILE, n - tbase);
     for (uint32_t j = tid; j < cnt; j += kRsThreads) {
         const uint64_t kk = sk[j];
         const uint32_t vv = sv[j];
@@ -382,12 +388,14 @@ static __device__ __noinline__ void sort_short_run(uint64_t *__restrict__ key, u
 // to kShortRun pairs itself and lists a longer one, its end found by binary search (the
 // top bits are sorted within a box): up to kWarpRun pairs (mid, n_mid), more
 // (runs, n_long): both for k_runs_rest.  Other threads only read the top bits of pairs that
-// runs permute among themselves, so the concurrent sorts do not disturb them.
+// runs permute among themselves, so the concurrent sorts do not disturb them.  Without the
+// order of the top bits (a pass gave up) nothing is sorted or listed.
 __global__ void __launch_bounds__(256) k_runs_short(uint64_t *__restrict__ key, uint32_t *__restrict__ val, uint32_t n,
                                                     const uint32_t *__restrict__ box_off, int nbox,
                                                     uint32_t *__restrict__ runs, uint32_t run_cap,
                                                     uint32_t *__restrict__ n_long, uint32_t *__restrict__ mid,
-                                                    uint32_t mid_cap_, uint32_t *__restrict__ n_mid)
+                                                    uint32_t mid_cap_, uint32_t *__restrict__ n_mid,
+                                                    const DevStatus *__restrict__ st)
 {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -400,6 +408,7 @@ __global__ void __launch_bounds__(256) k_runs_short(uint64_t *__restrict__ key, 
         if (box_off[b] == i) head = true;
     }
     if (!head || i + 1 >= e_box || run_top(key[i + 1]) != t) return;  // not a head, or a run of one
+    if (st->flags & ST_TIMEOUT) return;
     uint32_t e = i + 2;
     while (e < e_box && e - i <= (uint32_t)kShortRun && run_top(key[e]) == t) e++;
     if (e - i <= (uint32_t)kShortRun) {
@@ -606,7 +615,7 @@ __global__ void __launch_bounds__(kRunThreads) k_runs_rest(uint64_t *__restrict_
 // k_keys has counted the digits (hist) and zeroed the rest of hist and the status words.
 void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t n, int key_passes, int box_passes,
                 const uint32_t *box_off, int nbox, uint32_t *hist, unsigned long long *status, uint32_t *runs,
-                DevStatus *st, uint64_t **k_out, uint32_t **v_out, cudaStream_t s, int nsm)
+                DevStatus *st, uint64_t **k_out, uint32_t **v_out, cudaStream_t s, int nsm, uint32_t polls)
 {
     // the shared-memory opt-in applies to the current device only: set once per device
     static std::atomic<bool> attr_set[kMaxDevices];
@@ -633,7 +642,8 @@ void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t
         const bool small = rs_items(n) == kRsItemsSmall;
         const auto kern = boxp ? (small ? k_rs_onesweep<1, kRsItemsSmall> : k_rs_onesweep<1, kRsItems>)
                                : (small ? k_rs_onesweep<0, kRsItemsSmall> : k_rs_onesweep<0, kRsItems>);
-        kern<<<ntile, kRsThreads, rs_smem(rs_items(n)), s>>>(ki, vi, ko, vo, n, shift, ds, sw, tk, box_off, nbox, st);
+        kern<<<ntile, kRsThreads, rs_smem(rs_items(n)), s>>>(ki, vi, ko, vo, n, shift, ds, sw, tk, box_off, nbox, st,
+                                                             polls);
         g_launches++;
         // ping-pong
         uint64_t *kt = ki;
@@ -648,7 +658,7 @@ void radix_sort(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, uint32_t
     uint32_t *n_long = hist + kRsMaxPasses * 256 + kRsMaxPasses;  // n_long, long work, n_mid, mid work
     uint32_t *mid = runs + 2 * (size_t)runs_cap(n);
     k_runs_short<<<(n + 255) / 256, 256, 0, s>>>(ki, vi, n, box_off, nbox, runs, runs_cap(n), n_long, mid, mid_cap(n),
-                                                  n_long + 2);
+                                                  n_long + 2, st);
     // no run is longer than the input: small calls ask for less shared memory and fewer blocks
     // (sort stage of 4 k particles 0.0303 -> 0.0285 ms)
     uint32_t cap = 512;  // at least the digit starts of the one-warp path
@@ -671,7 +681,7 @@ __global__ void __launch_bounds__(256) k_gather(const double *__restrict__ pos, 
 {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    uint32_t j = perm[i];
+    const uint32_t j = min(perm[i], N - 1);  // (a sort that gave up leaves any value)
     double L = bps[box_of(i, box_off, nbox)].L;
     xs[i] = wrap_pos_fast(pos[3 * (size_t)j], L);
     ys[i] = wrap_pos_fast(pos[3 * (size_t)j + 1], L);

@@ -175,7 +175,8 @@ __global__ void __launch_bounds__(256) k_start_table(const Node *__restrict__ no
                                                      const BoxPar *__restrict__ bps, int nbox,
                                                      uint32_t *__restrict__ tbl, const DevStatus *__restrict__ st)
 {
-    if (st->flags & ST_NODE_CAP) return;  // the tree is incomplete; the lists are not walked
+    // the tree is incomplete, or there is none after a wait that gave up: no list is walked
+    if (st->flags & (ST_NODE_CAP | ST_TIMEOUT)) return;
     for (int b = blockIdx.y; b < nbox; b += gridDim.y) {
         const BoxPar &bp = bps[b];
         const int K = bp.kstart;

@@ -49,7 +49,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *t
 
 // Each thread owns kScanItems consecutive elements.
 __global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t *in, size_t n, const uint32_t *__restrict__ n_dev,
-                                                       uint32_t *out, uint32_t *scratch, DevStatus *st)
+                                                       uint32_t *out, uint32_t *scratch, DevStatus *st, uint32_t polls)
 {
     __shared__ uint32_t s_tile, s_excl;
     if (threadIdx.x == 0) s_tile = atomicAdd(scratch, 1u);
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t *in, size_
     uint32_t tot;
     uint32_t run = block_exclusive_scan(s, &tot);
     if (threadIdx.x < 32) {
-        const uint32_t excl = tile_prefix(reinterpret_cast<unsigned long long *>(scratch + 2), tile, tot, st);
+        const uint32_t excl = tile_prefix(reinterpret_cast<unsigned long long *>(scratch + 2), tile, tot, st, polls);
         if (threadIdx.x == 0) s_excl = excl;
     }
     __syncthreads();
@@ -106,11 +106,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t *in, size_
 }
 
 void scan_u32(const uint32_t *in, uint32_t *out, size_t n, uint32_t *scratch, DevStatus *st, cudaStream_t s,
-              const uint32_t *n_dev, bool zeroed)
+              const uint32_t *n_dev, bool zeroed, uint32_t polls)
 {
     if (!zeroed) cudaMemsetAsync(scratch, 0, scan_zero_words(n) * sizeof(uint32_t), s);
     const unsigned nb = (unsigned)std::max<size_t>(1, ceil_div(n, kScanTile));
-    k_scan<<<nb, kScanThreads, 0, s>>>(in, n, n_dev, out, scratch, st);
+    k_scan<<<nb, kScanThreads, 0, s>>>(in, n, n_dev, out, scratch, st, polls);
     g_launches++;
 }
 

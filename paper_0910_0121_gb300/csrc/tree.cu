@@ -161,12 +161,14 @@ __device__ __forceinline__ void fill_nodes(const uint64_t *__restrict__ keys, ui
 
 // About one particle in five owns nodes.  Each warp queues the owners among its 32
 // particles in shared memory and fills nodes 32 owners at a time, so that every lane of
-// a filling warp has an owner's galloping searches to run.
+// a filling warp has an owner's galloping searches to run.  *n_nodes gets the number of
+// nodes; 0 after a sort or a scan that gave up, whose nodes are wrong (and written in bounds
+// all the same), so that no later kernel looks at one.
 __global__ void __launch_bounds__(256) k_tree_fill(const uint64_t *__restrict__ keys, uint32_t N,
                                                    const uint32_t *__restrict__ box_off, int nbox,
                                                    const uint8_t *__restrict__ d8, const uint8_t *__restrict__ K8,
                                                    const uint32_t *__restrict__ base, Node *__restrict__ nodes,
-                                                   uint32_t node_cap, DevStatus *st)
+                                                   uint32_t node_cap, uint32_t *__restrict__ n_nodes, DevStatus *st)
 {
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ uint32_t queue[8][64];
@@ -180,7 +182,10 @@ __global__ void __launch_bounds__(256) k_tree_fill(const uint64_t *__restrict__ 
         bool owner = false;
         if (i < N) {
             owner = base[i + 1] > base[i];
-            if (i == N - 1 && base[N] > node_cap) atomicOr(&st->flags, ST_NODE_CAP);
+            if (i == N - 1) {
+                *n_nodes = (st->flags & ST_TIMEOUT) ? 0u : base[N];
+                if (base[N] > node_cap) atomicOr(&st->flags, ST_NODE_CAP);
+            }
         }
         const unsigned m = __ballot_sync(FULL, owner);
         if (owner) q[qn + __popc(m & lt)] = i;
@@ -202,11 +207,11 @@ __global__ void __launch_bounds__(256) k_tree_fill(const uint64_t *__restrict__ 
 }
 
 void launch_tree_fill(const uint64_t *keys, uint32_t N, const uint32_t *box_off, int nbox, const uint8_t *d8,
-                      const uint8_t *K8, const uint32_t *base, Node *nodes, uint32_t node_cap, DevStatus *st,
-                      cudaStream_t s, int nsm)
+                      const uint8_t *K8, const uint32_t *base, Node *nodes, uint32_t node_cap, uint32_t *n_nodes,
+                      DevStatus *st, cudaStream_t s, int nsm)
 {
     const unsigned grid = (unsigned)std::min<size_t>((N + 255) / 256, (size_t)nsm * 8);
-    k_tree_fill<<<grid, 256, 0, s>>>(keys, N, box_off, nbox, d8, K8, base, nodes, node_cap, st);
+    k_tree_fill<<<grid, 256, 0, s>>>(keys, N, box_off, nbox, d8, K8, base, nodes, node_cap, n_nodes, st);
     g_launches++;
 }
 
@@ -732,7 +737,8 @@ __global__ void __launch_bounds__(256) k_group_select(const Node *__restrict__ n
                                                       const uint32_t *__restrict__ n_nodes, uint32_t node_cap,
                                                       const uint32_t *__restrict__ box_off, int nbox,
                                                       const BoxPar *__restrict__ bps, Group *__restrict__ groups,
-                                                      uint32_t *__restrict__ n_groups, uint32_t *status, DevStatus *st)
+                                                      uint32_t *__restrict__ n_groups, uint32_t *status, DevStatus *st,
+                                                      uint32_t polls)
 {
     __shared__ uint32_t s_tile, s_excl, wcnt[8 * kSelItems];
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
@@ -766,7 +772,7 @@ __global__ void __launch_bounds__(256) k_group_select(const Node *__restrict__ n
         }
         wcnt[tid] = x - v;
         const uint32_t tot = __shfl_sync(0xffffffffu, x, 31);
-        const uint32_t excl = tile_prefix(reinterpret_cast<unsigned long long *>(status + 2), tile, tot, st);
+        const uint32_t excl = tile_prefix(reinterpret_cast<unsigned long long *>(status + 2), tile, tot, st, polls);
         if (tid == 0) {
             s_excl = excl;
             if (nn - n0 <= kSelTile) {  // the last tile
@@ -800,24 +806,29 @@ __global__ void __launch_bounds__(256) k_group_select(const Node *__restrict__ n
 
 void launch_group_select(const Node *nodes, const uint32_t *n_nodes, uint32_t node_cap, const uint32_t *box_off, int nbox,
                          const BoxPar *bps, Group *groups, uint32_t *n_groups, uint32_t *status, DevStatus *st,
-                         cudaStream_t s)
+                         cudaStream_t s, uint32_t polls)
 {
     k_group_select<<<(node_cap + kSelTile - 1) / kSelTile, 256, 0, s>>>(nodes, n_nodes, node_cap, box_off, nbox, bps,
-                                                                        groups, n_groups, status, st);
+                                                                        groups, n_groups, status, st, polls);
     g_launches++;
 }
 
 // The box of finest-level cells that holds a group's particles, one warp per group:
 // centre minus the group's cell centre and half sides, in u (cells lo..hi span
 // [2 lo, 2 hi + 2]).  The list builder prunes against it (Eq. 2 vanishes beyond r_cut).
-__global__ void __launch_bounds__(256) k_group_box(const Group *__restrict__ groups,
-                                                   const uint32_t *__restrict__ n_groups,
+// The first kernel after the group selection: if that gave up, it leaves no groups.
+__global__ void __launch_bounds__(256) k_group_box(const Group *__restrict__ groups, uint32_t *n_groups,
                                                    const unsigned long long *__restrict__ pcell,
-                                                   int4 *__restrict__ gbox)
+                                                   int4 *__restrict__ gbox, const DevStatus *st)
 {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
+    const unsigned flags = st->flags;  // (not volatile: thousands of warps past the L1 cache took 1.5 us)
     const uint32_t G = *n_groups;
+    if (flags & ST_TIMEOUT) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *n_groups = 0;
+        return;
+    }
     const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
     for (uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < G; g += nw) {
         const Group gr = groups[g];
@@ -847,10 +858,10 @@ __global__ void __launch_bounds__(256) k_group_box(const Group *__restrict__ gro
     }
 }
 
-void launch_group_box(const Group *groups, const uint32_t *n_groups, const unsigned long long *pcell, int4 *gbox,
-                      cudaStream_t s, int nsm)
+void launch_group_box(const Group *groups, uint32_t *n_groups, const unsigned long long *pcell, int4 *gbox,
+                      const DevStatus *st, cudaStream_t s, int nsm)
 {
-    k_group_box<<<nsm * 8, 256, 0, s>>>(groups, n_groups, pcell, gbox);
+    k_group_box<<<nsm * 8, 256, 0, s>>>(groups, n_groups, pcell, gbox, st);
     g_launches++;
 }
 
