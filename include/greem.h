@@ -291,7 +291,9 @@ int greem_debug_dump_group_lists(greem_ctx *ctx, const int64_t *groups, int64_t 
 #define GREEM_LOOK_NODES 2     /* the node numbers */
 #define GREEM_LOOK_GROUPS 4    /* the group selection */
 #define GREEM_LOOK_SECOND 8    /* the places of the second-order lists */
-#define GREEM_LOOK_ALL 15
+#define GREEM_LOOK_DOMAIN 16   /* the places of greem_domain_pack */
+#define GREEM_LOOK_LET 32      /* the places of greem_let_export */
+#define GREEM_LOOK_ALL 63
 int greem_debug_set(greem_ctx *ctx, int what, int64_t value);
 
 /* The FP32 list entries of selected groups exactly as the force kernel reads them, for
@@ -389,7 +391,8 @@ int greem_cell_index(greem_ctx *ctx, const double *pos, int64_t N, double L, con
  * particles of domain 0, then 1, ..., each in input order (stable); counts (HOST int64
  * [ndom]) gets the number per domain.  All arrays but boxes and counts are DEVICE, N rows,
  * owned by the caller.  Waits for the stream.  Errors: INVALID_ARG (bad sizes, boxes out of
- * range, a particle in no box or with a NaN/Inf coordinate), CUDA, OOM. */
+ * range, a particle in no box or with a NaN/Inf coordinate), CUDA, OOM, TIMEOUT (nothing is
+ * written). */
 int greem_domain_pack(greem_ctx *ctx, const double *pos, const float *mass, const int64_t *ids, int64_t N, double L,
                       const int32_t *boxes, int ndom, int64_t *counts, double *pos_out, float *mass_out,
                       int64_t *ids_out);
@@ -411,7 +414,7 @@ int greem_domain_pack(greem_ctx *ctx, const double *pos, const float *mass, cons
  * theta = 0 no node is accepted and the items are exactly the particles within r_cut.
  * Waits for the stream.  Errors: INVALID_ARG (no tree, a multi-box call, bad boxes,
  * self >= ndom), CAPACITY (*total > cap: nothing past cap is written; call again with
- * cap >= *total), CUDA, OOM. */
+ * cap >= *total), CUDA, OOM, TIMEOUT (counts and items are incomplete). */
 int greem_let_export(greem_ctx *ctx, const int32_t *boxes, int ndom, int self, int64_t *counts, double *pos_out,
                      float *mass_out, int64_t *ref_out, int64_t cap, int64_t *total);
 

@@ -1852,8 +1852,10 @@ int greem_domain_pack(greem_ctx *c, const double *pos, const float *mass, const 
         !cuda_ok(cudaMemcpyAsync(c->dom_boxes.p, boxes, sizeof(int32_t) * 6 * ndom, cudaMemcpyHostToDevice, s)))
         return GREEM_ERR_CUDA;
     launch_dom_count(pos, n, L, bp.pow2_e, c->dom_boxes.p, ndom, c->dom.p, c->dom_cnt.p, c->st.p, s);
-    scan_u32(c->dom_cnt.p, c->dom_cnt.p, ncnt, c->scratch.p, c->st.p, s);
-    launch_dom_scatter(pos, mass, ids, n, L, c->dom.p, c->dom_cnt.p, ndom, pos_out, mass_out, ids_out, s);
+    scan_u32(c->dom_cnt.p, c->dom_cnt.p, ncnt, c->scratch.p, c->st.p, s, nullptr, false,
+             look_polls(c, GREEM_LOOK_DOMAIN));
+    launch_dom_scatter(pos, mass, ids, n, L, c->dom.p, c->dom_cnt.p, ndom, pos_out, mass_out, ids_out, c->st.p,
+                       s);
     std::vector<uint32_t> off(ncnt + 1);
     unsigned flags = 0;
     if (!cuda_ok(cudaGetLastError()) ||
@@ -1863,6 +1865,7 @@ int greem_domain_pack(greem_ctx *c, const double *pos, const float *mass, const 
         return GREEM_ERR_CUDA;
     c->stats.kernel_launches = greem::g_launches;
     if (flags & ST_NONFINITE) return GREEM_ERR_INVALID_ARG;
+    if (flags & ST_TIMEOUT) return GREEM_ERR_TIMEOUT;
     for (int d = 0; d < ndom; d++) counts[d] = (int64_t)off[(size_t)(d + 1) * nblk] - (int64_t)off[(size_t)d * nblk];
     return GREEM_OK;
 }
@@ -1899,7 +1902,7 @@ int greem_let_export(greem_ctx *c, const int32_t *boxes, int ndom, int self, int
     int rc;
     if (chunk > 0 &&
         ((rc = ensure(c, c->let_flag, ncap)) || (rc = ensure(c, c->let_cnt, run * chunk + 1)) ||
-         (rc = ensure(c, c->let_ends, (size_t)kLetChunk + 1)) ||
+         (rc = ensure(c, c->let_ends, (size_t)kLetChunk + 2)) ||
          (rc = ensure(c, c->scratch, scan_scratch_elems(run * chunk + 1) + 64))))
         return rc;
     const uint32_t *n_nodes = c->n_nodes.p;
@@ -1909,14 +1912,16 @@ int greem_let_export(greem_ctx *c, const int32_t *boxes, int ndom, int self, int
     for (int j0 = 0; j0 < nrecv; j0 += kLetChunk) {
         const int nb = std::min(kLetChunk, nrecv - j0);
         launch_let_count(c->nodes.p, n_nodes, ncap, lb.data() + j0, nb, c->bps.p, c->pcell.p, c->let_flag.p,
-                         c->let_cnt.p, s, c->nsm);
-        scan_u32(c->let_cnt.p, c->let_cnt.p, run * nb, c->scratch.p, c->st.p, s);
-        launch_let_ends(c->let_cnt.p, ncap, nb, c->let_ends.p, s);
-        uint32_t ends[kLetChunk + 1];
+                         c->let_cnt.p, c->st.p, s, c->nsm);
+        scan_u32(c->let_cnt.p, c->let_cnt.p, run * nb, c->scratch.p, c->st.p, s, nullptr, false,
+                 look_polls(c, GREEM_LOOK_LET));
+        launch_let_ends(c->let_cnt.p, ncap, nb, c->let_ends.p, c->st.p, s);
+        uint32_t ends[kLetChunk + 2];
         if (!cuda_ok(cudaGetLastError()) ||
-            !cuda_ok(cudaMemcpyAsync(ends, c->let_ends.p, sizeof(uint32_t) * (nb + 1), cudaMemcpyDeviceToHost, s)) ||
+            !cuda_ok(cudaMemcpyAsync(ends, c->let_ends.p, sizeof(uint32_t) * (nb + 2), cudaMemcpyDeviceToHost, s)) ||
             !cuda_ok(cudaStreamSynchronize(s)))
             return GREEM_ERR_CUDA;
+        if (ends[nb + 1] & ST_TIMEOUT) return GREEM_ERR_TIMEOUT;  // the places are wrong: nothing is filled
         for (int j = 0; j < nb; j++) counts[recv[j0 + j]] = (int64_t)ends[j + 1] - (int64_t)ends[j];
         const int64_t tot = ends[nb];
         if (run_items + tot <= cap && tot)

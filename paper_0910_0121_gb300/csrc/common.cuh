@@ -377,11 +377,11 @@ void launch_dom_count(const double *pos, uint32_t N, double L, int pow2_e, const
                       uint32_t *dom, uint32_t *cnt, DevStatus *st, cudaStream_t s);
 void launch_dom_scatter(const double *pos, const float *mass, const int64_t *ids, uint32_t N, double L,
                         const uint32_t *dom, const uint32_t *off, int ndom, double *pos_out, float *mass_out,
-                        int64_t *ids_out, cudaStream_t s);
+                        int64_t *ids_out, const DevStatus *st, cudaStream_t s);
 void launch_let_count(const Node *nodes, const uint32_t *n_nodes, uint32_t ncap, const LetBox *b, int nb,
-                      const BoxPar *bps, const unsigned long long *pcell, uint32_t *flag, uint32_t *cnt, cudaStream_t s,
-                      int nsm);
-void launch_let_ends(const uint32_t *off, uint32_t ncap, int nb, uint32_t *ends, cudaStream_t s);
+                      const BoxPar *bps, const unsigned long long *pcell, uint32_t *flag, uint32_t *cnt, DevStatus *st,
+                      cudaStream_t s, int nsm);
+void launch_let_ends(const uint32_t *off, uint32_t ncap, int nb, uint32_t *ends, const DevStatus *st, cudaStream_t s);
 void launch_let_fill(const Node *nodes, const uint32_t *n_nodes, uint32_t ncap, const LetBox *b, int nb,
                      const BoxPar *bps, const unsigned long long *pcell, const uint32_t *flag, const uint32_t *off,
                      const double *xs, const double *ys, const double *zs, const float *ms, const Dbl4 *mom64,

@@ -107,14 +107,15 @@ __global__ void __launch_bounds__(kDomThreads) k_dom_count(const double *__restr
 // Stable scatter by domain: off is the exclusive scan of cnt (domain-major), so domain
 // d's particles of block b start at off[d * nblk + b]; within a block, warps go in
 // order and lanes rank among equal domains by their position.  Positions are written
-// wrapped into [0, L).
+// wrapped into [0, L).  Nothing is written after a scan that gave up.
 __global__ void __launch_bounds__(kDomThreads) k_dom_scatter(const double *__restrict__ pos,
                                                             const float *__restrict__ mass,
                                                             const int64_t *__restrict__ ids, uint32_t N, double L,
                                                             const uint32_t *__restrict__ dom,
                                                             const uint32_t *__restrict__ off, int ndom,
                                                             double *__restrict__ pos_out, float *__restrict__ mass_out,
-                                                            int64_t *__restrict__ ids_out)
+                                                            int64_t *__restrict__ ids_out,
+                                                            const DevStatus *__restrict__ st)
 {
     extern __shared__ uint32_t wcnt[];  // [kDomWarps][ndom]
     const unsigned FULL = 0xffffffffu;
@@ -123,12 +124,13 @@ __global__ void __launch_bounds__(kDomThreads) k_dom_scatter(const double *__res
     __syncthreads();
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     const bool v = i < N;
+    const unsigned flags = st->flags;
     const uint32_t d = v ? dom[i] : 0xffffffffu;
     const unsigned peers = __match_any_sync(FULL, d);
     const uint32_t rank = (uint32_t)__popc(peers & ((1u << lane) - 1u));
     if (v && rank == 0) wcnt[w * ndom + d] = (uint32_t)__popc(peers);
     __syncthreads();
-    if (!v) return;
+    if (!v || (flags & ST_TIMEOUT)) return;
     uint32_t dst = off[(size_t)d * gridDim.x + blockIdx.x] + rank;
     for (int ww = 0; ww < w; ww++) dst += wcnt[ww * ndom + d];
     pos_out[3 * (size_t)dst] = wrap_pos_fast(pos[3 * (size_t)i], L);
@@ -152,10 +154,10 @@ void launch_dom_count(const double *pos, uint32_t N, double L, int pow2_e, const
 
 void launch_dom_scatter(const double *pos, const float *mass, const int64_t *ids, uint32_t N, double L,
                         const uint32_t *dom, const uint32_t *off, int ndom, double *pos_out, float *mass_out,
-                        int64_t *ids_out, cudaStream_t s)
+                        int64_t *ids_out, const DevStatus *st, cudaStream_t s)
 {
     k_dom_scatter<<<dom_blocks(N), kDomThreads, dom_scatter_smem(ndom), s>>>(pos, mass, ids, N, L, dom, off, ndom,
-                                                                              pos_out, mass_out, ids_out);
+                                                                              pos_out, mass_out, ids_out, st);
     g_launches++;
 }
 
@@ -210,7 +212,8 @@ __device__ __forceinline__ bool let_particle_in(unsigned long long pc, const Let
 }
 
 // Up to kLetChunk receiving boxes are handled by one set of passes: a node's status for
-// box j sits in bits 2j..2j+1 of its flag word.
+// box j sits in bits 2j..2j+1 of its flag word.  k_let_flags clears the status flags for the
+// scan of the counts, whose word for the host k_let_ends brings along.
 struct LetBoxes {
     LetBox b[kLetChunk];
     int n;
@@ -218,8 +221,9 @@ struct LetBoxes {
 
 __global__ void __launch_bounds__(256) k_let_flags(const Node *__restrict__ nodes, const uint32_t *__restrict__ n_nodes,
                                                    uint32_t ncap, LetBoxes bx, const BoxPar *__restrict__ bps,
-                                                   uint32_t *__restrict__ flag)
+                                                   uint32_t *__restrict__ flag, DevStatus *st)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->flags = 0;
     const uint32_t nn = min(*n_nodes, ncap);
     const BoxPar &bp = bps[0];
     for (uint32_t n = blockIdx.x * blockDim.x + threadIdx.x; n < nn; n += gridDim.x * blockDim.x) {
@@ -316,28 +320,32 @@ __global__ void __launch_bounds__(256) k_let_fill(const Node *__restrict__ nodes
     }
 }
 
-// The offsets at the ends of the boxes' runs: ends[j] = off[(j + 1) * (ncap + 1) - 1 + 1].
-__global__ void k_let_ends(const uint32_t *__restrict__ off, uint32_t ncap, int nb, uint32_t *__restrict__ ends)
+// The offsets at the ends of the boxes' runs: ends[j] = off[j * (ncap + 1)], j = 0 .. nb, and
+// the status flags in ends[nb + 1].
+__global__ void k_let_ends(const uint32_t *__restrict__ off, uint32_t ncap, int nb, uint32_t *__restrict__ ends,
+                           const DevStatus *__restrict__ st)
 {
     const int j = threadIdx.x;
     if (j <= nb) ends[j] = off[(size_t)j * ((size_t)ncap + 1)];
+    if (j == nb + 1) ends[j] = st->flags;
 }
 
 void launch_let_count(const Node *nodes, const uint32_t *n_nodes, uint32_t ncap, const LetBox *b, int nb,
-                      const BoxPar *bps, const unsigned long long *pcell, uint32_t *flag, uint32_t *cnt, cudaStream_t s,
-                      int nsm)
+                      const BoxPar *bps, const unsigned long long *pcell, uint32_t *flag, uint32_t *cnt, DevStatus *st,
+                      cudaStream_t s, int nsm)
 {
     LetBoxes bx;
     bx.n = nb;
     for (int j = 0; j < nb; j++) bx.b[j] = b[j];
-    k_let_flags<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, ncap, bx, bps, flag);
+    k_let_flags<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, ncap, bx, bps, flag, st);
     k_let_count<<<nsm * 8, 256, 0, s>>>(nodes, n_nodes, ncap, flag, pcell, bx, bps, cnt);
     g_launches += 2;
 }
 
-void launch_let_ends(const uint32_t *off, uint32_t ncap, int nb, uint32_t *ends, cudaStream_t s)
+void launch_let_ends(const uint32_t *off, uint32_t ncap, int nb, uint32_t *ends, const DevStatus *st, cudaStream_t s)
 {
-    k_let_ends<<<1, 32, 0, s>>>(off, ncap, nb, ends);
+    static_assert(kLetChunk + 2 <= 32, "one warp");
+    k_let_ends<<<1, 32, 0, s>>>(off, ncap, nb, ends, st);
     g_launches++;
 }
 

@@ -35,7 +35,8 @@ ASSIGN_TSC = 1
 
 DEBUG_WAIT_POLLS, DEBUG_NODE_CAP, DEBUG_LIST_CAP, DEBUG_STACK_CAP, DEBUG_MAX_ATTEMPTS, DEBUG_START_LEVEL, \
     DEBUG_REPLAY, DEBUG_LOOK_BACK = range(8)
-LOOK_SORT, LOOK_NODES, LOOK_GROUPS, LOOK_SECOND = 1, 2, 4, 8  # DEBUG_LOOK_BACK's bits
+# DEBUG_LOOK_BACK's bits
+LOOK_SORT, LOOK_NODES, LOOK_GROUPS, LOOK_SECOND, LOOK_DOMAIN, LOOK_LET = 1, 2, 4, 8, 16, 32
 
 DUMP_KEYS, DUMP_PERM, DUMP_NODES, DUMP_MOMENTS, DUMP_GROUPS, DUMP_LIST_OFFSETS, DUMP_LISTS, DUMP_QUADRUPOLES = range(8)
 

@@ -55,6 +55,30 @@ def test_a_look_back_that_gives_up(n, n_crit, which):
     ctx.close()
 
 
+@pytest.mark.parametrize("grid", [(2, 1, 1), (5, 2, 2)])  # one and two chunks of receiving boxes
+def test_domain_calls_report_a_sum_that_gave_up(grid):
+    n = 600000  # more than one tile of counts per call
+    P, M = _set(n, 5)
+    ctx = greem.Context()
+    cells = ctx.cell_index(P[:2000].contiguous(), 1.0).cpu().numpy()
+    boxes = greem.domain_boxes(cells, grid)
+    pack = lambda: ctx.domain_pack(P, M, None, 1.0, boxes)  # noqa: E731
+    let = lambda: ctx.let_export(boxes, 0, with_refs=True)  # noqa: E731
+    ctx.build_tree(P, M, greem.params(L=1.0, r_cut=0.04, theta=0.5))
+    ref_let = let()
+    ctx.debug_set(greem.DEBUG_LOOK_BACK, greem.LOOK_LET)
+    _timeout(let)
+    ctx.debug_set(greem.DEBUG_LOOK_BACK, greem.LOOK_DOMAIN)
+    again = let()
+    _timeout(pack)
+    ctx.debug_set(greem.DEBUG_LOOK_BACK, 0)
+    assert all(torch.equal(a, b) for a, b in zip(ref_let[:3], again[:3])) and np.array_equal(ref_let[3], again[3])
+    po, mo, io, counts = pack()
+    assert counts.sum() == n and torch.equal(io.sort().values, torch.arange(n, device="cuda"))
+    assert torch.equal(po, P[io]) and torch.equal(mo, M[io])
+    ctx.close()
+
+
 def test_bad_masks_are_refused():
     ctx = greem.Context()
     with pytest.raises(greem.GreemError) as e:
