@@ -303,7 +303,8 @@ __device__ __forceinline__ bool take_cells(const ListArgs &a, Team<W> &team, boo
 }
 
 // What a walk needs of its group, in shared memory: 64 bytes per warp, read by broadcast
-// where a test needs them.  Held in registers they would spill others: the walker keeps 32
+// where a test needs them (the memory clobber keeps the loads behind the stores of the next
+// group's words).  Held in registers they would spill others: the walker keeps 32
 // warps per SM at 64 registers (spills 268 -> 80 bytes; with the one scan per step and the
 // one copy of the walk: 1.120 / 3.204 / 5.94 -> 1.034 / 3.045 / 5.46 ms).
 //   0: cell centre and half side (u)        1: particle box centre minus cell centre; first particle
@@ -311,7 +312,7 @@ __device__ __forceinline__ bool take_cells(const ListArgs &a, Team<W> &team, boo
 __device__ __forceinline__ int4 group_word(uint32_t gsm, int k)
 {
     int4 v;
-    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(gsm + 16u * k));
+    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(gsm + 16u * k) : "memory");
     return v;
 }
 __device__ __forceinline__ long long word_tprune(const int4 w)
