@@ -800,8 +800,11 @@ static void grow_caps(greem_ctx *c)
     if (h.flags & ST_QLIST_CAP) c->qcap = std::max<size_t>(c->qcap * 2, (size_t)(h.sum_quad * 1.25) + 4096);
     if (h.flags & ST_STACK) c->stack_cap *= 4;
     if (h.flags & ST_LIST_CAP) {
-        // every allocation abandons less than the list that did not fit, and every warp
-        // holds at most one partly used page
+        // a warp leaves room behind when a list did not fit (less than that list) and before a
+        // walk (at most half of its lists in all), and ends with part of its last pages (a
+        // page and a mean list at most): 3.5 sum_padded + a page per warp in the worst case.
+        // Twice the sum holds all but lists of very unequal lengths; those take another
+        // retry or two, each with half as much again.
         const size_t warps = (size_t)c->nsm * kListBlocksPerSM * kListWarps;
         const size_t need = (size_t)(2.0 * (double)h.sum_padded) + warps * c->page;
         c->list_cap = std::max<size_t>(c->list_cap + c->list_cap / 2, need);

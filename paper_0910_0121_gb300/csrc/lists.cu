@@ -29,11 +29,14 @@
 //
 // Lists are contiguous per group inside pages handed out by an atomic counter; a list
 // that does not fit the warp's current page is walked again into fresh pages.  A second
-// walk costs as much as the first, so a warp takes a fresh page before the walk when the
-// room left is below its mean list length so far (and always before its first group: a
-// warp of a small call walks one or two groups in all).  List stage before and after, one
+// walk costs as much as the first, so a warp takes fresh pages for a mean list before the walk
+// when the room left is below its mean list length so far (and a page before its first
+// group: a warp of a small call walks one or two groups in all).  It leaves at most half as
+// much room behind that way as its lists take (the bound on the pool is in grow_caps); past
+// that it walks into the room there is.  List stage before and after, one
 // GB300: 4 k particles 0.096 -> 0.053 ms, 100 k 0.197 -> 0.107, 300 k 0.287 -> 0.176, 128^3
-// halo mix 1.200 -> 1.177.
+// halo mix 1.200 -> 1.177.  With a single page whatever the mean, 20000 lists of 6200 entries
+// took 8.20 ms and three pages each; 5.11 ms and two.
 //
 // The walk may start below the root.  Let K be a level at or above the first level at
 // which any node can be accepted: with the group's particle box inside its cell, a node of
@@ -151,7 +154,7 @@ constexpr uint32_t kMaxStartCells = 512;       // more candidate cells: walk fro
 
 // A list warp's counters, kept in shared memory by its lane 0 and added to the status
 // word once, when the warp runs out of groups.
-enum { kTallyPadded, kTallyLen, kTallyInter, kTallyStart, kTallyGroups, kTallyN };
+enum { kTallyPadded, kTallyLen, kTallyInter, kTallyStart, kTallyGroups, kTallyLeft, kTallyN };
 
 // A 10-bit integer's bits spread to every third bit (Morton interleave).
 __device__ __forceinline__ uint32_t spread_bits3(uint32_t v)
@@ -712,9 +715,13 @@ __device__ __forceinline__ void build_lists(const ListArgs &a, ListShared &sm, u
             w[3] = make_int4((int)(uint32_t)Tp, (int)(uint32_t)(Tp >> 32), __float_as_int(bp.k_f), bp.lmin);
         }
         const uint32_t root = a.base[bp.p_begin];
-        if (!exhausted && (page_cur == page_end ||
-                           (page_end - page_cur) * tally[kTallyGroups] < tally[kTallyPadded]))
-            take_pages(1);
+        const uint32_t left = (uint32_t)(page_end - page_cur);
+        const float sum = (float)tally[kTallyPadded], ng = (float)tally[kTallyGroups];
+        if (!exhausted && (left == 0 || ((float)left * ng < sum && 2.0f * (float)(tally[kTallyLeft] + left) <= sum))) {
+            // one page more than the whole pages of a mean list
+            take_pages(1u + (uint32_t)__fdividef(sum, fmaxf(ng, 1.0f) * (float)a.page));
+            if (first) tally[kTallyLeft] += left;
+        }
         team.sync();
         uint32_t nacc = 0, len = 0, padded = 0;
         bool placed = false;
