@@ -811,6 +811,23 @@ static void grow_caps(greem_ctx *c)
     }
 }
 
+// The pages that the warps of the list builder hold at a time: one each, but no more than
+// there are groups, which number about 4 n / n_crit and are at least as deep as l_min.  Twice
+// that is assumed, and a call that has more groups still finds its room in the 32 entries a
+// particle or takes a retry.  A call of one particle has a pool of 66 KB and one of 4 k
+// particles 40 MB, where a page for every warp is 319 MB.
+static size_t held_pages(const greem_ctx *c, int nbox)
+{
+    const size_t warps = (size_t)c->nsm * kListBlocksPerSM * kListWarps;
+    size_t groups = 0;
+    for (int b = 0; b < nbox && groups < warps; b++) {
+        const BoxPar &bp = c->bps_host[b];
+        const size_t n = bp.p_end - bp.p_begin, cells = (size_t)1 << std::min(3 * bp.lmin, 32);
+        groups += std::min(n, 8 * n / (size_t)bp.n_crit + cells + 1);
+    }
+    return std::min(warps, groups);
+}
+
 static int run(greem_ctx *c, RunCfg r)
 {
     c->have_tree = c->have_lists = c->have_index = c->have_quad = false;
@@ -821,9 +838,8 @@ static int run(greem_ctx *c, RunCfg r)
     uint32_t pg = choose_page(r.N, c->nsm);
     if (pg > c->page) c->page = pg;
     if (r.lists_force) {
-        const size_t warps = (size_t)c->nsm * kListBlocksPerSM * kListWarps;
         if (c->next_list_cap) c->list_cap = c->next_list_cap;
-        else c->list_cap = std::max<size_t>(c->list_cap, (size_t)r.N * 32 + warps * c->page);
+        else c->list_cap = std::max<size_t>(c->list_cap, (size_t)r.N * 32 + held_pages(c, r.nbox) * c->page);
         // accepted nodes are a minority of the entries: a first guess of 4 per particle
         if (r.quad) c->qcap = std::max<size_t>(c->qcap, (size_t)r.N * 4 + 4096);
     }

@@ -1,0 +1,45 @@
+"""The list pool of small calls: pages for the groups there can be, not for every warp of the
+GPU, and no retry for it; a larger call of the same context grows it."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_0910_0121_gb300 import build as _build  # noqa: E402
+
+_build.build()
+from paper_0910_0121_gb300 import greem  # noqa: E402
+
+PAGE = 4096
+
+
+def _set(n, clustered):
+    rng = np.random.default_rng(n)
+    pos = rng.random((n, 3))
+    if clustered:
+        pos[: n // 2] = np.mod(0.2 + 0.01 * rng.standard_normal((n // 2, 3)), 1.0)
+    return torch.from_numpy(pos).cuda(), torch.ones(n, dtype=torch.float32, device="cuda")
+
+
+@pytest.mark.parametrize("clustered", [False, True])
+@pytest.mark.parametrize("n,n_crit,theta", [(1, 64, 0.5), (1000, 1, 0.5), (4096, 64, 0.5), (4096, 64, 0.0), (8192, 64, 0.5)])
+def test_pool_of_small_calls(n, n_crit, theta, clustered):
+    warps = 32 * torch.cuda.get_device_properties(0).multi_processor_count
+    p = greem.params(L=1.0, r_cut=0.15, theta=theta, n_crit=n_crit)
+    ctx = greem.Context()
+    ref = ctx.short_force(*_set(n, clustered), p)
+    st = ctx.stats()
+    assert st["retries"] == 0
+    assert st["list_capacity"] <= 32 * n + PAGE * min(n, 8 * n // n_crit + 8 ** st["l_min"] + 1) < 2048 * warps
+    big = _set(100000, clustered)
+    acc = ctx.short_force(*big, p)
+    assert ctx.stats()["list_capacity"] >= 32 * 100000 + PAGE * warps
+    assert torch.equal(ctx.short_force(*_set(n, clustered), p), ref)
+    other = greem.Context()
+    assert torch.equal(other.short_force(*big, p), acc)
+    other.close()
+    ctx.close()
