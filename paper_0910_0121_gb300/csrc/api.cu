@@ -108,8 +108,8 @@ struct greem_ctx {
 
     // PM
     PmPlan pm;
-    DBuf<float> pm_grid, pm_table;
-    DBuf<cufftComplex> pm_spec, pm_tmp;
+    DBuf<float> pm_table;
+    DBuf<cufftComplex> pm_tmp;
     DBuf<float4> pm_field;
     int pm_tab_n = 0, pm_tab_scheme = -1;
     double pm_tab_L = 0, pm_tab_rc = 0;
@@ -364,9 +364,9 @@ static int check_common(const greem_params &p)
 static int pm_prepare(greem_ctx *c, int n, double L, double r_cut, int scheme)
 {
     int rc;
-    const size_t cells = (size_t)n * n * n, half = (size_t)n * n * (n / 2 + 1), h = (size_t)(n / 2 + 1);
-    if ((rc = ensure(c, c->pm_grid, cells)) || (rc = ensure(c, c->pm_spec, half)) ||
-        (rc = ensure(c, c->pm_tmp, 3 * pm_plane(n))) || (rc = ensure(c, c->pm_table, h * h * h)) ||
+    const size_t cells = (size_t)n * n * n, h = (size_t)(n / 2 + 1);
+    // 28 bytes a grid point, the table aside
+    if ((rc = ensure(c, c->pm_tmp, 3 * pm_plane(n))) || (rc = ensure(c, c->pm_table, h * h * h)) ||
         (rc = ensure(c, c->pm_field, cells)))
         return rc;
     if (!(c->pm.have && c->pm.n == n)) {
@@ -737,8 +737,8 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
             if ((rc = pm_prepare(c, r.n_pm, b0.L, 2.0 * b0.eta, r.assign))) return rc;
             // input order: Morton-sorted particles of dense halos make consecutive lanes hit the
             // same cells and serialise the assignment atomics
-            if (run_pm(c->pm, r.pos, r.mass, N, b0.L, r.n_pm, r.assign, b0.pow2_e, c->pm_table.p, c->pm_grid.p,
-                       c->pm_spec.p, c->pm_tmp.p, c->pm_field.p, (float *)r.acc, 1, s, nsm))
+            if (run_pm(c->pm, r.pos, r.mass, N, b0.L, r.n_pm, r.assign, b0.pow2_e, c->pm_table.p, c->pm_tmp.p,
+                       c->pm_field.p, (float *)r.acc, 1, s, nsm))
                 return GREEM_ERR_CUDA;
         }
         ev_record(c, r, ev, 6);
@@ -974,7 +974,7 @@ void greem_destroy(greem_ctx *c)
     for (auto &e : c->stage_ev)
         if (e) cudaEventDestroy(e);
     pm_plan_destroy(c->pm);
-    release(c->pm_grid); release(c->pm_table); release(c->pm_spec); release(c->pm_tmp); release(c->pm_field);
+    release(c->pm_table); release(c->pm_tmp); release(c->pm_field);
     if (c->own_stream) cudaStreamDestroy(c->own_stream);
     for (cudaStream_t hs : {c->h2d, c->d2h})
         if (hs) {
@@ -1255,8 +1255,8 @@ int greem_pm_force(greem_ctx *c, const double *pos, const float *mass, int64_t N
     int rc = pm_prepare(c, n_pm, L, r_cut, assign);
     if (rc) return rc;
     greem::g_launches = 0;
-    if (run_pm(c->pm, pos, mass, (uint32_t)N, L, n_pm, assign, pow2_exponent(L), c->pm_table.p, c->pm_grid.p,
-               c->pm_spec.p, c->pm_tmp.p, c->pm_field.p, acc_pm, 0, c->stream, c->nsm))
+    if (run_pm(c->pm, pos, mass, (uint32_t)N, L, n_pm, assign, pow2_exponent(L), c->pm_table.p, c->pm_tmp.p,
+               c->pm_field.p, acc_pm, 0, c->stream, c->nsm))
         return GREEM_ERR_CUDA;
     if (!cuda_ok(cudaGetLastError()) || !cuda_ok(cudaStreamSynchronize(c->stream))) return GREEM_ERR_CUDA;
     c->stats.kernel_launches = greem::g_launches;

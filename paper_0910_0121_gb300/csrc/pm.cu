@@ -318,11 +318,12 @@ void launch_pm_table(int n, double L, double r_cut, int scheme, float *table, cu
     g_launches++;
 }
 
-// The whole PM force: grid n^3 floats, spec n*n*(n/2+1) complex, tmp 3 pm_plane(n)
-// complex, field n^3 float4, table from launch_pm_table.  acc gets (or accumulates) input order.
+// The whole PM force: tmp 3 pm_plane(n) complex, field n^3 float4, table from
+// launch_pm_table.  acc gets (or accumulates) input order.  The density and its spectrum are
+// done with when the field is made, and lie in its buffer: 4 n^3 bytes, then 8 n^2 (n/2+1)
+// from a multiple of 256 on, less than 16 n^3 for n >= 8.
 int run_pm(const PmPlan &pl, const double *pos, const float *mass, uint32_t N, double L, int n, int scheme, int pow2_e,
-           const float *table, float *grid, cufftComplex *spec, cufftComplex *tmp, float4 *field, float *acc,
-           int accumulate, cudaStream_t s, int nsm)
+           const float *table, cufftComplex *tmp, float4 *field, float *acc, int accumulate, cudaStream_t s, int nsm)
 {
     PmGeom g;
     g.n = n;
@@ -335,6 +336,8 @@ int run_pm(const PmPlan &pl, const double *pos, const float *mass, uint32_t N, d
         if ((1 << q) == n) lg = q;
     g.log2n = lg;
     const size_t cells = (size_t)n * n * n, plane = pm_plane(n);
+    float *grid = reinterpret_cast<float *>(field);
+    cufftComplex *spec = reinterpret_cast<cufftComplex *>(grid + (cells + 63) / 64 * 64);
     cudaMemsetAsync(grid, 0, cells * sizeof(float), s);
     const unsigned pb = (N + 255) / 256;
     if (scheme == 0) k_pm_assign<0><<<pb, 256, 0, s>>>(pos, mass, N, g, grid);

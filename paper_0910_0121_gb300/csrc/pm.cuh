@@ -15,6 +15,5 @@ void pm_plan_destroy(PmPlan &pl);
 // Complex values from one component's spectrum to the next (whole cache lines).
 inline size_t pm_plane(int n) { return ((size_t)n * n * (n / 2 + 1) + 31) / 32 * 32; }
 int run_pm(const PmPlan &pl, const double *pos, const float *mass, uint32_t N, double L, int n, int scheme, int pow2_e,
-           const float *table, float *grid, cufftComplex *spec, cufftComplex *tmp, float4 *field, float *acc,
-           int accumulate, cudaStream_t s, int nsm);
+           const float *table, cufftComplex *tmp, float4 *field, float *acc, int accumulate, cudaStream_t s, int nsm);
 }  // namespace greem
