@@ -240,7 +240,7 @@ __global__ void k_pm_table(int n, double L, double eta, int scheme, float *__res
 }
 
 // The three spectra -i k_c phi_k, phi_k = rho_k G, on the half-complex spectrum
-// [n][n][n/2+1] (the Nyquist component of each k_c is zero): one read of rho_k and G for
+// [n][n][n/2+1] (the Nyquist component of each k_c, mode n/2 of an even n, is zero): one read of rho_k and G for
 // what took a pass for phi and one per component (256^3 mesh: 0.128 -> 0.046 ms).
 __global__ void __launch_bounds__(256) k_pm_fields(const cufftComplex *__restrict__ rho, int n, double L,
                                                    const float *__restrict__ table, cufftComplex *__restrict__ out,
@@ -257,9 +257,8 @@ __global__ void __launch_bounds__(256) k_pm_fields(const cufftComplex *__restric
         cufftComplex v = rho[t];
         v.x *= gk;
         v.y *= gk;
-        auto sided = [n](int m) { return m < n / 2 ? m : (m == n / 2 ? 0 : m - n); };
-        const float kx = twopi_L * (float)sided(x), ky = twopi_L * (float)sided(y),
-                    kz = twopi_L * (float)(z == n / 2 ? 0 : z);
+        auto sided = [n](int m) { return 2 * m < n ? m : (2 * m == n ? 0 : m - n); };
+        const float kx = twopi_L * (float)sided(x), ky = twopi_L * (float)sided(y), kz = twopi_L * (float)sided(z);
         out[t] = make_cuFloatComplex(kx * v.y, -kx * v.x);
         out[plane + t] = make_cuFloatComplex(ky * v.y, -ky * v.x);
         out[2 * plane + t] = make_cuFloatComplex(kz * v.y, -kz * v.x);
