@@ -34,6 +34,7 @@
 #include <atomic>
 
 #include "common.cuh"
+#include "rsqrt64.cuh"
 
 namespace greem {
 
@@ -1003,30 +1004,12 @@ void launch_force_f32(const ForceArgs &a, cudaStream_t s, int nsm, bool soft, bo
 // else is free: tests are made on the high words, a lane's pair out of range is masked by
 // integer selects, whole warps skip what none of their lanes needs (the rest of a pair
 // when all 32 are beyond r_cut, the u term when none is within r_cut/2), and the square
-// root starts from the FP32 unit.  Per pair 7 instructions for xi^2, 5 for w = 1/xi and 13
+// root starts from the FP32 unit (rsqrt64.cuh).  Per pair 7 instructions for xi^2, 5 for w = 1/xi and 13
 // for the force with the cancellation-free form of Eq. 2 in units of 32/35 (the FP32
 // kernel's), 8 more with the u term; the plain form took about 62 (rsqrt(), divisions by
 // constants, FP64 compares).  64^3 halo mix, force stage: 24.0 -> 11.0 ms, 9.5 with the
 // capped passes below.  Against an 80-bit sum (4096 particles, theta 0) the median error is
 // 2.44e-16 (2.54e-16 before), the 99th percentile 3.3e-15 (3.4e-15).
-//
-// 1/sqrt(x): x = m 2^2q with m in [1, 4), the FP32 approximation y0 of 1/sqrt(m) (2^-22)
-// times 2^-q, and one third-order Householder step, y = y0 + y0 e (1/2 + 3/8 e), e = 1 - x
-// y0^2.  (5/16) e^3 is below 2^-64, y0^2 is exact (24 bits squared) and e exact to 2^-75,
-// which leaves the last rounding.
-__device__ __forceinline__ double rsqrt_fp64(double x)
-{
-    const int hi = __double2hiint(x);
-    if (hi < 0x00100000) return rsqrt(x);  // subnormal
-    const int ex = hi >> 20, odd = (ex & 1) ^ 1;
-    const int mb = ((127 + odd) << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)__double2loint(x) >> 29);
-    const int yb = __float_as_int(rsqrtf(__int_as_float(mb)));
-    const int q = (ex - 1023 - odd) >> 1;
-    const double y0 = __hiloint2double((yb >> 3) + 0x38000000 - (q << 20), (int)((unsigned)yb << 29));
-    const double e = fma(-x, y0 * y0, 1.0);
-    return fma(y0 * e, fma(e, 0.375, 0.5), y0);
-}
-
 template <int I, bool SOFT>
 __device__ __noinline__ void group_pass_f64(const ForceArgs &a, const Group &gr, const BoxPar &bp, uint32_t done,
                                             int S, unsigned long long lo, uint32_t len, Dbl4 *jb, int lane)
