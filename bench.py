@@ -4,7 +4,8 @@ One step = one call of greem_short_force_ex over the whole particle set: keys, r
 sort, tree + moments, groups, interaction lists and the FP32 force (S1-S6), inputs
 resident in HBM.  Workload: 256^3 particles (Zel'dovich P(k) ~ k^-2 grid, rms 0.5
 spacing, plus 5000 NFW halos), L = 1, r_cut = 3/256, theta = 0.5, n_leaf = 10, n_crit
-autotuned (untimed, before the warm-up).  Inputs (470 MB) are larger than the 129 MB L2.
+autotuned (untimed, before the warm-up; SETTING, which the reference arm names too, where it
+takes at most 1% longer).  Inputs (470 MB) are larger than the 129 MB L2.
 
 The e2e figure runs the same steps through greem_short_force_host: each step copies its
 inputs in from pinned host memory and its result out, the copies overlapping the
@@ -38,6 +39,10 @@ WORKLOAD = "zeldovich256+5000nfw_theta0.5"
 # FP32 flops credited per interaction (FMA = 2): 3 subtractions, 5 for r^2, 1 for r, 1 for R,
 # 12 for the inner polynomial of Eq. 2, 10 for its (R-1)^6 correction, 4 for m g / r^3, 6 to accumulate
 FLOPS_PER_INTERACTION = 42
+# The setting both arms time: several n_crit are within 0.4% of the best at 256^3 (96 / 128 /
+# 160 / 192 / 256: 16.30 / 16.10 / 16.04 / 16.10 / 16.26 ms), and the autotuner's pick among
+# them is timing noise
+SETTING = {"n_crit": 192, "list_chunk": 256, "block_shape": 16}
 SM_COUNT_NOMINAL = 152
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0
@@ -212,8 +217,7 @@ def reference_arm(args, rank, world):
     from paper_0910_0121_gb300 import synth
     pos, mass, prm = synth.config_zel256()
     N = len(pos)
-    # the n_crit the GPU arm's autotuner settles on for this workload (its config line)
-    n_crit = args.n_crit or 192
+    n_crit = args.n_crit or SETTING["n_crit"]
     times, walls, trees = [], [], []
     nth, ns, G = 1, 0, 0
     for k in range(args.warmup + args.steps):
@@ -235,12 +239,32 @@ def reference_arm(args, rank, world):
             "scaling": "strong", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "impl": "reference",
             "config": {"workload": WORKLOAD, "N": N, "L": 1.0, "r_cut": prm["r_cut"], "theta": prm["theta"],
-                       "n_crit": n_crit, "n_leaf": 10, "list_chunk": 256, "block_shape": 16,
+                       "n_crit": n_crit, "n_leaf": 10, "list_chunk": SETTING["list_chunk"],
+                       "block_shape": SETTING["block_shape"],
                        "l2": "inputs (470 MB) larger than L2, no flush", "parallelism": "domains 1x1x1"},
             "cpu_baseline": {"value": v, "unit": "particles/s", "cores": nth, "kind": "oracle", "sample": desc},
             "projected": True, "sample_wall_ms_per_step": 1e3 * statistics.mean(walls),
             "e2e": {"value": v, "unit": "particles/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
     print(json.dumps(line), flush=True)
+
+
+def settle(ctx, P, M, acc, pick):
+    """The autotuner's pick, or SETTING where it takes at most 1% longer."""
+    import torch
+    from paper_0910_0121_gb300 import greem
+    fixed = greem.params(L=pick.L, r_cut=pick.r_cut, theta=pick.theta, n_leaf=pick.n_leaf, **SETTING)
+    best = []
+    for p in (pick, fixed):
+        times = []
+        for _ in range(6):  # the first sizes the buffers
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ctx.short_force(P, M, p, acc)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        best.append(min(times[1:]))
+    return fixed if best[1] <= 1.01 * best[0] else pick
 
 
 def traffic_per_launch(list_entries):
@@ -707,8 +731,8 @@ def domain_arm(args, rank, world, local):
     stream = torch.cuda.current_stream()
     ctx = greem.Context(stream)
     comp = CountingCompute(ctx)
-    fprm = dict(L=prm["L"], r_cut=prm["r_cut"], theta=prm["theta"], n_crit=args.n_crit or 192, n_leaf=10,
-                list_chunk=256, block_shape=16)
+    fprm = dict(L=prm["L"], r_cut=prm["r_cut"], theta=prm["theta"], n_crit=args.n_crit or SETTING["n_crit"], n_leaf=10,
+                list_chunk=SETTING["list_chunk"], block_shape=SETTING["block_shape"])
     step = domain.DomainStep(comm, comp, fprm, grid, rate=4e-4, alpha=0.2, seed=synth.SEED0)
     P, M, I = step.decompose(P, M, I, N)       # by particle count
     step.force(P, M)
@@ -755,7 +779,8 @@ def domain_arm(args, rank, world, local):
         "warmup": max(3, args.warmup), "ms_per_step": ms, "higher_is_better": True, "scaling": "strong",
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": WORKLOAD, "N": N, "L": 1.0, "r_cut": fprm["r_cut"], "theta": fprm["theta"],
-                   "n_crit": fprm["n_crit"], "n_leaf": 10, "list_chunk": 256, "block_shape": 16,
+                   "n_crit": fprm["n_crit"], "n_leaf": 10, "list_chunk": fprm["list_chunk"],
+                   "block_shape": fprm["block_shape"],
                    "l2": "inputs (470 MB) larger than L2, no flush",
                    "parallelism": f"domains {grid[0]}x{grid[1]}x{grid[2]}",
                    "dist_backend": args.dist_backend},
@@ -804,7 +829,7 @@ def gpu_arm(args, rank, world, local):
     if args.n_crit:
         best = greem.params(L=prm["L"], r_cut=prm["r_cut"], theta=prm["theta"], n_crit=args.n_crit, n_leaf=10)
     else:
-        best = ctx.autotune(P, M, base, acc, candidates=[48, 64, 96, 128, 192, 256])
+        best = settle(ctx, P, M, acc, ctx.autotune(P, M, base, acc, candidates=[48, 64, 96, 128, 192, 256]))
     p = greem.params(L=best.L, r_cut=best.r_cut, theta=best.theta, n_crit=best.n_crit, n_leaf=best.n_leaf,
                      list_chunk=best.list_chunk, block_shape=best.block_shape, flags=greem.FLAG_STAGE_TIMES)
 
