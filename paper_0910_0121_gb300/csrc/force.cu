@@ -915,8 +915,10 @@ size_t force_smem_bytes(int chunk, int warps)
 // warp) 0.053 / 0.026 / 0.037 / 0.053 ms; 32^3 uniform (0.8) 0.088 / 0.055 / 0.051 / 0.067;
 // 100 k halo particles, n_crit 128 (1.3) 0.342 / 0.137 / 0.129 / 0.184; 300 k, n_crit 96
 // (5.1) 0.336 / - / 0.276 / 0.268; 1 M, n_crit 128, with the second-order pass (12.8) 1.57 /
-// - / 1.74 / 1.46; at cap 64 1.49.  At n_crit 64 a cap of 32 splits only the largest groups
-// in two and gains nothing.
+// - / 1.74 / 1.46; at cap 64 1.49.  The last line and the one at n_crit 64 were drawn on one
+// side only; on the other a cap of 32 is the faster one as well (halo sets, uncapped / 32):
+// n_crit 128, 1.2 M (16) 1.08 / 1.00, 2.1 M (27) 1.72 / 1.58; 192, 3.2 M (27) 2.75 / 2.57; 256,
+// 3.1 M (20) 2.87 / 2.78; n_crit 64, 156 k (4) 0.180 / 0.150, 506 k (13) 0.421 / 0.395.
 static double box_groups(uint32_t n, int n_crit) { return 4.0 * (double)n / (double)n_crit; }
 constexpr double kRefWarps = 152.0 * 16.0;
 constexpr double kCapWarps = 14.0;  // groups per warp above which no pass is capped

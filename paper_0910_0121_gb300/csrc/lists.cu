@@ -308,7 +308,8 @@ __device__ __forceinline__ bool take_cells(const ListArgs &a, Team<W> &team, boo
 // What a walk needs of its group, in shared memory: 64 bytes per warp, read by broadcast
 // where a test needs them (the memory clobber keeps the loads behind the stores of the next
 // group's words).  Held in registers they would spill others: the walker keeps 32
-// warps per SM at 64 registers (spills 268 -> 80 bytes; with the one scan per step and the
+// warps per SM at 64 registers (spill stores 268 -> 80 bytes before the teams, 184 with them;
+// with the one scan per step and the
 // one copy of the walk: 1.120 / 3.204 / 5.94 -> 1.034 / 3.045 / 5.46 ms).
 //   0: cell centre and half side (u)        1: particle box centre minus cell centre; first particle
 //   2: its half sides; end of the particles 3: T_prune (two words), k_f, l_min
