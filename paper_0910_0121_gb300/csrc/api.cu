@@ -71,7 +71,7 @@ struct greem_ctx {
     // S5-S6
     DBuf<float4> flist;
     DBuf<unsigned long long> ilist, loff;
-    DBuf<uint32_t> llen, lraw, kids, stack, order, bins, n_nodes, n_groups;
+    DBuf<uint32_t> llen, lraw, kids, stack, order, bins, n_counts;  // (n_counts: the numbers of groups and of nodes)
     DBuf<uint32_t> tbl;   // the list walk's start tables (k_start_table)
     int tbl_kmax = 0;     // the deepest start level of the current call's boxes
     int start_cap = 7;    // the deepest level a list walk may start at (greem_debug_set)
@@ -482,8 +482,7 @@ static int size_buffers(greem_ctx *c, const RunCfg &r)
         ENS(qlist, c->qcap * 3);
     }
     ENS(kids, nc * 8);
-    ENS(n_nodes, 1);
-    ENS(n_groups, 1);
+    ENS(n_counts, 2);
     ENS(bins, kBinWords);
     ENS(bps, (size_t)r.nbox);
     ENS(box_off, (size_t)r.nbox + 1);
@@ -632,7 +631,7 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
                   s);
     ev_record(c, r, ev, 2);
     ZeroList zt = {};  // the number of groups, the group selection's look-back words, the work-order bins
-    zt.p[0] = c->n_groups.p;
+    zt.p[0] = c->n_counts.p;
     zt.n[0] = 1;
     zt.p[1] = c->gstat.p;
     zt.n[1] = (uint32_t)group_status_words(ncap);
@@ -640,7 +639,7 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     zt.n[2] = kBinWords;
     launch_tree_prep(ks, N, c->box_off.p, nbox, c->bps.p, c->d8.p, c->K8.p, c->own.p, zt, s);
     scan_u32(c->own.p, c->base.p, N, c->scratch.p, c->st.p, s, nullptr, true, look_polls(c, GREEM_LOOK_NODES));
-    uint32_t *n_nodes = c->n_nodes.p;
+    uint32_t *n_groups = c->n_counts.p, *n_nodes = c->n_counts.p + 1;
     launch_tree_fill(ks, N, c->box_off.p, nbox, c->d8.p, c->K8.p, c->base.p, c->nodes.p, ncap, n_nodes, c->st.p, s, nsm);
     launch_tree_links(c->nodes.p, n_nodes, ncap, c->kids.p, c->pend.p, s, nsm);
     // fork: the moments (FP64-bound) on s; the particle offsets and the groups (integer
@@ -650,7 +649,6 @@ static int enqueue(greem_ctx *c, const RunCfg &r, cudaEvent_t *ev)
     cudaStreamWaitEvent(s2, c->ev_fork, 0);
     launch_leaf_offsets(ks, c->K8.p, N, c->box_off.p, nbox, c->bps.p, c->xs.p, c->ys.p, c->zs.p, c->ms.p, c->poff.p,
                         c->pcell.p, s2);
-    uint32_t *n_groups = c->n_groups.p;
     launch_group_select(c->nodes.p, n_nodes, ncap, c->box_off.p, nbox, c->bps.p, c->groups.p, n_groups, c->gstat.p,
                         c->st.p, s2, look_polls(c, GREEM_LOOK_GROUPS));
     launch_group_box(c->groups.p, n_groups, c->pcell.p, c->gbox.p, c->st.p, s2, nsm);
@@ -998,7 +996,7 @@ void greem_destroy(greem_ctx *c)
     release(c->poff); release(c->pcell); release(c->lbox); release(c->irel); release(c->groups); release(c->gbox); release(c->quad);
     release(c->flist); release(c->ilist); release(c->loff);
     release(c->llen); release(c->lraw); release(c->kids); release(c->stack); release(c->order); release(c->bins);
-    release(c->n_nodes); release(c->n_groups); release(c->bps); release(c->box_off); release(c->small); release(c->st);
+    release(c->n_counts); release(c->bps); release(c->box_off); release(c->small); release(c->st);
     release(c->qlist); release(c->qcnt); release(c->qoff);
     release(c->dom_boxes); release(c->dom); release(c->dom_cnt); release(c->let_flag); release(c->let_cnt);
     release(c->let_ends); release(c->tbl);
@@ -1924,7 +1922,7 @@ int greem_let_export(greem_ctx *c, const int32_t *boxes, int ndom, int self, int
          (rc = ensure(c, c->let_ends, (size_t)kLetChunk + 2)) ||
          (rc = ensure(c, c->scratch, scan_scratch_elems(run * chunk + 1) + 64))))
         return rc;
-    const uint32_t *n_nodes = c->n_nodes.p;
+    const uint32_t *n_nodes = c->n_counts.p + 1;
     cudaStream_t s = c->stream;
     greem::g_launches = 0;
     int64_t run_items = 0;
