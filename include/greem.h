@@ -119,7 +119,7 @@ void greem_destroy(greem_ctx *ctx);
  * Errors: INVALID_ARG (N < 1, N >= 2^31, L <= 0, r_cut outside (0, L/2), theta < 0,
  * eps < 0, n_crit < 1, n_leaf < 1, a NaN/Inf position, a mass that is NaN or of
  * magnitude >= 2^38: the FP32 force keeps the zero-distance pair of a particle with
- * itself finite only below that), CUDA, OOM. */
+ * itself finite only below that), CUDA, OOM, TIMEOUT. */
 int greem_build_tree(greem_ctx *ctx, const double *pos, const float *mass, int64_t N, const greem_params *p);
 
 /* The whole short-range force (S1-S6) with default settings: n_leaf 10, eps 0, FP32

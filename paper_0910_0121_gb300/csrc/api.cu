@@ -809,21 +809,25 @@ static void grow_caps(greem_ctx *c)
     }
 }
 
-// The pages that the warps of the list builder hold at a time: one each, but no more than
-// there are groups, which number about 4 n / n_crit and are at least as deep as l_min.  Twice
-// that is assumed, and a call that has more groups still finds its room in the 32 entries a
-// particle or takes a retry.  A call of one particle has a pool of 66 KB and one of 4 k
-// particles 40 MB, where a page for every warp is 319 MB.
-static size_t held_pages(const greem_ctx *c, int nbox)
+// The first size of the list pool: 32 entries a particle, and room for the pages that the
+// warps of the list builder hold.  That is a page each, but no more than there are groups,
+// which number about 4 n / n_crit and are at least as deep as l_min (twice that is assumed, a
+// call with more finds its room in the rest or takes a retry).  Half a page a warp is there
+// in any case, for replays of a captured graph whose lists grow, unless no lists of that many
+// particles can need it.  A call of one particle has a pool of 66 KB and one of 4 k particles
+// 160 MB, where a page for every warp is 319 MB.
+static size_t first_pool(const greem_ctx *c, const RunCfg &r)
 {
-    const size_t warps = (size_t)c->nsm * kListBlocksPerSM * kListWarps;
-    size_t groups = 0;
-    for (int b = 0; b < nbox && groups < warps; b++) {
+    const size_t warps = (size_t)c->nsm * kListBlocksPerSM * kListWarps, half = warps * (c->page / 2);
+    size_t groups = 0, most = 0;
+    for (int b = 0; b < r.nbox && (groups < warps || most < half); b++) {
         const BoxPar &bp = c->bps_host[b];
         const size_t n = bp.p_end - bp.p_begin, cells = (size_t)1 << std::min(3 * bp.lmin, 32);
         groups += std::min(n, 8 * n / (size_t)bp.n_crit + cells + 1);
+        const size_t m = std::min<size_t>(n, 1u << 20);
+        most += 4 * m * (m + 8);  // n lists of n entries, and what the pages leave over
     }
-    return std::min(warps, groups);
+    return (size_t)r.N * 32 + std::max(std::min(warps, groups) * c->page, std::min(half, most));
 }
 
 static int run(greem_ctx *c, RunCfg r)
@@ -837,7 +841,7 @@ static int run(greem_ctx *c, RunCfg r)
     if (pg > c->page) c->page = pg;
     if (r.lists_force) {
         if (c->next_list_cap) c->list_cap = c->next_list_cap;
-        else c->list_cap = std::max<size_t>(c->list_cap, (size_t)r.N * 32 + held_pages(c, r.nbox) * c->page);
+        else c->list_cap = std::max<size_t>(c->list_cap, first_pool(c, r));
         // accepted nodes are a minority of the entries: a first guess of 4 per particle
         if (r.quad) c->qcap = std::max<size_t>(c->qcap, (size_t)r.N * 4 + 4096);
     }

@@ -1,5 +1,6 @@
-"""The list pool of small calls: pages for the groups there can be, not for every warp of the
-GPU, and no retry for it; a larger call of the same context grows it."""
+"""The list pool of small calls: no page for every warp of the GPU, but at least half of one where
+lists of that many particles can fill it, and no retry; a larger call of the same context grows
+it."""
 import numpy as np
 import pytest
 
@@ -34,7 +35,10 @@ def test_pool_of_small_calls(n, n_crit, theta, clustered):
     ref = ctx.short_force(*_set(n, clustered), p)
     st = ctx.stats()
     assert st["retries"] == 0
-    assert st["list_capacity"] <= 32 * n + PAGE * min(n, 8 * n // n_crit + 8 ** st["l_min"] + 1) < 2048 * warps
+    assert st["list_capacity"] <= 32 * n + PAGE // 2 * warps
+    assert st["list_capacity"] >= 32 * n + min(PAGE // 2 * warps, n * n)
+    if n == 1:
+        assert st["list_capacity"] <= 2 * PAGE
     big = _set(100000, clustered)
     acc = ctx.short_force(*big, p)
     assert ctx.stats()["list_capacity"] >= 32 * 100000 + PAGE * warps
